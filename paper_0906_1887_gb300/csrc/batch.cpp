@@ -155,6 +155,7 @@ bool build_groups(corr_batch_s* b, const TuneChoice& ch) {
                 const corr_job& j = b->jobs[k];
                 const void* data = planes ? static_cast<const void*>(b->d_planes + b->plane_off[k]) : j.packed;
                 TcJobSpec sp{j.n_inputs, j.n_chan, j.n_time, 1, j.sample_bits, data, j.vis, cpi_of(j)};
+                if (!planes) sp.pack = tc_channel_pack(j.n_inputs, j.sample_bits == 8 ? 2 : 1, j.n_chan, 1, 0);
                 CUtensorMap m, mw{};
                 if (!(planes ? tc_make_plane_map(&m, sp, f8) : tc_make_raw_map(&m, sp, f8))) return false;
                 const int nb = blocks_of(j);
@@ -163,7 +164,8 @@ bool build_groups(corr_batch_s* b, const TuneChoice& ch) {
                 g.maps.push_back(m);
                 g.maps_wide.push_back(mw);
                 const int per_chan = sp.tw == 2 ? ((nb + 1) / 2) * ((nb + 2) / 2) : nb * (nb + 1) / 2;
-                b->items += (int64_t)((j.n_chan + sp.cpi - 1) / sp.cpi) * per_chan;
+                const int chan_tiles = (j.n_chan + sp.pack - 1) / sp.pack;
+                b->items += (int64_t)((chan_tiles + sp.cpi - 1) / sp.cpi) * per_chan;
             }
             g.tune.op_stages = ch.op_stages;
             g.tune.f8_operands = f8 ? 1 : 0;

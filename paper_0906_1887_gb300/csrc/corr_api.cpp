@@ -214,7 +214,7 @@ corr_status corr_xengine_run_batch(corr_plan plan, const void* d_packed, int n_d
     if (engine == CORR_ENGINE_TC) {
         if (p->sample_bits == 32)
             return set_error(CORR_EUNSUPPORTED, "float samples run on CORR_ENGINE_BF16X3 or CORR_ENGINE_FP32");
-        if (!d_workspace || !tc_use_planes(*p)) {
+        if (!d_workspace || !tc_use_planes(*p) || tc_raw_by_packing(*p)) {
             e = launch_xeng_tc_raw(*p, d_packed, n_dumps, d_vis, accumulate, s);
         } else {
             e = launch_tc_plane_path(*p, d_packed, n_dumps, d_workspace, d_vis, accumulate, s);

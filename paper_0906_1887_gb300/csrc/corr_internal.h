@@ -87,6 +87,9 @@ constexpr int kPlaneMinBlocks = 4;
 constexpr int kPlaneMinBlocksE4m3 = 3;
 bool tc_use_planes(const Plan& p);
 bool tc_raw_supported(int n_inputs, int sample_bits);
+// Rows that TMA cannot address one channel at a time, of a small array whose channels it can address
+// packed side by side (tc_channel_pack): the packed feed takes them too, and needs no planes.
+bool tc_raw_by_packing(const Plan& p);
 // The workspace's planes: e4m3 bytes for 4-bit samples of TMA-addressable rows (rows of
 // tc_kp_e4m3 = n_time rounded up to 128 bytes, read by kind::f8f6f4 MMAs), fp16 otherwise.  The
 // public planes calls (corr_unpack, corr_xengine_run_planes) keep fp16 planes.
@@ -113,6 +116,7 @@ struct TcJobSpec {
     int out_mode = 0;   // 1: dump mode, float32 [n_dumps][C][P][2] of V / n_accum * phasor_i conj(phasor_j)
     const void* phasor = nullptr;   // float2 [C][N] (device) or nullptr
     float inv_n = 1.0f;
+    int pack = 1;       // channels side by side in one 64-input tile (tc_channel_pack; packed feeds)
     int tw = 1;         // plane path: 2 = wide items (block I against blocks J, J + 1 in one MMA)
 };
 // Launch-shape knobs the autotuner chooses (0 = default).
@@ -123,6 +127,7 @@ struct TcTuning {
     int64_t stall_item = -1;      // self-test of the bounded waits (-1: off)
     int f8_operands = 0;          // packed 4-bit samples: e4m3 operands (kind::f8f6f4; maps with 128-sample boxes)
 };
+int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm);   // n_sm = 0: as many as fit
 int tc_default_cpi(int n_inputs, int64_t channels, int n_sm);   // channels = dumps x n_chan of the launch
 // BF16x3 on float samples with the hi/lo split done in the tensor-core kernel (single-block arrays)
 bool tc_rawf32_supported(const Plan& p);

@@ -88,14 +88,14 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, u
     }
 }
 
-// Warp-wide wait: lane 0 polls, the warp learns the outcome (and is ordered after the
-// observed phase) through __syncwarp and a broadcast.
+// Warp-wide wait: every lane polls (a completed phase costs one try and one vote; a poll by lane 0
+// with a broadcast took some 170 clocks per wait even then), and the warp decides as one.
 __device__ __forceinline__ bool mbar_wait_bounded_warp(uint32_t bar, uint32_t parity, volatile int* abort,
                                                        uint64_t limit_ns) {
-    uint32_t ok = 0;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait_bounded(bar, parity, abort, limit_ns) ? 1u : 0u;
-    __syncwarp();
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    bool ok = mbar_try_wait(bar, parity);
+    if (__all_sync(0xffffffffu, ok)) return true;
+    ok = mbar_wait_bounded(bar, parity, abort, limit_ns);
+    return __all_sync(0xffffffffu, ok);
 }
 
 // ---- TMA ------------------------------------------------------------------------

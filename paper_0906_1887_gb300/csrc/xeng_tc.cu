@@ -39,10 +39,10 @@
 // CTA roles (one CTA per SM, persistent over work items = (dump, channel, I, J)):
 //   warp 0       TMA producer
 //   warp 1       tensor-memory allocator and single-thread MMA issuer
-//   warps 2..5   epilogue, one warp per tensor-memory lane quarter: tensor memory ->
-//                registers -> lane-pair combine -> int64 -> baseline order, stored from
-//                registers (single-block arrays) or staged in shared memory and bulk-copied
-//   warps 6..13  (raw only) converters: packed bytes -> fp16 (floats -> bf16 hi/lo) K-major
+//   warps 2..9   epilogue, two warps per tensor-memory lane quarter: tensor memory ->
+//                registers -> lane-pair combine -> int64 -> baseline order, staged in shared
+//                memory and bulk-copied (single-block arrays: one run per quarter)
+//   warps 10..17 (raw only) converters: packed bytes -> fp16 (floats -> bf16 hi/lo) K-major
 //                swizzled tiles
 // Shared memory is carved at launch: when the array has a single 64-input block every
 // item is a diagonal tile (B = A), so stages hold one tile and the rings get deeper.
@@ -70,7 +70,7 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;            // 2 s per wait
 constexpr uint64_t kDrainLimitNs = 200000000ull;            // 0.2 s for in-flight work at exit
 constexpr int kMaxOpStages = 16;
 constexpr int kMaxRawStages = 32;
-constexpr int kBarBytes = 8 * (2 * kMaxOpStages + 2 * kMaxRawStages + 5) + 16;
+constexpr int kBarBytes = 8 * (2 * kMaxOpStages + 2 * kMaxRawStages + 13) + 16;
 constexpr int kSmemBudget = 227 * 1024 - kBarBytes - 1024;  // ring space after barriers and alignment
 // Staged epilogue: a warp's 16 rows of 64 baselines (16 bytes each), row pitch 65 x 16 B so
 // that the 16-byte stores of a quarter-warp fall in 8 distinct bank groups.
@@ -80,6 +80,17 @@ constexpr int kStageBytes = 4 * 16 * kStageRowBytes;
 // row at slot (j - J0) + s, with s the parity of the row's first global element index, so a
 // slot and its destination are 16-byte aligned together and the bulk copies stay aligned.
 constexpr int kStageRowBytesF = 66 * 8;
+constexpr int kStageWarpD = 16 * kStageRowBytesF + kBlockInputs * 8;   // dump mode: and the J block's phasors
+// Single-block jobs: an item's tile holds whole channels, so the baselines of a warp's 16 rows are
+// one contiguous run of the output.  The warp packs its rows there without gaps and issues one bulk
+// copy (or one bulk add) for the run.  Quarter q's rows need at most sum of (64 - u), u = 16 q ..
+// 16 q + 15, slots whatever the array's size and packing, so quarter q starts at slot kTriSlot(q)
+// (float pairs: one more 16-byte unit per warp, for a run that starts at an odd element).
+__host__ __device__ constexpr int tri_slot(int q) { return 64 * 16 * q - 8 * q * (16 * q - 1); }
+constexpr int kTriBytes = tri_slot(4) * 16;                 // int64 pairs
+constexpr int kTriPhasors = tri_slot(4) * 8 + 4 * 16;       // float pairs, then 64 phasors per warp
+constexpr int kTriBytesF = kTriPhasors + 4 * kBlockInputs * 8;
+static_assert(tri_slot(4) == 2080 && tri_slot(1) * 16 <= 16 * kStageRowBytes, "staging area");
 
 enum Mode : int { kPlanesF16 = 0, kPlanesBF16x3 = 1, kRaw8 = 2, kRaw4 = 3, kRawF32 = 4, kRaw4F8 = 5, kPlanesF8 = 6 };
 
@@ -95,7 +106,7 @@ struct Cfg {
     static constexpr bool kRaw = (MODE == kRaw8 || MODE == kRaw4 || kFloat || MODE == kRaw4F8);
     static constexpr bool kBits8 = MODE == kRaw8;
     static constexpr bool kSplit = (MODE == kPlanesBF16x3 || kFloat);
-    static constexpr int kEpiWarps = 4;     // one per tensor-memory lane quarter
+    static constexpr int kEpiWarps = 8;     // two per tensor-memory lane quarter
     static constexpr int kConvWarps = 8;
     static constexpr int kThreads = 64 + 32 * kEpiWarps + (kRaw ? 32 * kConvWarps : 0);
     static constexpr int kBps = kFloat ? 8 : (kBits8 ? 2 : 1);            // packed bytes per sample
@@ -121,8 +132,12 @@ struct TcJob {
     int kp;              // samples per dump rounded up to 64
     int n_tiles;         // work items per channel group: nb (nb + 1) / 2 tiles, or S(nb) wide items
     int tw;              // 2: wide items (block I against blocks J0, J0 + 1, one N = 256 MMA); 1: tiles
-    int cpi;             // channels per work item (2: adjacent channel pair, single-block arrays)
-    int n_groups;        // channel groups per dump = ceil(n_chan / cpi)
+    int cpi;             // tiles of adjacent channels per work item (2: single-block arrays)
+    int n_groups;        // item groups per dump = ceil(ceil(n_chan / pack) / cpi)
+    int pack;            // channels side by side in one 64-input tile (arrays of at most 32 inputs), else 1
+    int x_step, y_step;  // TMA coordinates of channel tile k: x = I kMapX + k x_step, y = k y_step
+    int pair_off;        // packed feed, cpi = 2: bytes from the first to the second tile in a sample row
+    uint32_t idesc;      // instruction descriptor of a tile's MMA (N = the columns the tile uses)
     int chunk_kb;        // stages (64 samples; 128 with e4m3 operands) per exactly-flushed chunk
     // division by n_tiles and n_groups as q = (umulhi(n, m) + n) >> s (n < 2^31; Granlund and
     // Montgomery, division by invariant integers using multiplication)
@@ -157,8 +172,8 @@ struct TcLaunch {
     int bar_offset;      // start of the barriers
     uint64_t wait_limit_ns;  // bound of every mbarrier wait
     int64_t stall_item;  // self-test: the producer withholds the first stage of this item (-1: none)
-    int staged;          // 1: epilogue stages rows in shared memory and bulk-copies them out
-    int staging_offset;  // start of the staging area (4 warps x 16 rows x kStageRowBytes)
+    int staged;          // 1: the staging area holds tile rows (jobs of several blocks), 0: packed runs only
+    int staging_offset;  // start of the staging area
     TcJob jobs[MAXJ];
 };
 
@@ -241,8 +256,12 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
                  : "memory");
 }
 
-__device__ __forceinline__ void st_shared_v2_u64(uint32_t addr, uint64_t a, uint64_t b) {
-    asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(addr), "l"(a), "l"(b) : "memory");
+__device__ __forceinline__ void st_shared_u64(uint32_t addr, uint64_t a) {
+    asm volatile("st.shared.u64 [%0], %1;" ::"r"(addr), "l"(a) : "memory");
+}
+
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, float a) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
 }
 
 __device__ __forceinline__ void st_shared_v2_f32(uint32_t addr, float a, float b) {
@@ -488,7 +507,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     uint8_t* rawring = smem + prm.raw_offset;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + prm.bar_offset);
     const int OS = prm.op_stages, RS = prm.raw_stages;
-    // barriers: op_full[OS], op_empty[OS], raw_full[RS], raw_empty[RS], acc_full[2], acc_empty[2], drain
+    // barriers: op_full[OS], op_empty[OS], raw_full[RS], raw_empty[RS], acc_full[2], acc_empty[2], drain,
+    // stage_free[4], stage_full[4] (the two epilogue warps of a lane quarter)
     const uint32_t bar_op_full = ptx::smem_u32(bars);
     const uint32_t bar_op_empty = bar_op_full + 8 * OS;
     const uint32_t bar_raw_full = bar_op_empty + 8 * OS;
@@ -496,7 +516,9 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     const uint32_t bar_acc_full = bar_raw_empty + 8 * RS;
     const uint32_t bar_acc_empty = bar_acc_full + 16;
     const uint32_t bar_drain = bar_acc_empty + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * OS + 2 * RS + 5);
+    const uint32_t bar_stage_free = bar_drain + 8;
+    const uint32_t bar_stage_full = bar_stage_free + 32;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * OS + 2 * RS + 13);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -515,6 +537,10 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             ptx::mbar_init(bar_acc_empty + 8 * b, C::kEpiWarps);
         }
         ptx::mbar_init(bar_drain, 1);
+        for (int b = 0; b < 4; ++b) {
+            ptx::mbar_init(bar_stage_free + 8 * b, 2);
+            ptx::mbar_init(bar_stage_full + 8 * b, 2);
+        }
         *abort_flag = 0;
         ptx::fence_mbar_init();
         for (int j = 0; j < prm.n_jobs; ++j) {
@@ -572,7 +598,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                         const uint32_t st = ptx::smem_u32(rawring + s * prm.raw_stage_bytes);
                         // one box covers cpi adjacent channels (cpi x 64 inputs per sample row)
                         ptx::mbar_expect_tx(fb, (same ? (uint32_t)jb.cpi : 2u) * (uint32_t)C::kRawTileBytes);
-                        tma_load_4d(st, &jb.map, I * C::kMapX, it.c0, kb * C::kStageT, (int)it.d, fb);
+                        tma_load_4d(st, &jb.map, I * C::kMapX + it.c0 * jb.x_step, it.c0 * jb.y_step,
+                                    kb * C::kStageT, (int)it.d, fb);
                         if (!same)
                             tma_load_4d(st + C::kRawTileBytes, &jb.map, J * C::kMapX, it.c0, kb * C::kStageT,
                                         (int)it.d, fb);
@@ -623,7 +650,6 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            constexpr uint32_t idesc = ptx::idesc_f16(128, 128, C::kSplit);
             constexpr uint32_t idesc_wide = ptx::idesc_f16(128, 256, C::kSplit);
             constexpr uint32_t desc_hi = ptx::sw128_desc_hi();
             const uint32_t desc_lo_ring = ptx::sw128_desc_lo(ptx::smem_u32(ring));
@@ -640,6 +666,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 ItemCtx it;
                 decode_item(prm, item, jc, it);
                 const TcJob& jb = prm.jobs[it.j];
+                const uint32_t idesc = jb.idesc;
                 const bool same = it.same;
                 const int nkb = jb.kp / C::kStageT;
                 for (int kb0 = 0; ok && kb0 < nkb; kb0 += jb.chunk_kb) {
@@ -719,38 +746,48 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         }
         __syncwarp();
     } else if (warp < 2 + C::kEpiWarps) {
-        // ---------------- epilogue (warps 2..5) ----------------
+        // ---------------- epilogue (warps 2..9) ----------------
         // Lane L of quadrant q holds operand row 32q + L: input i_loc = 16q + L/2, real part
-        // for even L, imaginary part for odd L.  Per 32 columns (16 inputs j, re/im each)
-        // the even lane finishes j = 0..7 and the odd lane j = 8..15 of the chunk.
-        const int q = warp & 3;
+        // for even L, imaginary part for odd L.  Two warps share a quadrant: both stage into the
+        // same 16 rows, warp `half` the column sixteenths m = half, half + 2, and each issues half
+        // of the row copies.  (One warp per quadrant spent 4600 clocks on a 64 x 64 tile of a
+        // 1024-input array, 1900 in the column loop and 1500 issuing copies, and bounded every
+        // output-heavy shape.)
+        const int q = warp & 3, half = (warp - 2) >> 2;
         const int i_loc = 16 * q + (lane >> 1);
         const bool odd = lane & 1;
         constexpr bool kIntOut = !C::kSplit;
-        const uint32_t staging_q = ptx::smem_u32(smem + prm.staging_offset) + (uint32_t)(q * 16 * kStageRowBytes);
+        const uint32_t staging = ptx::smem_u32(smem + prm.staging_offset);
+        const uint32_t staging_q = staging + (uint32_t)(q * (kIntOut && !DUMP ? 16 * kStageRowBytes
+                                                                              : DUMP ? kStageWarpD : 16 * kStageRowBytesF));
         int abuf = 0;
-        uint32_t aph = 0;
+        uint32_t aph = 0, sph = 0;   // phases of the accumulator and of the quadrant's staging rows
         bool ok = true;
         int jc = 0;
+        // Packed-triangle staging (single-block jobs): tile row u = sub n + i is input i of channel
+        // cx + sub; its baselines j >= i sit in tile columns u .. t_end - 1 (t_end = sub n + n) and, in
+        // the warp's part of the tile's run of elements, at slots t_slot + column.  The values depend
+        // only on the job and on how many channels of the tile exist: kept from tile to tile.
+        int t_rows = -1, t_job = -1, t_end = 0, t_slot = 0, t_len = 0, t_s0 = 0, t_mhi = 0;
         for (int64_t item = blockIdx.x; ok && item < prm.n_items; item += gridDim.x) {
             ItemCtx it;
             decode_item(prm, item, jc, it);
             const TcJob& jb = prm.jobs[it.j];
             const int n_in = jb.n_inputs;
-            const int64_t P = (int64_t)n_in * (n_in + 1) / 2;
+            const int P = n_in * (n_in + 1) / 2;
             const int I = it.I, J = it.J;
             const int nkb = jb.kp / C::kStageT;
-            const int i = I * kBlockInputs + i_loc;
-            const bool row_ok = i < n_in;
-            // baseline b(i, j) = row_off + j within one channel's [P] block
-            const int64_t row_off = (int64_t)i * n_in - (int64_t)i * (i - 1) / 2 - i;
+            const bool tri = jb.nb == 1;
+            // baseline b(i, j) = row_off(i) + j within one channel's [P] block
+            auto row_off = [&](int i) { return i * n_in - (i * (i - 1) >> 1) - i; };
+            // float pairs: 1 when the output starts at an odd 8-byte unit (16-byte alignment of the copies)
+            const int vis_odd = (int)((reinterpret_cast<uintptr_t>(jb.vis) >> 3) & 1);
             for (int kb0 = 0; kb0 < nkb; kb0 += jb.chunk_kb) {
-                // lane 0 observes the phase; the warp decides as one.  An accumulator spans a
-                // whole chunk of stages, so this wait gets twice the bound: a stage that never
-                // arrives is reported by the role waiting for that stage
+                // An accumulator spans a whole chunk of stages, so this wait gets twice the bound: a
+                // stage that never arrives is reported by the role waiting for that stage
                 const bool got =
                     ptx::mbar_wait_bounded_warp(bar_acc_full + 8 * abuf, aph, abort_flag, 2 * prm.wait_limit_ns);
-                if (!got) {
+                if (!got) {   // the warp decides as one
                     if (lane == 0) record_error(prm.status, abort_flag, kDevTimeoutAccFull, kb0);
                     ok = false;
                     break;
@@ -758,19 +795,50 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 ptx::tc_fence_after();
                 const bool add = prm.accumulate || kb0 > 0;
                 for (int ch = 0; ch < it.nsub; ++ch) {
-                // sub-accumulator ch: channel c0 + ch of a channel-pair item, or tile (I, J + ch)
-                // of a wide item
+                // sub-accumulator ch: channel tile c0 + ch of a single-block item, or tile
+                // (I, J + ch) of a wide item
                 const int Jx = it.wide ? J + ch : J;
-                const int cx = it.wide ? it.c0 : it.c0 + ch;
-                const bool ch_ok = row_ok && cx < jb.n_chan;
-                const int64_t chan_base = (it.d * jb.n_chan + cx) * P;
-                const int64_t row_base = chan_base + row_off;
+                const int J0 = Jx * kBlockInputs;
+                const int cx = (it.wide ? it.c0 : it.c0 + ch) * jb.pack;   // first channel of the tile
+                const int64_t chan_base = (it.d * jb.n_chan + cx) * (int64_t)P;
                 const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) +
                                        (uint32_t)(abuf * (int)(prm.tmem_cols / 2) + ch * 128);
-                if (kIntOut && prm.staged) {
-                    // the bulk copies of the previous channel must have read the staging rows
-                    if (lane < 16) bulk_wait_read();
-                    __syncwarp();
+                int m_lo = (it.same && Jx == I) ? q : 0, m_hi = 4;   // column sixteenths the quadrant needs
+                if (tri) {
+                    const int rows = max(0, min(jb.pack, jb.n_chan - cx)) * n_in;
+                    if (rows != t_rows || it.j != t_job) {
+                        t_rows = rows;
+                        t_job = it.j;
+                        const int r0 = 16 * q, r1 = min(r0 + 16, rows);
+                        auto start = [&](int u) {   // element of row u's first baseline within the tile's run
+                            const int sub = u / n_in, iu = u - sub * n_in;
+                            return sub * P + row_off(iu) + iu;
+                        };
+                        t_mhi = t_len = t_end = 0;
+                        if (r0 < r1) {
+                            t_s0 = start(r0);
+                            t_len = start(r1) - t_s0;
+                            t_mhi = (((r1 - 1) / n_in + 1) * n_in + 15) >> 4;
+                            t_end = i_loc < r1 ? (i_loc / n_in + 1) * n_in : 0;
+                            t_slot = start(i_loc) - t_s0 - i_loc;
+                        }
+                    }
+                    m_hi = t_mhi;
+                }
+                const int64_t tri_first = chan_base + t_s0;   // the quadrant's run of output elements
+                const int tri_odd = (!kIntOut || DUMP) ? (int)((tri_first + vis_odd) & 1) : 0;
+                // both warps' bulk copies of the previous tile must have read the staging rows; a later
+                // chunk adds into elements that the copies of the one before it wrote
+                if (lane < 16) {
+                    if (kb0 > 0) bulk_wait_all();
+                    else bulk_wait_read();
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar_stage_free + 8 * q);
+                if (!ptx::mbar_wait_bounded_warp(bar_stage_free + 8 * q, sph, abort_flag, prm.wait_limit_ns)) {
+                    if (lane == 0) record_error(prm.status, abort_flag, kDevTimeoutAccFull, kb0);
+                    ok = false;
+                    break;
                 }
                 // dump mode: this channel's phasors -- gi for the lane's row, and the J block's
                 // 64 in shared memory after the warp's staging rows (staged launches)
@@ -779,25 +847,30 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 uint32_t phs = 0;
                 if constexpr (DUMP) {
                     if (jb.phasor && cx < jb.n_chan) {   // warp-uniform: every lane stages
-                        gch = jb.phasor + (size_t)cx * n_in;
-                        if (row_ok) gi = gch[i];
-                        if (prm.staged) {
-                            phs = staging_q + 16u * (uint32_t)kStageRowBytesF;
-                            for (int u = lane; u < kBlockInputs; u += 32) {
-                                const int j = Jx * kBlockInputs + u;
-                                const float2 g = j < n_in ? gch[j] : make_float2(1.f, 0.f);
-                                st_shared_v2_f32(phs + 8u * (uint32_t)u, g.x, g.y);
-                            }
-                            __syncwarp();
-                        }
+                        gch = jb.phasor + (size_t)cx * n_in;   // [channel][input]: tile column j of row cx
+                        const int n_ph = tri ? t_rows : n_in;
+                        if (I * kBlockInputs + i_loc < n_ph) gi = gch[I * kBlockInputs + i_loc];
+                        phs = tri ? staging + (uint32_t)(kTriPhasors + q * kBlockInputs * 8)
+                                  : staging_q + 16u * (uint32_t)kStageRowBytesF;
+                        // each warp stages the 32 it uses: columns 16 m .. 16 m + 15, m = half, half + 2
+                        const int u = (lane >> 4) * 32 + half * 16 + (lane & 15);
+                        const float2 g = J0 + u < n_ph ? gch[J0 + u] : make_float2(1.f, 0.f);
+                        st_shared_v2_f32(phs + 8u * (uint32_t)u, g.x, g.y);
+                        __syncwarp();
                     }
                 }
+                // beside jobs of several blocks the run nests in the warp's own staging rows: another
+                // warp may still be on such a job's tile
+                const uint32_t tri_q = prm.staged ? staging_q
+                                                  : staging + (kIntOut && !DUMP ? (uint32_t)(tri_slot(q) * 16)
+                                                                                : (uint32_t)(tri_slot(q) * 8 + q * 16));
 #pragma unroll 1
-                for (int m = 0; m < 4; ++m) {
+                for (int m = m_lo + ((m_lo ^ half) & 1); m < m_hi; m += 2) {
                     uint32_t v[32];
                     __syncwarp();
                     ptx::tmem_ld32(tbase + 32u * m, v);
                     ptx::tmem_wait_ld();
+                    if constexpr (DUMP) {
                     // exchange: the even lane keeps j-slots 0..7 and receives the odd lane's
                     // (xi_i xr_j, xi_i xi_j) for them; the odd lane keeps 8..15 likewise
                     uint32_t own0[8], own1[8], oth0[8], oth1[8];
@@ -810,170 +883,191 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                         own0[k] = odd ? v[2 * k + 16] : v[2 * k];
                         own1[k] = odd ? v[2 * k + 17] : v[2 * k + 1];
                     }
-                    const int j0 = Jx * kBlockInputs + 16 * m + (odd ? 8 : 0);
-                    if constexpr (kIntOut && DUMP) {
+                    const int j0 = 16 * m + (odd ? 8 : 0);   // first of the lane's 8 tile columns
                         // dump mode: rr + ii and ir - ri in fp32 (each term exact, the sum rounded
                         // once), scaled by 1 / n_accum and rotated by phasor_i conj(phasor_j)
                         float2 wv[8];
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
-                            const int j = j0 + k;
                             const float rr = __uint_as_float(odd ? oth0[k] : own0[k]);
                             const float ri = __uint_as_float(odd ? oth1[k] : own1[k]);
                             const float ir = __uint_as_float(odd ? own0[k] : oth0[k]);
                             const float ii = __uint_as_float(odd ? own1[k] : oth1[k]);
                             float2 w = make_float2((rr + ii) * jb.inv_n, (ir - ri) * jb.inv_n);
-                            if (gch && j < n_in) {
-                                const float2 gj = prm.staged ? ld_shared_v2_f32(phs + 8u * (uint32_t)(j - Jx * kBlockInputs))
-                                                             : gch[j];
+                            if (gch) {   // columns past the array: phasor 1, never stored
+                                const float2 gj = ld_shared_v2_f32(phs + 8u * (uint32_t)(j0 + k));
                                 const float2 t = make_float2(w.x * gi.x - w.y * gi.y, w.x * gi.y + w.y * gi.x);
                                 w = make_float2(t.x * gj.x + t.y * gj.y, t.y * gj.x - t.x * gj.y);
                             }
                             wv[k] = w;
                         }
-                        if (prm.staged) {
+                        if (tri) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k)
+                                if (j0 + k >= i_loc && j0 + k < t_end)
+                                    st_shared_v2_f32(tri_q + 8u * (uint32_t)(t_slot + tri_odd + j0 + k), wv[k].x, wv[k].y);
+                        } else {   // dump mode of several blocks is always staged
                             // slot (j - J0) + s of row lane/2, s = parity of the row's element J0
-                            const int s_r = (int)((chan_base + row_off + Jx * kBlockInputs) & 1);
+                            const int s_r = (int)((chan_base + row_off(I * kBlockInputs + i_loc) + J0 + vis_odd) & 1);
                             const uint32_t rowp = staging_q + (uint32_t)(lane >> 1) * kStageRowBytesF +
-                                                  (uint32_t)(j0 - Jx * kBlockInputs + s_r) * 8u;
+                                                  (uint32_t)(j0 + s_r) * 8u;
 #pragma unroll
                             for (int k = 0; k < 8; ++k) st_shared_v2_f32(rowp + 8u * (uint32_t)k, wv[k].x, wv[k].y);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const int j = j0 + k;
-                                if (!ch_ok || j < i || j >= n_in) continue;
-                                reinterpret_cast<float2*>(jb.vis)[row_base + j] = wv[k];
-                            }
-                        }
-                    } else if constexpr (kIntOut) {
-                        // (rr, ri) from the real-part row, (ir, ii) from the imaginary-part row;
-                        // every D element is an integer of magnitude <= 2^24: exact in int32
-                        long long re[8], imv[8];
-                        if (jb.f32_combine) {
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const float rr = __uint_as_float(odd ? oth0[k] : own0[k]);
-                                const float ri = __uint_as_float(odd ? oth1[k] : own1[k]);
-                                const float ir = __uint_as_float(odd ? own0[k] : oth0[k]);
-                                const float ii = __uint_as_float(odd ? own1[k] : oth1[k]);
-                                re[k] = __float2int_rn(rr + ii);
-                                imv[k] = __float2int_rn(ir - ri);
-                            }
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const float rr = __uint_as_float(odd ? oth0[k] : own0[k]);
-                                const float ri = __uint_as_float(odd ? oth1[k] : own1[k]);
-                                const float ir = __uint_as_float(odd ? own0[k] : oth0[k]);
-                                const float ii = __uint_as_float(odd ? own1[k] : oth1[k]);
-                                re[k] = (long long)__float2int_rn(rr) + __float2int_rn(ii);
-                                imv[k] = (long long)__float2int_rn(ir) - __float2int_rn(ri);
-                            }
-                        }
-                        if (prm.staged) {
-                            // row lane/2 of this warp's staging rows, slots j - J0; odd lanes
-                            // write their slots rotated by 4 so a quarter-warp never shares banks
-                            const uint32_t rowp = staging_q + (uint32_t)(lane >> 1) * kStageRowBytes +
-                                                  (uint32_t)(j0 - Jx * kBlockInputs) * 16u;
-#pragma unroll
-                            for (int kk = 0; kk < 8; ++kk) {
-                                const int k_even = kk, k_odd = (kk + 4) & 7;
-                                const long long xr = odd ? re[k_odd] : re[k_even];
-                                const long long xi = odd ? imv[k_odd] : imv[k_even];
-                                const int k = odd ? k_odd : k_even;
-                                st_shared_v2_u64(rowp + 16u * (uint32_t)k, (uint64_t)xr, (uint64_t)xi);
-                            }
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const int j = j0 + k;
-                                if (!ch_ok || j < i || j >= n_in) continue;
-                                longlong2 val = make_longlong2(re[k], imv[k]);
-                                longlong2* dst = reinterpret_cast<longlong2*>(jb.vis) + row_base + j;
-                                if (add) {
-                                    const longlong2 old = *dst;
-                                    val.x += old.x;
-                                    val.y += old.y;
-                                }
-                                *dst = val;
-                            }
                         }
                     } else {
+                        // column k of the sixteenth: the real-part row (even lane) holds (rr, ri), the
+                        // imaginary-part row (odd lane) (ir, ii); one exchange of the second values
+                        // gives the even lane Re = rr + ii and the odd lane Im = ir - ri, with no
+                        // selects, and each lane stores its half of the output pair
+                        const float sgn = odd ? -1.f : 1.f;
+                        const int col = 16 * m;
+                        if constexpr (kIntOut) {
+                            // every D element is an integer of magnitude <= 2^24: exact in int32
+                            int w[16];
+                            if (jb.f32_combine) {
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int j = j0 + k;
-                            if (!ch_ok || j < i || j >= n_in) continue;
-                            const float rr = __uint_as_float(odd ? oth0[k] : own0[k]);
-                            const float ri = __uint_as_float(odd ? oth1[k] : own1[k]);
-                            const float ir = __uint_as_float(odd ? own0[k] : oth0[k]);
-                            const float ii = __uint_as_float(odd ? own1[k] : oth1[k]);
-                            float2 val = make_float2(rr + ii, ir - ri);
-                            float2* dst = reinterpret_cast<float2*>(jb.vis) + row_base + j;
-                            if (add) {
-                                const float2 old = *dst;
-                                val.x += old.x;
-                                val.y += old.y;
+                                for (int k = 0; k < 16; ++k) {
+                                    const float x = __uint_as_float(__shfl_xor_sync(0xffffffffu, v[2 * k + 1], 1));
+                                    w[k] = __float2int_rn(fmaf(sgn, x, __uint_as_float(v[2 * k])));
+                                }
+                            } else {
+#pragma unroll
+                                for (int k = 0; k < 16; ++k) {
+                                    const float x = __uint_as_float(__shfl_xor_sync(0xffffffffu, v[2 * k + 1], 1));
+                                    w[k] = __float2int_rn(__uint_as_float(v[2 * k])) + __float2int_rn(sgn * x);
+                                }
                             }
-                            *dst = val;
+                            if (tri) {
+                                const uint32_t rowp = tri_q + (uint32_t)(t_slot + col) * 16u + (odd ? 8u : 0u);
+#pragma unroll
+                                for (int k = 0; k < 16; ++k)
+                                    if (col + k >= i_loc && col + k < t_end)
+                                        st_shared_u64(rowp + 16u * (uint32_t)k, (uint64_t)(long long)w[k]);
+                            } else {
+                                // row lane/2 of the warp's staging rows, slots j - J0: the pairs of a
+                                // half-warp's 8 rows fall in distinct banks (row pitch 65 x 16 bytes)
+                                const uint32_t rowp = staging_q + (uint32_t)(lane >> 1) * kStageRowBytes +
+                                                      (uint32_t)col * 16u + (odd ? 8u : 0u);
+#pragma unroll
+                                for (int k = 0; k < 16; ++k)
+                                    st_shared_u64(rowp + 16u * (uint32_t)k, (uint64_t)(long long)w[k]);
+                            }
+                        } else {
+                            float w[16];
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) {
+                                const float x = __uint_as_float(__shfl_xor_sync(0xffffffffu, v[2 * k + 1], 1));
+                                w[k] = fmaf(sgn, x, __uint_as_float(v[2 * k]));
+                            }
+                            if (tri) {
+                                const uint32_t rowp = tri_q + (uint32_t)(t_slot + tri_odd + col) * 8u + (odd ? 4u : 0u);
+#pragma unroll
+                                for (int k = 0; k < 16; ++k)
+                                    if (col + k >= i_loc && col + k < t_end)
+                                        st_shared_f32(rowp + 8u * (uint32_t)k, w[k]);
+                            } else {
+                                const int s_r = (int)((chan_base + row_off(I * kBlockInputs + i_loc) + J0 + vis_odd) & 1);
+                                const uint32_t rowp = staging_q + (uint32_t)(lane >> 1) * kStageRowBytesF +
+                                                      (uint32_t)(col + s_r) * 8u + (odd ? 4u : 0u);
+#pragma unroll
+                                for (int k = 0; k < 16; ++k) st_shared_f32(rowp + 8u * (uint32_t)k, w[k]);
+                            }
                         }
                     }
                 }
-                if (DUMP && prm.staged) {
-                    // lane r (< 16) writes row r's float pairs [max(J0, i_r), min(J0 + 64, N)):
-                    // an unaligned first element by a plain store, the 16-byte-aligned body by a
-                    // bulk copy, an odd last element by a plain store
-                    fence_async_shared();
-                    __syncwarp();
-                    if (lane < 16) {
-                        const int ir_ = I * kBlockInputs + 16 * q + lane;
-                        const int j_lo = max(Jx * kBlockInputs, ir_);
-                        const int j_hi = min(Jx * kBlockInputs + kBlockInputs, n_in);
-                        if (ir_ < n_in && j_lo < j_hi && cx < jb.n_chan) {
-                            const int64_t rstart = chan_base + (int64_t)ir_ * n_in - (int64_t)ir_ * (ir_ - 1) / 2 - ir_;
-                            const int s_r = (int)((rstart + Jx * kBlockInputs) & 1);
-                            const uint32_t row_src = staging_q + (uint32_t)lane * kStageRowBytesF;
-                            float2* vis2 = reinterpret_cast<float2*>(jb.vis);
-                            int j = j_lo;
-                            if ((rstart + j) & 1) {
-                                vis2[rstart + j] =
-                                    ld_shared_v2_f32(row_src + (uint32_t)(j - Jx * kBlockInputs + s_r) * 8u);
-                                ++j;
-                            }
-                            const int body = (j_hi - j) & ~1;
-                            if (body > 0)
-                                bulk_store(vis2 + rstart + j, row_src + (uint32_t)(j - Jx * kBlockInputs + s_r) * 8u,
-                                           (uint32_t)body * 8u);
-                            j += body;
-                            if (j < j_hi)
-                                vis2[rstart + j] =
-                                    ld_shared_v2_f32(row_src + (uint32_t)(j - Jx * kBlockInputs + s_r) * 8u);
+                // both warps have staged their columns: the staged rows are visible to the bulk-copy
+                // engine and to the other warp
+                fence_async_shared();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar_stage_full + 8 * q);
+                if (!ptx::mbar_wait_bounded_warp(bar_stage_full + 8 * q, sph, abort_flag, prm.wait_limit_ns)) {
+                    if (lane == 0) record_error(prm.status, abort_flag, kDevTimeoutAccFull, kb0);
+                    ok = false;
+                    break;
+                }
+                sph ^= 1u;
+                // this warp's row of the tile in its lane (several blocks): lanes 0..7
+                const int r_own = 8 * half + lane;
+                const int i_own = I * kBlockInputs + 16 * q + r_own;
+                const int j_lo = max(J0, i_own), j_hi = min(J0 + kBlockInputs, n_in);
+                const bool own_ok = lane < 8 && i_own < n_in && j_lo < j_hi;   // one channel per tile: cx exists
+                if (C::kSplit && add) {
+                    // float sums in place: each warp adds half of the staged elements, lanes along the output
+                    float2* const vis2 = reinterpret_cast<float2*>(jb.vis);
+                    auto add_run = [&](int64_t first, uint32_t src, int len, int e0, int step) {
+                        for (int e = e0 + lane; e < len; e += step) {
+                            const float2 w = ld_shared_v2_f32(src + 8u * (uint32_t)e);
+                            float2 o = vis2[first + e];
+                            o.x += w.x;
+                            o.y += w.y;
+                            vis2[first + e] = o;
                         }
-                        bulk_commit();
-                    }
-                } else if (kIntOut && prm.staged) {
-                    // make the staged rows visible to the bulk-copy engine, then lane r (< 16)
-                    // copies row r's valid run of baselines [max(J0, i_r), min(J0 + 64, N))
-                    fence_async_shared();
-                    __syncwarp();
-                    if (lane < 16) {
-                        const int ir_ = I * kBlockInputs + 16 * q + lane;
-                        const int j_lo = max(Jx * kBlockInputs, ir_);
-                        const int j_hi = min(Jx * kBlockInputs + kBlockInputs, n_in);
-                        if (ir_ < n_in && j_lo < j_hi && cx < jb.n_chan) {
-                            const int64_t b0 = chan_base + (int64_t)ir_ * n_in - (int64_t)ir_ * (ir_ - 1) / 2 +
-                                               (j_lo - ir_);
-                            const uint32_t src = staging_q + (uint32_t)lane * kStageRowBytes +
-                                                 (uint32_t)(j_lo - Jx * kBlockInputs) * 16u;
-                            void* dst = reinterpret_cast<longlong2*>(jb.vis) + b0;
-                            const uint32_t bytes = (uint32_t)(j_hi - j_lo) * 16u;
-                            if (add) bulk_add_u64(dst, src, bytes);
-                            else bulk_store(dst, src, bytes);
+                    };
+                    if (tri) {
+                        add_run(tri_first, tri_q + 8u * (uint32_t)tri_odd, t_len, 32 * half, 64);
+                    } else {
+                        for (int r = 8 * half; r < 8 * half + 8; ++r) {
+                            const int ir_ = I * kBlockInputs + 16 * q + r;
+                            if (ir_ >= n_in) break;
+                            const int lo = max(J0, ir_);
+                            const int64_t rstart = chan_base + row_off(ir_);
+                            const int s_r = (int)((rstart + J0 + vis_odd) & 1);
+                            add_run(rstart + lo, staging_q + (uint32_t)r * kStageRowBytesF + (uint32_t)(lo - J0 + s_r) * 8u,
+                                    j_hi - lo, 0, 32);
                         }
-                        bulk_commit();
                     }
+                } else if (tri) {
+                    // one lane copies the quadrant's run: int64 pairs whole; float pairs the 16-byte-aligned
+                    // body, with an unaligned first and an odd last element by plain stores
+                    if (half == 0 && lane == 0 && t_len > 0) {
+                        if constexpr (kIntOut && !DUMP) {
+                            void* dst = reinterpret_cast<longlong2*>(jb.vis) + tri_first;
+                            if (add) bulk_add_u64(dst, tri_q, (uint32_t)t_len * 16u);
+                            else bulk_store(dst, tri_q, (uint32_t)t_len * 16u);
+                        } else {
+                            float2* dst = reinterpret_cast<float2*>(jb.vis) + tri_first;
+                            if (tri_odd) dst[0] = ld_shared_v2_f32(tri_q + 8u);
+                            const int body = (t_len - tri_odd) & ~1;
+                            if (body > 0) bulk_store(dst + tri_odd, tri_q + 16u * (uint32_t)tri_odd, (uint32_t)body * 8u);
+                            if (tri_odd + body < t_len)
+                                dst[t_len - 1] = ld_shared_v2_f32(tri_q + 8u * (uint32_t)(t_len - 1 + tri_odd));
+                        }
+                    }
+                    bulk_commit();
+                } else if (DUMP || !kIntOut) {
+                    // the row's float pairs [max(J0, i), min(J0 + 64, N)): an unaligned first element by
+                    // a plain store, the 16-byte-aligned body by a bulk copy, an odd last element by a
+                    // plain store
+                    if (own_ok) {
+                        const int64_t rstart = chan_base + row_off(i_own);
+                        const int s_r = (int)((rstart + J0 + vis_odd) & 1);
+                        const uint32_t row_src = staging_q + (uint32_t)r_own * kStageRowBytesF;
+                        float2* vis2 = reinterpret_cast<float2*>(jb.vis);
+                        int j = j_lo;
+                        if ((rstart + j + vis_odd) & 1) {
+                            vis2[rstart + j] = ld_shared_v2_f32(row_src + (uint32_t)(j - J0 + s_r) * 8u);
+                            ++j;
+                        }
+                        const int body = (j_hi - j) & ~1;
+                        if (body > 0)
+                            bulk_store(vis2 + rstart + j, row_src + (uint32_t)(j - J0 + s_r) * 8u, (uint32_t)body * 8u);
+                        j += body;
+                        if (j < j_hi) vis2[rstart + j] = ld_shared_v2_f32(row_src + (uint32_t)(j - J0 + s_r) * 8u);
+                    }
+                    bulk_commit();
+                } else {
+                    // the row's run of baselines [max(J0, i), min(J0 + 64, N))
+                    if (own_ok) {
+                        const uint32_t src = staging_q + (uint32_t)r_own * kStageRowBytes + (uint32_t)(j_lo - J0) * 16u;
+                        void* dst = reinterpret_cast<longlong2*>(jb.vis) + chan_base + (row_off(i_own) + j_lo);
+                        const uint32_t bytes = (uint32_t)(j_hi - j_lo) * 16u;
+                        if (add) bulk_add_u64(dst, src, bytes);
+                        else bulk_store(dst, src, bytes);
+                    }
+                    bulk_commit();
                 }
                 }  // sub-accumulators of the item
+                if (!ok) break;
                 // accumulator drained (the loads completed at tcgen05.wait::ld): hand the
                 // tensor-memory buffer back to the MMA warp
                 ptx::tc_fence_before();
@@ -986,7 +1080,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             }
         }
         // every bulk copy of ours must have completed before the CTA exits
-        if (kIntOut && prm.staged && lane < 16) bulk_wait_all();
+        if (lane < 16) bulk_wait_all();
     } else if constexpr (C::kRaw) {
         // ---------------- converters (the last kConvWarps warps) ----------------
         const int cwarp = warp - 2 - C::kEpiWarps;   // 0 .. kConvWarps - 1
@@ -1001,6 +1095,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             ItemCtx it;
             decode_item(prm, item, jc, it);
             const int cpi = prm.jobs[it.j].cpi;
+            const uint32_t pair_off = (uint32_t)prm.jobs[it.j].pair_off;
             const bool same = it.same;
             const int nkb = prm.jobs[it.j].kp / C::kStageT;
             // The stage holds n_tl packed tiles: cpi channels side by side in each sample row
@@ -1035,7 +1130,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     for (int sl = cwarp; sl < n_tl * kSlices; sl += C::kConvWarps) {
                         const int tl = sl / kSlices;
                         const int c = 2 * (sl % kSlices) + (lane >> 4);
-                        const uint32_t src = (same ? raw + tl * kRow : raw + tl * C::kRawTileBytes) +
+                        const uint32_t src = (same ? raw + tl * pair_off : raw + tl * C::kRawTileBytes) +
                                              (uint32_t)c * 16u * pitch;
                         uint32_t w[16];
 #pragma unroll
@@ -1060,7 +1155,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     if (sl < n_tl * kSlices) {
                         const int tl = split_ch ? (lane >> 4) : sl / kSlices, part = sl % kSlices;
                         const int q = C::kBits8 ? part : (split_ch ? sl : 2 * part + (lane >> 4));
-                        const uint32_t src = (same ? raw + tl * kRow : raw + tl * C::kRawTileBytes) +
+                        const uint32_t src = (same ? raw + tl * pair_off : raw + tl * C::kRawTileBytes) +
                                              (uint32_t)q * 8u * pitch;
 #pragma unroll
                         for (int e = 0; e < 8; ++e) w[v][e] = ld_shared_u32(src + (uint32_t)(e ^ eflip) * pitch);
@@ -1139,14 +1234,24 @@ bool make_plane_map(CUtensorMap* map, const void* base, int kp, int64_t rows, CU
 // 4-D map over packed bytes [dump][time][chan][input*bps]; box = 64 inputs x box_chans channels
 // x box_t samples (64, or 128 for e4m3 operands).
 // Out-of-range inputs (ragged last block) and samples (ragged last block) read as zero.
+// pack > 1 (arrays of at most 32 inputs): `pack` adjacent channels fill one 64-input tile, so the map
+// runs over whole time samples (all channels' inputs as one row) and a box of one or two tiles
+// starts at the first channel's input 0, a multiple of 16 bytes.
 bool make_raw_map(CUtensorMap* map, const void* base, int n_inputs, int n_chan, int n_time, int n_dumps, int bps,
-                  int box_chans, int box_t) {
+                  int box_chans, int box_t, int pack) {
     auto enc = get_encode();
     if (!enc) return false;
     const cuuint64_t row = (cuuint64_t)n_inputs * bps;
     cuuint64_t dims[4] = {row, (cuuint64_t)n_chan, (cuuint64_t)n_time, (cuuint64_t)n_dumps};
     cuuint64_t strides[3] = {row, row * n_chan, row * n_chan * n_time};
     cuuint32_t box[4] = {(cuuint32_t)(kBlockInputs * bps), (cuuint32_t)box_chans, (cuuint32_t)box_t, 1};
+    if (pack > 1) {
+        dims[0] = row * n_chan;
+        dims[1] = 1;
+        strides[0] = row * n_chan;
+        box[0] = (cuuint32_t)(kBlockInputs * bps * box_chans);
+        box[1] = 1;
+    }
     cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base), dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1197,7 +1302,15 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
         jb.kp = (sp.n_time + C::kStageT - 1) / C::kStageT * C::kStageT;   // whole stages (zeros past n_time)
         jb.n_tiles = jb.tw == 2 ? wide_items(jb.nb) : jb.nb * (jb.nb + 1) / 2;
         jb.cpi = sp.cpi;
-        jb.n_groups = (sp.n_chan + jb.cpi - 1) / jb.cpi;
+        jb.pack = C::kRaw && jb.nb == 1 ? sp.pack : 1;
+        jb.n_groups = ((sp.n_chan + jb.pack - 1) / jb.pack + jb.cpi - 1) / jb.cpi;
+        // packed channels: the map's rows are whole time samples (all channels), see make_raw_map
+        const int tile_x = jb.pack * sp.n_inputs * (C::kMapX / kBlockInputs);
+        jb.x_step = jb.pack > 1 ? tile_x : 0;
+        jb.y_step = jb.pack > 1 ? 0 : 1;
+        jb.pair_off = jb.pack > 1 ? jb.pack * sp.n_inputs * C::kBps : kBlockInputs * C::kBps;
+        // a single-block tile's MMA stops at the columns its inputs fill (N a multiple of 16)
+        jb.idesc = ptx::idesc_f16(128, jb.nb == 1 ? (2 * jb.pack * sp.n_inputs + 15) / 16 * 16 : 128, C::kSplit);
         // samples per exact chunk: 8-bit 1024 (|sum| <= 1024 * 2^14 = 2^24), 4-bit 131072, float: all
         // (in stages: 64 samples each, 128 for e4m3 operands)
         jb.chunk_kb = C::kSplit ? (jb.kp / kTimeBlock)
@@ -1228,14 +1341,16 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     }
     prm->n_items = items;
     prm->tmem_cols = any_pair ? 512u : 256u;
-    // shared-memory carve-up; multi-block arrays (output-heavy tiles) stage their epilogue rows
+    // shared-memory carve-up; arrays of several blocks stage tile rows, single-block ones packed runs
     bool any_multi = false, any_dump = false;
     for (int j = 0; j < n_jobs; ++j) {
         any_multi = any_multi || prm->jobs[j].nb > 1;
         any_dump = any_dump || prm->jobs[j].out_mode != 0;
     }
-    prm->staged = (!C::kSplit && any_multi) ? 1 : 0;
-    const int stage_space = prm->staged ? kStageBytes : 0;
+    prm->staged = any_multi ? 1 : 0;
+    const int stage_space = any_dump ? (any_multi ? 4 * kStageWarpD : kTriBytesF)
+                            : C::kSplit ? (any_multi ? 4 * 16 * kStageRowBytesF : kTriPhasors)
+                                        : (any_multi ? kStageBytes : kTriBytes);
     const int operand_bytes = C::kTilesPerOperand * kTileBytes;
     prm->op_stage_bytes = op_tiles * operand_bytes;
     prm->b_offset = operand_bytes;
@@ -1368,6 +1483,11 @@ bool tc_raw_supported(int n_inputs, int sample_bits) {
 
 bool tc_raw_supported(const Plan& p) { return tc_raw_supported(p.n_inputs, p.sample_bits); }
 
+bool tc_raw_by_packing(const Plan& p) {
+    return (p.sample_bits == 4 || p.sample_bits == 8) && !tc_raw_supported(p) && p.tc_operands == 0 &&
+           tc_channel_pack(p.n_inputs, p.sample_bits == 8 ? 2 : 1, p.n_chan, 1, p.n_sm) > 1;
+}
+
 // Channel pairs (256-byte TMA rows, one item's epilogue under the next item's MMAs) for
 // single-block arrays, unless there are too few channels to give every SM a pair: a small dump
 // then spreads its channels over twice as many CTAs.
@@ -1376,10 +1496,32 @@ int tc_default_cpi(int n_inputs, int64_t channels, int n_sm) {
     return channels >= 2 * (int64_t)n_sm ? 2 : 1;
 }
 
+// Channels side by side in one 64-input tile for arrays of at most 32 inputs (1: one channel per
+// tile; 0: the packed feed cannot address the samples).  A packed sample row holds the channels one
+// after another, so `pack` adjacent channels of n inputs are pack n adjacent inputs of one tile, of
+// whose products the epilogue keeps each channel's own: TMA boxes, conversions and MMAs then carry
+// pack channels for the price of one padded one.  Tiles start at 16-byte multiples and time samples
+// are 16-byte multiples (TMA), which also admits rows of fewer than 16 bytes or odd ones.  A small
+// launch keeps one tile per SM rather than fewer fuller ones.
+int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm) {
+    const int64_t row = (int64_t)n_inputs * bps;
+    const bool aligned = row % 16 == 0;
+    if (n_inputs > kBlockInputs / 2 || row * n_chan % 16 != 0) return aligned ? 1 : 0;
+    int step = 1;   // smallest pack whose tiles are 16-byte multiples
+    while (row * step % 16) ++step;
+    const int most = kBlockInputs / n_inputs;
+    if (step > most) return 0;
+    int64_t pk = n_sm > 0 ? n_dumps * n_chan / n_sm : most;
+    pk = pk > most ? most : pk;
+    pk = pk > n_chan ? n_chan : pk;
+    pk = pk / step * step;
+    return (int)(pk < step ? step : pk);
+}
+
 bool tc_make_raw_map(CUtensorMap* map, const TcJobSpec& sp, bool f8) {
     const int bps = sp.sample_bits == 8 ? 2 : 1;
     return make_raw_map(map, sp.data, sp.n_inputs, sp.n_chan, sp.n_time, sp.n_dumps, bps, sp.cpi,
-                        f8 ? Cfg<kRaw4F8>::kStageT : kTimeBlock);
+                        f8 ? Cfg<kRaw4F8>::kStageT : kTimeBlock, sp.pack);
 }
 
 cudaError_t launch_xeng_tc_raw_jobs(const TcJobSpec* specs, const CUtensorMap* maps, int n_jobs, int accumulate,
@@ -1387,7 +1529,9 @@ cudaError_t launch_xeng_tc_raw_jobs(const TcJobSpec* specs, const CUtensorMap* m
     if (n_jobs < 1) return cudaErrorInvalidValue;
     const int bits = specs[0].sample_bits;
     for (int j = 0; j < n_jobs; ++j)
-        if (specs[j].sample_bits != bits || !tc_raw_supported(specs[j].n_inputs, bits) ||
+        if (specs[j].sample_bits != bits || specs[j].pack < 1 ||
+            (specs[j].pack > 1 ? specs[j].pack * specs[j].n_inputs > kBlockInputs
+                               : !tc_raw_supported(specs[j].n_inputs, bits)) ||
             (specs[j].cpi != 1 && specs[j].cpi != 2) || (specs[j].cpi == 2 && specs[j].n_inputs > kBlockInputs))
             return cudaErrorInvalidValue;
     if (tune.f8_operands) {   // e4m3 operands: 4-bit samples (maps with 128-sample boxes)
@@ -1449,7 +1593,10 @@ cudaError_t launch_xeng_tc_plane_jobs(const TcJobSpec* specs, const CUtensorMap*
 namespace {
 cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, void* d_vis, int accumulate,
                             cudaStream_t s, const TcTuning* tune, int out_mode, const void* phasor, float inv_n) {
-    if (!tc_raw_supported(p) || (reinterpret_cast<uintptr_t>(d_packed) & 15u)) return cudaErrorInvalidValue;
+    const int bps = p.sample_bits == 8 ? 2 : 1;
+    const int pack = tc_channel_pack(p.n_inputs, bps, p.n_chan, n_dumps, p.n_sm);
+    if ((p.sample_bits != 4 && p.sample_bits != 8) || pack < 1 || (reinterpret_cast<uintptr_t>(d_packed) & 15u))
+        return cudaErrorInvalidValue;
     TcTuning plan_tune;
     plan_tune.op_stages = p.tc_op_stages;
     // 4-bit samples take e4m3 operands unless the plan asks for fp16 (CORR_OPERANDS_PACKED):
@@ -1457,18 +1604,20 @@ cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, vo
     const bool f8 = p.sample_bits == 4 && (p.tc_operands == 0 || p.tc_operands == 3);
     TcTuning run_tune = tune ? *tune : plan_tune;
     run_tune.f8_operands = f8 ? 1 : 0;
-    const int cpi = tc_default_cpi(p.n_inputs, (int64_t)n_dumps * p.n_chan, p.n_sm);
+    const int chan_tiles = (p.n_chan + pack - 1) / pack;
+    const int cpi = tc_default_cpi(p.n_inputs, (int64_t)n_dumps * chan_tiles, p.n_sm);
     // one launch covers fewer than 2^31 work items (the kernel decodes 32-bit item indices)
-    const int64_t items_per_dump = (int64_t)((p.n_chan + cpi - 1) / cpi) * (p.nb * (p.nb + 1) / 2);
+    const int64_t items_per_dump = (int64_t)((chan_tiles + cpi - 1) / cpi) * (p.nb * (p.nb + 1) / 2);
     const int64_t max_dumps = ((int64_t{1} << 31) - 1) / items_per_dump;
     if (max_dumps < 1) return cudaErrorInvalidValue;
-    const size_t packed_dump = (size_t)p.n_time * p.n_chan * p.n_inputs * (p.sample_bits == 8 ? 2 : 1);
+    const size_t packed_dump = (size_t)p.n_time * p.n_chan * p.n_inputs * bps;
     const size_t vis_dump = (size_t)p.n_chan * (size_t)p.n_baselines * (out_mode ? 8 : 16);
     for (int d0 = 0; d0 < n_dumps;) {
         const int nd = (int)((n_dumps - d0) < max_dumps ? (n_dumps - d0) : max_dumps);
         TcJobSpec sp{p.n_inputs, p.n_chan, p.n_time, nd, p.sample_bits,
                      static_cast<const uint8_t*>(d_packed) + (size_t)d0 * packed_dump,
                      static_cast<uint8_t*>(d_vis) + (size_t)d0 * vis_dump, cpi};
+        sp.pack = pack;
         sp.out_mode = out_mode;
         sp.phasor = phasor;
         sp.inv_n = inv_n;
@@ -1494,11 +1643,18 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
     if ((int64_t)n_dumps * p.n_chan >= (int64_t{1} << 31)) return cudaErrorInvalidValue;   // 32-bit item indices
     auto enc = get_encode();
     if (!enc) return cudaErrorInvalidValue;
-    // [dump][time][chan][input] of 8-byte complex floats; box = 64 inputs x 1 channel x 64 samples
+    // [dump][time][chan][input] of 8-byte complex floats; box = 64 inputs x 1 channel x 64 samples.
+    // The register epilogue that adds float sums in place takes one channel per tile.
     CUtensorMap m;
+    const int pack = accumulate ? 1 : tc_channel_pack(p.n_inputs, 8, p.n_chan, n_dumps, p.n_sm);
     const cuuint64_t row = (cuuint64_t)p.n_inputs * 8;
     cuuint64_t dims[4] = {(cuuint64_t)p.n_inputs, (cuuint64_t)p.n_chan, (cuuint64_t)p.n_time, (cuuint64_t)n_dumps};
     cuuint64_t strides[3] = {row, row * p.n_chan, row * p.n_chan * p.n_time};
+    if (pack > 1) {   // whole time samples as rows, as in make_raw_map
+        dims[0] *= (cuuint64_t)p.n_chan;
+        dims[1] = 1;
+        strides[0] = row * p.n_chan;
+    }
     cuuint32_t box[4] = {(cuuint32_t)kBlockInputs, 1, (cuuint32_t)kTimeBlock, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(d_samples), dims, strides, box, estr,
@@ -1506,6 +1662,7 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     TcJobSpec sp{p.n_inputs, p.n_chan, p.n_time, n_dumps, 32, d_samples, d_vis, 1};
+    sp.pack = pack;
     TcTuning tune;
     tune.op_stages = p.tc_op_stages;
     return launch_jobs<kRawF32, 1>(&sp, 1, &m, nullptr, accumulate, p.d_status, p.n_sm, tune, s);
