@@ -33,6 +33,8 @@
 #include <vector>
 
 #include "corr_internal.h"
+#include "fengine_wide.h"
+#include "fft_reg.cuh"
 
 namespace corr {
 namespace {
@@ -92,73 +94,10 @@ struct FPlan {
     int device = 0;
     int n_sm = 0;
     float2* d_tw = nullptr;   // the stage twiddle tables (f_tw_entries(log2L) values, at least one)
+    float2* d_tw_wide = nullptr;   // tables of the fengine_wide.cu kernel, for plans that take it
     int n_taps = 1;           // PFB taps M (input frames per output frame)
     float* d_taps = nullptr;  // PFB prototype, M L values; nullptr: plain transform
 };
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-
-// x * exp(-2 pi i a / 16) for a compile-time a in 0..7 (the roots a DFT of size <= 16 uses);
-// the constants are cos and sin of multiples of pi / 8, correctly rounded to float
-template <int A>
-__device__ __forceinline__ float2 rot16(float2 x) {
-    constexpr float kC1 = 0.92387953251128676f;   // cos(pi / 8)
-    constexpr float kS1 = 0.38268343236508977f;   // sin(pi / 8)
-    constexpr float kH = 0.70710678118654752f;    // cos(pi / 4)
-    if constexpr (A == 0) return x;
-    else if constexpr (A == 4) return make_float2(x.y, -x.x);
-    else if constexpr (A == 2) return make_float2(kH * (x.x + x.y), kH * (x.y - x.x));
-    else if constexpr (A == 6) return make_float2(kH * (x.y - x.x), -kH * (x.x + x.y));
-    else if constexpr (A == 1) return cmul(x, make_float2(kC1, -kS1));
-    else if constexpr (A == 3) return cmul(x, make_float2(kS1, -kC1));
-    else if constexpr (A == 5) return cmul(x, make_float2(-kS1, -kC1));
-    else return cmul(x, make_float2(-kC1, -kS1));
-}
-
-template <int M>
-__host__ __device__ constexpr int bit_reverse(int r) {
-    int o = 0;
-    for (int b = 0; b < M; ++b) o |= ((r >> b) & 1) << (M - 1 - b);
-    return o;
-}
-
-// one radix-2 butterfly level of an in-register DIT DFT: groups of SIZE, element j of a group
-// combined with j + SIZE / 2 after a rotation by exp(-2 pi i j / SIZE)
-template <int R, int SIZE, int J>
-__device__ __forceinline__ void dit_level(float2 (&x)[R], int k0) {
-    if constexpr (J < SIZE / 2) {
-        const float2 u = x[k0 + J];
-        const float2 t = rot16<J * (16 / SIZE)>(x[k0 + J + SIZE / 2]);
-        x[k0 + J] = cadd(u, t);
-        x[k0 + J + SIZE / 2] = csub(u, t);
-        dit_level<R, SIZE, J + 1>(x, k0);
-    }
-}
-
-template <int R, int SIZE>
-__device__ __forceinline__ void dit_levels(float2 (&x)[R]) {
-    if constexpr (SIZE <= R) {
-#pragma unroll
-        for (int k0 = 0; k0 < R; k0 += SIZE) dit_level<R, SIZE, 0>(x, k0);
-        dit_levels<R, SIZE * 2>(x);
-    }
-}
-
-// forward R-point DFT in registers (R = 2, 4, 8, 16): y_q = sum_r v_r exp(-2 pi i r q / R)
-template <int R>
-__device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
-    constexpr int M = R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : 1;
-    float2 x[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) x[bit_reverse<M>(r)] = v[r];
-    dit_levels<R, 2>(x);
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = x[r];
-}
 
 // Task -> row of a transposed-path stage.  When a half-warp spans several rows (L / R < 16),
 // the rows it takes are spread by rotating the low four bits of the row index, which puts
@@ -259,10 +198,6 @@ __device__ __forceinline__ void fft_last_stage(const float2* __restrict__ a, con
     }
 }
 
-// bytes per packed sample: 2 for complex 8-bit, 1 otherwise
-template <int KIND>
-__host__ __device__ constexpr int f_bps() { return KIND == CORR_F_COMPLEX8 ? 2 : 1; }
-
 // V consecutive inputs of one sample: 8 bytes (complex 8-bit, V = 4) or at most 4
 template <int KIND, int LG>
 using FRaw = std::conditional_t<KIND == CORR_F_COMPLEX8 && FGeom<LG>::V == 4, uint2, uint32_t>;
@@ -331,15 +266,6 @@ __device__ __forceinline__ void fetch_frame(FRaw<KIND, LG> (&raw)[FGeom<LG>::NVE
     }
 }
 
-// small integers to float by the 2^23 exponent trick: a byte u (or nibble) placed in the low
-// mantissa of 2^23 gives the float 2^23 + u exactly; the sign offset is flipped into u first
-// (u = x + 128 for a signed byte, x + 8 for a signed nibble), then one exact subtraction
-__device__ __forceinline__ float f_byte(uint32_t w, uint32_t sel, float bias) {
-    return __int_as_float((int)__byte_perm(w, 0x4B000000u, sel)) - bias;
-}
-constexpr float kBias8 = 8388736.0f;   // 2^23 + 128
-constexpr float kBias4 = 8388616.0f;   // 2^23 + 8
-
 // vector load -> V complex values (inputs g .. g + V - 1)
 template <int KIND, int LG>
 __device__ __forceinline__ void unpack_vec(FRaw<KIND, LG> r, float2 (&x)[FGeom<LG>::V]) {
@@ -398,20 +324,6 @@ __device__ __forceinline__ void fetch_task(uint32_t (&raw)[FFirst<LG>::R], const
         raw[r] = !active ? 0u
                          : (BPS == 2 ? (uint32_t)*reinterpret_cast<const unsigned short*>(src + r * step)
                                      : (uint32_t)src[r * step]);
-}
-
-// one packed sample -> complex float (exact)
-template <int KIND>
-__device__ __forceinline__ float2 unpack1(uint32_t r) {
-    if constexpr (KIND == CORR_F_COMPLEX8) {
-        const uint32_t w = r ^ 0x8080u;
-        return make_float2(f_byte(w, 0x7540u, kBias8), f_byte(w, 0x7541u, kBias8));
-    } else if constexpr (KIND == CORR_F_COMPLEX4) {
-        const uint32_t w = r ^ 0x88u;
-        return make_float2(f_byte((w >> 4) & 15u, 0x7540u, kBias4), f_byte(w & 15u, 0x7540u, kBias4));
-    } else {
-        return make_float2(f_byte(r ^ 0x80u, 0x7540u, kBias8), 0.f);
-    }
 }
 
 // Persistent over frames: frame f + gridDim.y's samples are fetched into registers while frame
@@ -607,6 +519,7 @@ cudaError_t launch_fengine_l(const FPlan& p, const void* d_in, int n_frames, voi
     return cudaGetLastError();
 }
 
+// fengine_wide.cu takes the longer plain transforms (fwide_takes)
 template <int KIND, bool PFB>
 cudaError_t launch_fengine(const FPlan& p, const void* d_in, int n_frames, void* d_out, cudaStream_t s) {
     switch (p.log2L) {
@@ -615,13 +528,19 @@ cudaError_t launch_fengine(const FPlan& p, const void* d_in, int n_frames, void*
         case 5: return launch_fengine_l<KIND, PFB, 5>(p, d_in, n_frames, d_out, s);
         case 6: return launch_fengine_l<KIND, PFB, 6>(p, d_in, n_frames, d_out, s);
         case 7: return launch_fengine_l<KIND, PFB, 7>(p, d_in, n_frames, d_out, s);
-        case 8: return launch_fengine_l<KIND, PFB, 8>(p, d_in, n_frames, d_out, s);
-        case 9: return launch_fengine_l<KIND, PFB, 9>(p, d_in, n_frames, d_out, s);
-        case 10: return launch_fengine_l<KIND, PFB, 10>(p, d_in, n_frames, d_out, s);
-        case 11: return launch_fengine_l<KIND, PFB, 11>(p, d_in, n_frames, d_out, s);
-        case 12: return launch_fengine_l<KIND, PFB, 12>(p, d_in, n_frames, d_out, s);
-        default: return cudaErrorInvalidValue;
+        default: break;
     }
+    if constexpr (PFB) {
+        switch (p.log2L) {
+            case 8: return launch_fengine_l<KIND, PFB, 8>(p, d_in, n_frames, d_out, s);
+            case 9: return launch_fengine_l<KIND, PFB, 9>(p, d_in, n_frames, d_out, s);
+            case 10: return launch_fengine_l<KIND, PFB, 10>(p, d_in, n_frames, d_out, s);
+            case 11: return launch_fengine_l<KIND, PFB, 11>(p, d_in, n_frames, d_out, s);
+            case 12: return launch_fengine_l<KIND, PFB, 12>(p, d_in, n_frames, d_out, s);
+            default: break;
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
 // the stage twiddle tables for L = 2^LG, each entry rounded from double precision
@@ -675,8 +594,15 @@ corr_status corr_fplan_create(corr_fplan* out, int n_inputs, int n_chan, int kin
     const std::vector<float2> tw = make_twiddles(p->log2L);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tw, tw.size() * sizeof(float2));
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (p->log2L >= 5) {
+        const std::vector<float2> tww = fwide_tables(kind, p->log2L);
+        if (e == cudaSuccess) e = cudaMalloc(&p->d_tw_wide, tww.size() * sizeof(float2));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(p->d_tw_wide, tww.data(), tww.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         if (p->d_tw) cudaFree(p->d_tw);
+        if (p->d_tw_wide) cudaFree(p->d_tw_wide);
         delete p;
         return cuda_error(e, "corr_fplan_create");
     }
@@ -688,6 +614,7 @@ corr_status corr_fplan_destroy(corr_fplan plan) {
     if (!plan) return CORR_OK;
     FPlan* p = reinterpret_cast<FPlan*>(plan);
     if (p->d_tw) cudaFree(p->d_tw);
+    if (p->d_tw_wide) cudaFree(p->d_tw_wide);
     if (p->d_taps) cudaFree(p->d_taps);
     delete p;
     return CORR_OK;
@@ -760,7 +687,10 @@ corr_status corr_fengine_run(corr_fplan plan, const void* d_time, int n_frames, 
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e;
     const bool pfb = p->d_taps != nullptr;
-    if (p->kind == CORR_F_COMPLEX8)
+    if (p->d_tw_wide && fwide_takes(p->kind, p->log2L, p->n_inputs, pfb ? p->n_taps : 0))
+        e = launch_fwide({p->kind, p->log2L, p->n_inputs, n_frames, p->n_taps, p->n_sm, d_time, d_spectra,
+                          p->d_tw_wide, p->d_taps}, s);
+    else if (p->kind == CORR_F_COMPLEX8)
         e = pfb ? launch_fengine<CORR_F_COMPLEX8, true>(*p, d_time, n_frames, d_spectra, s)
                 : launch_fengine<CORR_F_COMPLEX8, false>(*p, d_time, n_frames, d_spectra, s);
     else if (p->kind == CORR_F_COMPLEX4)
