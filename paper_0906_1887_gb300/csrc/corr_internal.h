@@ -94,13 +94,16 @@ bool tc_raw_by_packing(const Plan& p);
 // tc_kp_e4m3 = n_time rounded up to 128 bytes, read by kind::f8f6f4 MMAs), fp16 otherwise.  The
 // public planes calls (corr_unpack, corr_xengine_run_planes) keep fp16 planes.
 bool tc_planes_e4m3(const Plan& p);
+bool tc_use_pairs(const Plan& p, bool packed);   // CTA pairs (PAIR in xeng_tc.cu) rather than single CTAs
+bool tc_packed_pairs(const Plan& p);             // packed feed with pairs although the plan has a plane workspace
 int tc_kp_e4m3(const Plan& p);
 size_t tc_workspace_planes_bytes(const Plan& p, int n_dumps);
 cudaError_t launch_unpack_e4m3(const Plan& p, const void* d_packed, int n_dumps, void* d_planes, cudaStream_t s,
                                int blocks_per_sm = 0);
 cudaError_t launch_xeng_tc_e4m3_planes(const Plan& p, const void* d_planes, int n_dumps, void* d_vis, int accumulate,
                                        cudaStream_t s);
-// unpack into the workspace's planes, then the plane-fed tensor-core X stage
+// unpack into the workspace's planes, then the plane-fed tensor-core X stage (or, where that is
+// faster, the packed feed with CTA pairs: tc_packed_pairs)
 cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
                                  int accumulate, cudaStream_t s);
 struct TcTuning;
@@ -125,6 +128,7 @@ struct TcTuning {
     int smem_reserve = 0;         // plane feed: shared memory per SM left free for a concurrent kernel
     uint64_t wait_limit_ns = 0;   // 0: the default bound (2 s)
     int64_t stall_item = -1;      // self-test of the bounded waits (-1: off)
+    int pair = 0;                 // CTA pairs on 2 x 2 squares of tiles where every job has several blocks
     int f8_operands = 0;          // packed 4-bit samples: e4m3 operands (kind::f8f6f4; maps with 128-sample boxes)
 };
 int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm);   // n_sm = 0: as many as fit

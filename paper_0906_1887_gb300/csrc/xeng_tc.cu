@@ -70,7 +70,7 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;            // 2 s per wait
 constexpr uint64_t kDrainLimitNs = 200000000ull;            // 0.2 s for in-flight work at exit
 constexpr int kMaxOpStages = 16;
 constexpr int kMaxRawStages = 32;
-constexpr int kBarBytes = 8 * (2 * kMaxOpStages + 2 * kMaxRawStages + 13) + 16;
+constexpr int kBarBytes = 8 * (3 * kMaxOpStages + 2 * kMaxRawStages + 13) + 16;
 constexpr int kSmemBudget = 227 * 1024 - kBarBytes - 1024;  // ring space after barriers and alignment
 // Staged epilogue: a warp's 16 rows of 64 baselines (16 bytes each), row pitch 65 x 16 B so
 // that the 16-byte stores of a quarter-warp fall in 8 distinct bank groups.
@@ -221,8 +221,10 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, uint32_t m, int s) {
     return (uint32_t)(((uint64_t)__umulhi(n, m) + n) >> s);
 }
 
-template <int MAXJ>
-__device__ __forceinline__ void decode_item(const TcLaunch<MAXJ>& L, int64_t item, int& j, ItemCtx& it) {
+// PAIR: tiles are the upper triangle of block pairs (a <= b); CTA `rank` takes block I = 2 a + rank
+// against blocks J = 2 b and J + 1.
+template <int MAXJ, bool PAIR>
+__device__ __forceinline__ void decode_item(const TcLaunch<MAXJ>& L, int64_t item, int& j, ItemCtx& it, int rank) {
     while (j + 1 < L.n_jobs && item >= L.jobs[j + 1].item_begin) ++j;
     const TcJob& jb = L.jobs[j];
     const uint32_t local = (uint32_t)(item - jb.item_begin);   // < 2^31 per job (host-checked)
@@ -232,7 +234,16 @@ __device__ __forceinline__ void decode_item(const TcLaunch<MAXJ>& L, int64_t ite
     it.j = j;
     it.d = d;
     it.c0 = (int)(dg - d * (uint32_t)jb.n_groups) * jb.cpi;
-    it.wide = jb.tw == 2;
+    it.wide = PAIR || jb.tw == 2;
+    if constexpr (PAIR) {
+        int a, b;
+        tile_coords(tile, (jb.nb + 1) >> 1, a, b);
+        it.I = 2 * a + rank;
+        it.J = 2 * b;
+        it.nsub = 2;
+        it.same = a == b;
+        return;
+    }
     if (it.wide) {
         wide_coords(tile, jb.nb, it.I, it.J);
         it.nsub = min(2, jb.nb - it.J);
@@ -498,7 +509,15 @@ __device__ __forceinline__ void mma_op(uint32_t d, uint32_t a_lo, uint32_t b_lo,
 
 // DUMP: the epilogue writes the dump-mode float pairs (out_mode = 1 jobs) instead of int64
 // sums; a separate instantiation so the exact-output kernels keep their registers.
-template <int MODE, int MAXJ, bool DUMP>
+//
+// PAIR (arrays of several blocks): two CTAs of a cluster work on a 2 x 2 square of tiles, blocks
+// 2 a, 2 a + 1 against 2 b, 2 b + 1, with one M = 256, N = 256 MMA (cta_group::2) per K step: each
+// CTA holds its own block's 128 rows of A and half of B, so it loads (or converts) two blocks for
+// its two tiles -- one, on the diagonal -- where single tiles take two per tile, and its shared
+// memory feeds 8 KB instead of 16 KB of operands per tile and K step.  The even CTA's MMA thread
+// issues for both; converters and epilogue warps of the odd CTA arrive on its barriers, and its
+// commits arrive in both.  On planes the odd CTA's MMA thread relays "stage loaded".
+template <int MODE, int MAXJ, bool DUMP, bool PAIR>
 __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const __grid_constant__ TcLaunch<MAXJ> prm) {
     using C = Cfg<MODE>;
     extern __shared__ uint8_t smem_raw[];
@@ -508,7 +527,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + prm.bar_offset);
     const int OS = prm.op_stages, RS = prm.raw_stages;
     // barriers: op_full[OS], op_empty[OS], raw_full[RS], raw_empty[RS], acc_full[2], acc_empty[2], drain,
-    // stage_free[4], stage_full[4] (the two epilogue warps of a lane quarter)
+    // stage_free[4], stage_full[4] (the two epilogue warps of a lane quarter), peer_full[OS] (pairs)
     const uint32_t bar_op_full = ptx::smem_u32(bars);
     const uint32_t bar_op_empty = bar_op_full + 8 * OS;
     const uint32_t bar_raw_full = bar_op_empty + 8 * OS;
@@ -518,15 +537,20 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     const uint32_t bar_drain = bar_acc_empty + 16;
     const uint32_t bar_stage_free = bar_drain + 8;
     const uint32_t bar_stage_full = bar_stage_free + 32;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * OS + 2 * RS + 13);
+    const uint32_t bar_peer_full = bar_stage_full + 32;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * OS + 2 * RS + 13);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kCtas = PAIR ? 2 : 1;
+    const int rank = PAIR ? (int)ptx::cluster_rank() : 0;
+    const int64_t item0 = blockIdx.x / kCtas, item_step = gridDim.x / kCtas;   // the CTA's (pair's) items
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < OS; ++s) {
-            ptx::mbar_init(bar_op_full + 8 * s, C::kRaw ? C::kConvWarps : 1);
+            ptx::mbar_init(bar_op_full + 8 * s, C::kRaw ? C::kConvWarps * kCtas : 1);
             ptx::mbar_init(bar_op_empty + 8 * s, 1);
+            ptx::mbar_init(bar_peer_full + 8 * s, 1);
         }
         for (int s = 0; s < RS; ++s) {
             ptx::mbar_init(bar_raw_full + 8 * s, 1);
@@ -534,7 +558,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(bar_acc_full + 8 * b, 1);
-            ptx::mbar_init(bar_acc_empty + 8 * b, C::kEpiWarps);
+            ptx::mbar_init(bar_acc_empty + 8 * b, C::kEpiWarps * kCtas);
         }
         ptx::mbar_init(bar_drain, 1);
         for (int b = 0; b < 4; ++b) {
@@ -550,11 +574,16 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         if (C::kSplit && !C::kRaw) ptx::prefetch_tensormap(&prm.map_lo);
     }
     if (warp == 1) {
-        ptx::tmem_alloc(ptx::smem_u32(tmem_slot), prm.tmem_cols);
-        ptx::tmem_relinquish();
+        ptx::tmem_alloc<PAIR>(ptx::smem_u32(tmem_slot), prm.tmem_cols);
+        ptx::tmem_relinquish<PAIR>();
     }
     ptx::tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) {
+        __syncwarp();
+        ptx::cluster_sync();   // the other CTA's barriers exist before anything arrives on them
+    } else {
+        __syncthreads();
+    }
     ptx::tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
@@ -571,9 +600,9 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             int64_t withheld = -1;     // the slot the self-test withheld
             bool ok = true;
             int jc = 0;
-            for (int64_t item = blockIdx.x; ok && item < prm.n_items; item += gridDim.x) {
+            for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
                 ItemCtx it;
-                decode_item(prm, item, jc, it);
+                decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
                 const TcJob& jb = prm.jobs[it.j];
                 const int I = it.I, J = it.J;
                 const bool same = it.same;
@@ -601,15 +630,15 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                         tma_load_4d(st, &jb.map, I * C::kMapX + it.c0 * jb.x_step, it.c0 * jb.y_step,
                                     kb * C::kStageT, (int)it.d, fb);
                         if (!same)
-                            tma_load_4d(st + C::kRawTileBytes, &jb.map, J * C::kMapX, it.c0, kb * C::kStageT,
+                            tma_load_4d(st + C::kRawTileBytes, &jb.map, (J + rank) * C::kMapX, it.c0, kb * C::kStageT,
                                         (int)it.d, fb);
                     } else {
                         const uint32_t st = ptx::smem_u32(ring + s * prm.op_stage_bytes);
                         const int64_t dc = it.d * jb.n_chan + it.c0;   // planes: one channel per item
                         const int rowA = (int)((dc * jb.nb + I) * kBlockRows);
-                        const int rowB = (int)((dc * jb.nb + J) * kBlockRows);
+                        const int rowB = (int)((dc * jb.nb + J + rank) * kBlockRows);
                         const uint32_t bo = (uint32_t)prm.b_offset;
-                        if (it.wide) {
+                        if (!PAIR && it.wide) {
                             // B = blocks J (, J + 1) in one box at b_offset; A = block I, or on the
                             // diagonal the first half of the B box itself
                             const uint32_t nB = (uint32_t)it.nsub;
@@ -649,8 +678,43 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            constexpr uint32_t idesc_wide = ptx::idesc_f16(128, 256, C::kSplit);
+        if (PAIR && rank != 0) {
+            // planes: tell the issuing CTA which of this CTA's stages have landed
+            if (!C::kRaw && lane == 0) {
+                const uint32_t peer = ptx::map_shared(bar_peer_full, 0);
+                int s = 0;
+                uint32_t ph = 0;
+                bool ok = true;
+                int jc = 0;
+                for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
+                    ItemCtx it;
+                    decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
+                    const int nkb = prm.jobs[it.j].kp / C::kStageT;
+                    for (int kb = 0; kb < nkb; ++kb) {
+                        if (!ptx::mbar_wait_bounded(bar_op_full + 8 * s, ph, abort_flag, prm.wait_limit_ns)) {
+                            record_error(prm.status, abort_flag, kDevTimeoutFull, kb);
+                            ok = false;
+                            break;
+                        }
+                        ptx::mbar_arrive_cluster(peer + 8 * s);
+                        if (++s == OS) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
+                    }
+                }
+            }
+            // the issuing CTA's last commits must have arrived here before this CTA exits
+            if (lane == 0) ptx::mbar_wait_drain(bar_drain, 0, kDrainLimitNs);
+        } else if (lane == 0) {
+            constexpr uint32_t idesc_wide = ptx::idesc_f16(PAIR ? 256 : 128, 256, C::kSplit);
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                return ptx::mbar_wait_bounded(bar, parity, abort_flag, prm.wait_limit_ns);
+            };
+            auto commit = [&](uint32_t bar) {
+                if constexpr (PAIR) ptx::mma_commit_pair(bar);
+                else ptx::mma_commit(bar);
+            };
             constexpr uint32_t desc_hi = ptx::sw128_desc_hi();
             const uint32_t desc_lo_ring = ptx::sw128_desc_lo(ptx::smem_u32(ring));
             const uint32_t stage16 = (uint32_t)prm.op_stage_bytes >> 4;
@@ -662,16 +726,16 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             bool ok = true;
             bool any = false;
             int jc = 0;
-            for (int64_t item = blockIdx.x; ok && item < prm.n_items; item += gridDim.x) {
+            for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
                 ItemCtx it;
-                decode_item(prm, item, jc, it);
+                decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
                 const TcJob& jb = prm.jobs[it.j];
                 const uint32_t idesc = jb.idesc;
                 const bool same = it.same;
                 const int nkb = jb.kp / C::kStageT;
                 for (int kb0 = 0; ok && kb0 < nkb; kb0 += jb.chunk_kb) {
                     const int kb1 = min(nkb, kb0 + jb.chunk_kb);
-                    if (!ptx::mbar_wait_bounded(bar_acc_empty + 8 * abuf, aph ^ 1u, abort_flag, prm.wait_limit_ns)) {
+                    if (!wait(bar_acc_empty + 8 * abuf, aph ^ 1u)) {
                         record_error(prm.status, abort_flag, kDevTimeoutAccEmpty, kb0);
                         ok = false;
                         break;
@@ -679,7 +743,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     ptx::tc_fence_after();
                     const uint32_t dset = tmem_base + (uint32_t)(abuf * (int)(prm.tmem_cols / 2));
                     for (int kb = kb0; kb < kb1; ++kb) {
-                        if (!ptx::mbar_wait_bounded(bar_op_full + 8 * s, ph, abort_flag, prm.wait_limit_ns)) {
+                        if (!wait(bar_op_full + 8 * s, ph) ||
+                            (PAIR && !C::kRaw && !wait(bar_peer_full + 8 * s, ph))) {
                             record_error(prm.status, abort_flag, kDevTimeoutFull, kb);
                             ok = false;
                             break;
@@ -689,7 +754,13 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                         // 16 KB tile, +2 per 16-sample step along the swizzled rows
                         const uint32_t a0 = desc_lo_ring + (uint32_t)s * stage16;
                         const uint32_t acc0 = kb > kb0 ? 1u : 0u;
-                        if (!C::kRaw && !C::kSplit && it.wide) {
+                        if constexpr (PAIR) {
+                            const uint32_t b0 = same ? a0 : a0 + boff16;
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                ptx::mma_pair_lo<C::kF8>(dset, a0 + 2u * k, b0 + 2u * k, desc_hi, idesc_wide,
+                                                         (k > 0) | acc0);
+                        } else if (!C::kRaw && !C::kSplit && it.wide) {
                             // one M = 128, N = 256 MMA covers tiles (I, J) and (I, J + 1); on the
                             // diagonal A is the first half of the B box
                             const uint32_t b0 = a0 + boff16;
@@ -724,14 +795,14 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                                 mma_op<C::kF8>(dset, a0 + 2u * k, b0 + 2u * k, desc_hi, idesc, (k > 0) | acc0);
                         }
                         any = true;
-                        ptx::mma_commit(bar_op_empty + 8 * s);
+                        commit(bar_op_empty + 8 * s);
                         if (++s == OS) {
                             s = 0;
                             ph ^= 1u;
                         }
                     }
                     if (!ok) break;
-                    ptx::mma_commit(bar_acc_full + 8 * abuf);
+                    commit(bar_acc_full + 8 * abuf);
                     if (++abuf == 2) {
                         abuf = 0;
                         aph ^= 1u;
@@ -740,7 +811,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             }
             // every MMA of ours must be complete before tensor memory is released
             if (any) {
-                ptx::mma_commit(bar_drain);
+                commit(bar_drain);
                 ptx::mbar_wait_drain(bar_drain, 0, kDrainLimitNs);
             }
         }
@@ -769,9 +840,9 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         // the warp's part of the tile's run of elements, at slots t_slot + column.  The values depend
         // only on the job and on how many channels of the tile exist: kept from tile to tile.
         int t_rows = -1, t_job = -1, t_end = 0, t_slot = 0, t_len = 0, t_s0 = 0, t_mhi = 0;
-        for (int64_t item = blockIdx.x; ok && item < prm.n_items; item += gridDim.x) {
+        for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
             ItemCtx it;
-            decode_item(prm, item, jc, it);
+            decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
             const TcJob& jb = prm.jobs[it.j];
             const int n_in = jb.n_inputs;
             const int P = n_in * (n_in + 1) / 2;
@@ -795,6 +866,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 ptx::tc_fence_after();
                 const bool add = prm.accumulate || kb0 > 0;
                 for (int ch = 0; ch < it.nsub; ++ch) {
+                // a pair's square reaches below the diagonal and past the last block
+                if (PAIR && (J + ch < I || J + ch >= jb.nb || I >= jb.nb)) continue;
                 // sub-accumulator ch: channel tile c0 + ch of a single-block item, or tile
                 // (I, J + ch) of a wide item
                 const int Jx = it.wide ? J + ch : J;
@@ -803,7 +876,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 const int64_t chan_base = (it.d * jb.n_chan + cx) * (int64_t)P;
                 const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) +
                                        (uint32_t)(abuf * (int)(prm.tmem_cols / 2) + ch * 128);
-                int m_lo = (it.same && Jx == I) ? q : 0, m_hi = 4;   // column sixteenths the quadrant needs
+                int m_lo = Jx == I ? q : 0, m_hi = 4;   // column sixteenths the quadrant needs
                 if (tri) {
                     const int rows = max(0, min(jb.pack, jb.n_chan - cx)) * n_in;
                     if (rows != t_rows || it.j != t_job) {
@@ -1072,7 +1145,10 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 // tensor-memory buffer back to the MMA warp
                 ptx::tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_acc_empty + 8 * abuf);
+                if (lane == 0) {
+                    if constexpr (PAIR) ptx::mbar_arrive_cluster(ptx::map_shared(bar_acc_empty + 8 * abuf, 0));
+                    else ptx::mbar_arrive(bar_acc_empty + 8 * abuf);
+                }
                 if (++abuf == 2) {
                     abuf = 0;
                     aph ^= 1u;
@@ -1091,9 +1167,9 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         uint32_t rph = 0, oph = 0;
         bool ok = true;
         int jc = 0;
-        for (int64_t item = blockIdx.x; ok && item < prm.n_items; item += gridDim.x) {
+        for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
             ItemCtx it;
-            decode_item(prm, item, jc, it);
+            decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
             const int cpi = prm.jobs[it.j].cpi;
             const uint32_t pair_off = (uint32_t)prm.jobs[it.j].pair_off;
             const bool same = it.same;
@@ -1175,7 +1251,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 fence_async_shared();   // generic-proxy writes -> visible to the tensor core
                 __syncwarp();
                 if (lane == 0) {
-                    ptx::mbar_arrive(bar_op_full + 8 * os);
+                    if constexpr (PAIR) ptx::mbar_arrive_cluster(ptx::map_shared(bar_op_full + 8 * os, 0));
+                    else ptx::mbar_arrive(bar_op_full + 8 * os);
                     ptx::mbar_arrive(bar_raw_empty + 8 * rs);
                 }
                 if (++rs == RS) {
@@ -1191,9 +1268,15 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     }
 
     ptx::tc_fence_before();
-    __syncthreads();
+    if constexpr (PAIR) {
+        __syncwarp();
+        ptx::cluster_sync();   // neither CTA's memory goes while the other may still arrive there or read it
+    } else {
+        __syncthreads();
+    }
     ptx::tc_fence_after();
-    if (warp == 1) ptx::tmem_dealloc(tmem_base, prm.tmem_cols);
+    if (warp == 1) ptx::tmem_dealloc<PAIR>(tmem_base, prm.tmem_cols);
+    if constexpr (PAIR) ptx::cluster_sync();
 }
 
 // ---- host side --------------------------------------------------------------------
@@ -1287,20 +1370,22 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     if (map_lo) prm->map_lo = *map_lo;
     int64_t items = 0;
     int op_tiles = 1, raw_tiles = 1;
-    bool any_pair = false;
+    bool any_pair = false, pair = tune.pair != 0 && !C::kSplit && MODE != kRaw4;
+    for (int j = 0; j < n_jobs; ++j) pair = pair && specs[j].n_inputs > kBlockInputs;
     for (int j = 0; j < n_jobs; ++j) {
         const TcJobSpec& sp = specs[j];
         TcJob& jb = prm->jobs[j];
         jb.map = maps[j];
         // wide items only where the MMA feed reads fp16 planes (two blocks per TMA box)
-        jb.tw = ((MODE == kPlanesF16 || MODE == kPlanesF8) && sp.tw == 2 && maps_wide) ? 2 : 1;
+        jb.tw = ((MODE == kPlanesF16 || MODE == kPlanesF8) && sp.tw == 2 && maps_wide && !pair) ? 2 : 1;
         if (jb.tw == 2) jb.map_wide = maps_wide[j];
         jb.vis = sp.vis;
         jb.n_inputs = sp.n_inputs;
         jb.n_chan = sp.n_chan;
         jb.nb = (sp.n_inputs + kBlockInputs - 1) / kBlockInputs;
         jb.kp = (sp.n_time + C::kStageT - 1) / C::kStageT * C::kStageT;   // whole stages (zeros past n_time)
-        jb.n_tiles = jb.tw == 2 ? wide_items(jb.nb) : jb.nb * (jb.nb + 1) / 2;
+        const int ng = (jb.nb + 1) / 2;
+        jb.n_tiles = pair ? ng * (ng + 1) / 2 : jb.tw == 2 ? wide_items(jb.nb) : jb.nb * (jb.nb + 1) / 2;
         jb.cpi = sp.cpi;
         jb.pack = C::kRaw && jb.nb == 1 ? sp.pack : 1;
         jb.n_groups = ((sp.n_chan + jb.pack - 1) / jb.pack + jb.cpi - 1) / jb.cpi;
@@ -1337,7 +1422,7 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
         const int tiles = jb.tw == 2 ? 3 : (jb.nb == 1 ? jb.cpi : 2);
         op_tiles = tiles > op_tiles ? tiles : op_tiles;
         raw_tiles = tiles > raw_tiles ? tiles : raw_tiles;
-        any_pair = any_pair || jb.cpi == 2 || jb.tw == 2;   // two 256-column accumulator sets
+        any_pair = any_pair || jb.cpi == 2 || jb.tw == 2 || pair;   // two 256-column accumulator sets
     }
     prm->n_items = items;
     prm->tmem_cols = any_pair ? 512u : 256u;
@@ -1385,18 +1470,34 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     prm->staging_offset = prm->raw_offset + prm->raw_stages * prm->raw_stage_bytes;
     prm->bar_offset = prm->staging_offset + stage_space;
     const int smem_bytes = prm->bar_offset + kBarBytes + 1024;
-    auto kern = xeng_tc_kernel<MODE, MAXJ, false>;
+    auto kern = xeng_tc_kernel<MODE, MAXJ, false, false>;
+    if constexpr (!C::kSplit && MODE != kRaw4) {
+        if (pair) kern = xeng_tc_kernel<MODE, MAXJ, false, true>;
+    }
     if constexpr (C::kRaw && !C::kFloat && MAXJ == 1) {
-        if (any_dump) kern = xeng_tc_kernel<MODE, MAXJ, true>;
+        if (any_dump) kern = xeng_tc_kernel<MODE, MAXJ, true, false>;
+        if constexpr (MODE != kRaw4) {
+            if (any_dump && pair) kern = xeng_tc_kernel<MODE, MAXJ, true, true>;
+        }
     } else if (any_dump) {   // dump mode is built for single-job packed-sample launches only
         delete prm;
         return cudaErrorInvalidValue;
     }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e == cudaSuccess && items > 0) {
-        const int grid = (int)(items < n_sm ? items : n_sm);
-        kern<<<grid, C::kThreads, smem_bytes, s>>>(*prm);
-        e = cudaGetLastError();
+        const int per_item = pair ? 2 : 1, slots = n_sm / per_item;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(items < slots ? items : slots) * per_item);
+        cfg.blockDim = dim3(C::kThreads);
+        cfg.dynamicSmemBytes = (size_t)smem_bytes;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = pair ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, kern, *prm);
     }
     delete prm;
     return e;
@@ -1424,13 +1525,37 @@ cudaError_t launch_xeng_tc(const Plan& p, const void* d_planes, const void* d_pl
     // read-modify-write epilogue bounds them and which run faster on the deeper operand ring of
     // 32 KB stages (measured: 1024 inputs x 1228 channels x 472 samples, 4.05 against 4.41 ms)
     const bool wide = p.tc_items == 2 || (p.tc_items == 0 && !(accumulate && p.kp < 1024));
+    tune.pair = tc_use_pairs(p, false);
     CUtensorMap mw;
-    if (p.nb >= 2 && wide && make_plane_map(&mw, d_planes, p.kp, rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+    if (!tune.pair && p.nb >= 2 && wide && make_plane_map(&mw, d_planes, p.kp, rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
                                             2 * kBlockRows)) {
         sp.tw = 2;
         return launch_jobs<kPlanesF16, 1>(&sp, 1, &mh, nullptr, accumulate, p.d_status, p.n_sm, tune, s, &mw);
     }
     return launch_jobs<kPlanesF16, 1>(&sp, 1, &mh, nullptr, accumulate, p.d_status, p.n_sm, tune, s);
+}
+
+// CTA pairs work on 2 x 2 squares of tiles, so an odd block count leaves a block row and column of
+// squares half empty.  Measured (8-bit, 512 channels, us, single CTAs -> pairs): packed feed, 128
+// inputs x 256 / 2048 samples 40 -> 36 / 205 -> 127 (but 32 -> 34 at 128 samples), 192 inputs 57 -> 68
+// at 128 samples, 75 -> 72 / 417 -> 381 at 256 / 2048, 256 inputs x 2048 662 -> 396, 512 inputs x 2048
+// (476 channels) 1712 -> 936; plane feed, 512 inputs x 2048 1104 -> 998, 1024 inputs x 2048 (158
+// channels) 1107 -> 992, but 320 inputs x 2048 821 -> 856 and, 4-bit, 320 x 512 158 -> 179.
+bool tc_use_pairs(const Plan& p, bool packed) {
+    if (p.nb < 2 || p.tc_items != 0) return false;
+    if (p.nb % 2 == 0) return p.nb > 2 || p.kp > 128;
+    return packed && p.kp > 256;
+}
+
+// Arrays whose plan would take the plane feed but which pairs convert faster inside the kernel: each
+// block is converted once per square instead of once per tile.  Measured (8-bit, us, planes with
+// pairs -> packed with pairs; 128 / 512 / 2048 samples): 256 inputs 97 -> 85 / 168 -> 122 / 554 -> 396,
+// 512 inputs 273 -> 255 / 427 -> 392 / 998 -> 936, 768 inputs 321 -> 313 / 432 -> 446 / 990 -> 1085, 1024
+// inputs 310 -> 311 / 405 -> 451 / 992 -> 1185 (256 samples: 374 -> 344, 360 -> 343).  4-bit (e4m3
+// planes): 256 inputs 89 -> 84 / 125 -> 109 / 303 -> 320, 512 inputs 342 -> 346 at 512 samples.
+bool tc_packed_pairs(const Plan& p) {
+    if (p.tc_operands != 0 || p.nb % 2 || !tc_use_pairs(p, true) || !tc_raw_supported(p)) return false;
+    return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= 256 : p.nb == 4 && p.kp <= 512;
 }
 
 bool tc_planes_e4m3(const Plan& p) { return p.sample_bits == 4 && tc_raw_supported(p); }
@@ -1449,7 +1574,8 @@ cudaError_t launch_xeng_tc_e4m3_planes(const Plan& p, const void* d_planes, int 
     if (!make_plane_map(&mh, d_planes, kp8, rows, CU_TENSOR_MAP_DATA_TYPE_UINT8)) return cudaErrorInvalidValue;
     // item shape as for fp16 planes
     const bool wide = p.tc_items == 2 || (p.tc_items == 0 && !(accumulate && kp8 < 1024));
-    if (p.nb >= 2 && wide &&
+    tune.pair = tc_use_pairs(p, false);
+    if (!tune.pair && p.nb >= 2 && wide &&
         make_plane_map(&mw, d_planes, kp8, rows, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2 * kBlockRows)) {
         sp.tw = 2;
         return launch_jobs<kPlanesF8, 1>(&sp, 1, &mh, nullptr, accumulate, p.d_status, p.n_sm, tune, s, &mw);
@@ -1459,6 +1585,8 @@ cudaError_t launch_xeng_tc_e4m3_planes(const Plan& p, const void* d_planes, int 
 
 cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
                                  int accumulate, cudaStream_t s) {
+    if (tc_packed_pairs(p) && (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0)
+        return launch_xeng_tc_raw(p, d_packed, n_dumps, d_vis, accumulate, s);
     if (tc_planes_e4m3(p)) {
         const cudaError_t e = launch_unpack_e4m3(p, d_packed, n_dumps, d_ws, s);
         return e == cudaSuccess ? launch_xeng_tc_e4m3_planes(p, d_ws, n_dumps, d_vis, accumulate, s) : e;
@@ -1604,6 +1732,7 @@ cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, vo
     const bool f8 = p.sample_bits == 4 && (p.tc_operands == 0 || p.tc_operands == 3);
     TcTuning run_tune = tune ? *tune : plan_tune;
     run_tune.f8_operands = f8 ? 1 : 0;
+    run_tune.pair = tc_use_pairs(p, true) && !(p.sample_bits == 4 && !f8);
     const int chan_tiles = (p.n_chan + pack - 1) / pack;
     const int cpi = tc_default_cpi(p.n_inputs, (int64_t)n_dumps * chan_tiles, p.n_sm);
     // one launch covers fewer than 2^31 work items (the kernel decodes 32-bit item indices)
