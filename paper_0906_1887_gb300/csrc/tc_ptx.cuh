@@ -98,6 +98,16 @@ __device__ __forceinline__ bool mbar_wait_bounded_warp(uint32_t bar, uint32_t pa
     return __all_sync(0xffffffffu, ok);
 }
 
+// Two waits in this order, at the price of one where both phases are complete.
+__device__ __forceinline__ bool mbar_wait_bounded_warp2(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1,
+                                                        volatile int* abort, uint64_t limit_ns) {
+    bool ok = mbar_try_wait(bar0, parity0);
+    ok = ok && mbar_try_wait(bar1, parity1);
+    if (__all_sync(0xffffffffu, ok)) return true;
+    ok = mbar_wait_bounded(bar0, parity0, abort, limit_ns) && mbar_wait_bounded(bar1, parity1, abort, limit_ns);
+    return __all_sync(0xffffffffu, ok);
+}
+
 // ---- CTA pairs (clusters of two) ----------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;

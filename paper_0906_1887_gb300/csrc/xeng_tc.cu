@@ -108,6 +108,11 @@ struct Cfg {
     static constexpr bool kSplit = (MODE == kPlanesBF16x3 || kFloat);
     static constexpr int kEpiWarps = 8;     // two per tensor-memory lane quarter
     static constexpr int kConvWarps = 8;
+    // groups of converter warps, each taking every other stage: the e4m3 and float conversions gain (4-bit
+    // 64 inputs 126 -> 116 us, 128 inputs x 2048 samples 106 -> 86; BF16x3 109 -> 105), the 8-bit one,
+    // whose loads and stores crowd the shared-memory port, does not (129 -> 136)
+    static constexpr int kConvGroups = kF8 || kFloat ? 2 : 1;
+    static constexpr int kGroupWarps = kConvWarps / kConvGroups;
     static constexpr int kThreads = 64 + 32 * kEpiWarps + (kRaw ? 32 * kConvWarps : 0);
     static constexpr int kBps = kFloat ? 8 : (kBits8 ? 2 : 1);            // packed bytes per sample
     static constexpr int kStageT = kF8 ? 2 * kTimeBlock : kTimeBlock;    // samples per stage
@@ -548,13 +553,13 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < OS; ++s) {
-            ptx::mbar_init(bar_op_full + 8 * s, C::kRaw ? C::kConvWarps * kCtas : 1);
+            ptx::mbar_init(bar_op_full + 8 * s, C::kRaw ? C::kGroupWarps * kCtas : 1);
             ptx::mbar_init(bar_op_empty + 8 * s, 1);
             ptx::mbar_init(bar_peer_full + 8 * s, 1);
         }
         for (int s = 0; s < RS; ++s) {
             ptx::mbar_init(bar_raw_full + 8 * s, 1);
-            ptx::mbar_init(bar_raw_empty + 8 * s, C::kConvWarps);
+            ptx::mbar_init(bar_raw_empty + 8 * s, C::kGroupWarps);
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(bar_acc_full + 8 * b, 1);
@@ -1159,7 +1164,17 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         if (lane < 16) bulk_wait_all();
     } else if constexpr (C::kRaw) {
         // ---------------- converters (the last kConvWarps warps) ----------------
-        const int cwarp = warp - 2 - C::kEpiWarps;   // 0 .. kConvWarps - 1
+        // With two groups, one converts a whole stage while the other converts the next one: waits,
+        // fence and arrivals (some 400 clocks of a stage with eight warps on it) are paid per warp and
+        // visit, and a visit carries twice the work.  A barrier's phases are told apart by parity
+        // only, so no group may wait for a phase two ahead of the barrier's: a group's previous stage
+        // (two back) had its operand slot, so the MMAs are past the slot's use before last (rings have
+        // two slots at least); and once this stage's operand slot is free, the raw slot's previous
+        // stage is consumed -- where the raw ring is at least as deep as the operand ring, or its
+        // slots stay with one group (an even depth; the host makes it so).
+        const int cwarp = (warp - 2 - C::kEpiWarps) % C::kGroupWarps;
+        const int group = (warp - 2 - C::kEpiWarps) / C::kGroupWarps;
+        int turn = 0;
         const ConvLane cl = C::kBits8 ? conv_lane8(lane) : (C::kF8 ? conv_lane4_f8(lane) : conv_lane4(lane));
         constexpr uint32_t kRow = kBlockInputs * C::kBps;   // packed bytes of 64 inputs
         const uint32_t lane_byte = C::kBits8 ? 4u * lane : 4u * (lane & 15);
@@ -1182,9 +1197,12 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             const int n_tl = same ? cpi : 2;
             const bool pair_pitch = same && cpi == 2;
             for (int kb = 0; kb < nkb; ++kb) {
+                const bool mine = turn == group;
+                if (++turn == C::kConvGroups) turn = 0;
+                if (mine) {
                 const bool got =
-                    ptx::mbar_wait_bounded_warp(bar_raw_full + 8 * rs, rph, abort_flag, prm.wait_limit_ns) &&
-                    ptx::mbar_wait_bounded_warp(bar_op_empty + 8 * os, oph ^ 1u, abort_flag, prm.wait_limit_ns);
+                    ptx::mbar_wait_bounded_warp2(bar_op_empty + 8 * os, oph ^ 1u, bar_raw_full + 8 * rs, rph,
+                                                 abort_flag, prm.wait_limit_ns);
                 if (!got) {   // the warp decides as one
                     if (lane == 0) record_error(prm.status, abort_flag, kDevTimeoutFull, kb);
                     ok = false;
@@ -1195,7 +1213,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 if constexpr (C::kFloat) {
                     // single-block arrays only (one tile, B = A): slice q of the tile per warp
                     const uint32_t raw_tile = ptx::smem_u32(rawring + rs * prm.raw_stage_bytes);
-                    for (int sl = cwarp; sl < kTimeBlock / 8; sl += C::kConvWarps)
+                    for (int sl = cwarp; sl < kTimeBlock / 8; sl += C::kGroupWarps)
                         convert_slice_f32(raw_tile, dst, sl, lane);
                 } else if constexpr (C::kF8) {
                     // e4m3 operands, a slice per warp: 32 samples of one tile, lanes 0..15 chunk
@@ -1203,7 +1221,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     // converter's conflict-free orders below measured slower here: this converter
                     // is bound by its instruction count, not by shared-memory conflicts.)
                     const uint32_t pitch = pair_pitch ? 2 * kRow : kRow;
-                    for (int sl = cwarp; sl < n_tl * kSlices; sl += C::kConvWarps) {
+                    for (int sl = cwarp; sl < n_tl * kSlices; sl += C::kGroupWarps) {
                         const int tl = sl / kSlices;
                         const int c = 2 * (sl % kSlices) + (lane >> 4);
                         const uint32_t src = (same ? raw + tl * pair_off : raw + tl * C::kRawTileBytes) +
@@ -1215,9 +1233,9 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     }
                 } else {
                 const uint32_t pitch = pair_pitch ? 2 * kRow : kRow;
-                // all loads of the warp's slices (slices cwarp and cwarp + 8) are issued before
-                // the first conversion, so their shared-memory latencies overlap
-                constexpr int kSlots = (2 * kSlices + C::kConvWarps - 1) / C::kConvWarps;
+                // all loads of the warp's slices are issued before the first conversion, so their
+                // shared-memory latencies overlap
+                constexpr int kSlots = (2 * kSlices + C::kGroupWarps - 1) / C::kGroupWarps;
                 uint32_t w[kSlots][8];
                 // 4-bit slices (8 samples of 64 inputs per half-warp) split like the e4m3 ones:
                 // by channel with channel pairs, else by sample group with the upper half-warp
@@ -1227,7 +1245,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 const int eflip = (!C::kBits8 && !pair_pitch) ? (lane >> 4) : 0;
 #pragma unroll
                 for (int v = 0; v < kSlots; ++v) {
-                    const int sl = cwarp + C::kConvWarps * v;
+                    const int sl = cwarp + C::kGroupWarps * v;
                     if (sl < n_tl * kSlices) {
                         const int tl = split_ch ? (lane >> 4) : sl / kSlices, part = sl % kSlices;
                         const int q = C::kBits8 ? part : (split_ch ? sl : 2 * part + (lane >> 4));
@@ -1239,7 +1257,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 }
 #pragma unroll
                 for (int v = 0; v < kSlots; ++v) {
-                    const int sl = cwarp + C::kConvWarps * v;
+                    const int sl = cwarp + C::kGroupWarps * v;
                     if (sl < n_tl * kSlices) {
                         const int tl = split_ch ? (lane >> 4) : sl / kSlices, part = sl % kSlices;
                         const uint32_t out = dst + (same ? tl * kTileBytes : tl * prm.b_offset);
@@ -1255,6 +1273,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     else ptx::mbar_arrive(bar_op_full + 8 * os);
                     ptx::mbar_arrive(bar_raw_empty + 8 * rs);
                 }
+                }   // the group's stage
                 if (++rs == RS) {
                     rs = 0;
                     rph ^= 1u;
@@ -1449,6 +1468,8 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
         int raw_space = kSmemBudget - stage_space - prm->op_stages * prm->op_stage_bytes;
         prm->raw_stages = raw_space / prm->raw_stage_bytes;
         if (prm->raw_stages > kMaxRawStages) prm->raw_stages = kMaxRawStages;
+        // two converter groups on a shallower raw ring need an even one (see the converters' waits)
+        if (C::kConvGroups == 2 && prm->raw_stages < prm->op_stages) prm->raw_stages &= ~1;
         if (prm->raw_stages < 2) {
             delete prm;
             return cudaErrorInvalidValue;
