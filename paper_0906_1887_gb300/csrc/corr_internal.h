@@ -63,6 +63,9 @@ size_t planes_bytes(const Plan& p, int n_dumps);     // one set of planes
 // runs beside a tensor-core launch takes one, which fits next to its CTA in either launch order)
 cudaError_t launch_unpack_fp16(const Plan& p, const void* d_packed, int n_dumps, void* d_planes,
                                cudaStream_t s, int blocks_per_sm = 0);
+// Rows that are no 16-byte multiples -> rows of repack_pitch bytes, which TMA can address.
+int64_t repack_pitch(const Plan& p);
+cudaError_t launch_repack(const Plan& p, const void* d_packed, int n_dumps, void* d_out, cudaStream_t s);
 cudaError_t launch_unpack_f32(const Plan& p, const void* d_packed, int n_dumps, void* d_planes,
                               cudaStream_t s);
 cudaError_t launch_unpack_bf16x2(const Plan& p, const void* d_packed, int n_dumps, void* d_hi,
@@ -120,6 +123,7 @@ struct TcJobSpec {
     const void* phasor = nullptr;   // float2 [C][N] (device) or nullptr
     float inv_n = 1.0f;
     int pack = 1;       // channels side by side in one 64-input tile (tc_channel_pack; packed feeds)
+    int64_t row_pitch = 0;   // packed feed: bytes from one channel's row to the next (0: dense rows)
     int tw = 1;         // plane path: 2 = wide items (block I against blocks J, J + 1 in one MMA)
 };
 // Launch-shape knobs the autotuner chooses (0 = default).

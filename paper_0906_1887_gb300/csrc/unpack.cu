@@ -14,6 +14,7 @@
 #include <cuda_fp16.h>
 
 #include "corr_internal.h"
+#include "launch.cuh"
 #include "sample_convert.cuh"
 
 namespace corr {
@@ -22,29 +23,10 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kPad = 65;  // smem row stride (floats)
 
-enum OutKind { kOutF16 = 0, kOutF32 = 1, kOutBF16Split = 2 };
+enum OutKind { kOutF32 = 0, kOutBF16Split = 1 };
 
-template <int BITS>
-__device__ __forceinline__ void load_sample(const unsigned char* __restrict__ packed, int64_t idx, float& re,
-                                            float& im) {
-    if constexpr (BITS == 4) {
-        int b = packed[idx];
-        int r = (b >> 4) & 0xF, m = b & 0xF;
-        re = (float)(r >= 8 ? r - 16 : r);
-        im = (float)(m >= 8 ? m - 16 : m);
-    } else if constexpr (BITS == 8) {
-        unsigned short v = reinterpret_cast<const unsigned short*>(packed)[idx];
-        re = (float)(signed char)(v & 0xFF);
-        im = (float)(signed char)(v >> 8);
-    } else {
-        float2 v = reinterpret_cast<const float2*>(packed)[idx];
-        re = v.x;
-        im = v.y;
-    }
-}
-
-template <int BITS, int OUT>
-__global__ void __launch_bounds__(kThreads) unpack_kernel(const unsigned char* __restrict__ packed, int n_inputs,
+template <int OUT>
+__global__ void __launch_bounds__(kThreads) unpack_kernel(const float2* __restrict__ samples, int n_inputs,
                                                           int n_chan, int n_time, int nb_count, int kp,
                                                           int64_t n_tiles, void* __restrict__ out0,
                                                           void* __restrict__ out1) {
@@ -70,7 +52,9 @@ __global__ void __launch_bounds__(kThreads) unpack_kernel(const unsigned char* _
                 float re = 0.f, im = 0.f;
                 if (tg < n_time && ig < n_inputs) {
                     const int64_t idx = ((d * n_time + tg) * n_chan + c) * (int64_t)n_inputs + ig;
-                    load_sample<BITS>(packed, idx, re, im);
+                    const float2 v = samples[idx];
+                    re = v.x;
+                    im = v.y;
                 }
                 s_re[i * kPad + t] = re;
                 s_im[i * kPad + t] = im;
@@ -83,12 +67,7 @@ __global__ void __launch_bounds__(kThreads) unpack_kernel(const unsigned char* _
             const int r = q >> 3, ch = q & 7;
             const float* src = ((r & 1) ? s_im : s_re) + (r >> 1) * kPad + ch * 8;
             const int64_t off = (row0 + r) * (int64_t)kp + tb * kTimeBlock + ch * 8;
-            if constexpr (OUT == kOutF16) {
-                __align__(16) __half v[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = __float2half_rn(src[e]);
-                *reinterpret_cast<uint4*>(static_cast<__half*>(out0) + off) = *reinterpret_cast<uint4*>(v);
-            } else if constexpr (OUT == kOutF32) {
+            if constexpr (OUT == kOutF32) {
                 float4* dst = reinterpret_cast<float4*>(static_cast<float*>(out0) + off);
                 dst[0] = make_float4(src[0], src[1], src[2], src[3]);
                 dst[1] = make_float4(src[4], src[5], src[6], src[7]);
@@ -131,10 +110,30 @@ struct FastTile {
 // kGroup: tiles whose loads a block issues together (1 for the full grid; 8 for a launch of one
 // block per SM beside a tensor-core launch, 64 KB in flight per block).  F8 (4-bit only): the
 // planes hold e4m3 bytes instead of fp16 (rows of kp bytes), for the e4m3 plane feed.
-template <int BITS, int kGroup, bool F8 = false>
+// RAGGED: rows that are no whole 16-byte pieces; a piece is put together from the aligned words
+// around it, and bytes past the row are zero.  Tiles are counted in 32 bits (2^31 tiles of planes are
+// 17 TB); 64-bit divisions of the tile index took a tenth of the time.
+__device__ __forceinline__ uint4 load_piece(const unsigned char* __restrict__ base, int64_t off, int64_t last_word,
+                                            int n_valid) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(base);
+    const int64_t i = off >> 2;
+    const uint32_t sh = (uint32_t)(off & 3) * 8;
+    uint32_t x[5], v[4];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) x[k] = w[i + k < last_word ? i + k : last_word];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int left = n_valid - 4 * k;   // bytes of this word inside the row
+        v[k] = __funnelshift_r(x[k], x[k + 1], sh);
+        if (left < 4) v[k] = left <= 0 ? 0u : v[k] & ((1u << (8 * left)) - 1u);
+    }
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+template <int BITS, int kGroup, bool F8 = false, bool RAGGED = false>
 __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
     const unsigned char* __restrict__ packed, int n_inputs, int n_chan, int n_time, int nb_count, int kp,
-    int64_t n_tiles, void* __restrict__ planes_out) {
+    uint32_t n_tiles, void* __restrict__ planes_out, int64_t last_word) {
     static_assert(!F8 || BITS == 4, "e4m3 planes hold 4-bit samples only");
     __half* __restrict__ planes = static_cast<__half*>(planes_out);
     using F = FastTile<BITS>;
@@ -150,18 +149,18 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
     const uint32_t* src = tile + (size_t)(8 * q) * F::kWords;
     // A block takes kGroup tiles at a time (strided by the grid) and issues every load of the
     // group before converting any: kGroup x 8 KB in flight per block.
-    for (int64_t t_base = blockIdx.x; t_base < n_tiles; t_base += (int64_t)kGroup * gridDim.x) {
+    for (uint32_t t_base = blockIdx.x; t_base < n_tiles; t_base += kGroup * gridDim.x) {
         uint4 v[kGroup][kPer];
 #pragma unroll
         for (int gi = 0; gi < kGroup; ++gi) {
-            const int64_t t_idx = t_base + (int64_t)gi * gridDim.x;
+            const uint32_t t_idx = t_base + gi * gridDim.x;
             const bool tile_ok = t_idx < n_tiles;
-            const int tb = tile_ok ? (int)(t_idx % tb_count) : 0;
-            const int64_t rest = tile_ok ? t_idx / tb_count : 0;
-            const int nb = (int)(rest % nb_count);
-            const int64_t dc = rest / nb_count;          // dump * n_chan + chan
-            const int64_t d = dc / n_chan;
-            const int c = (int)(dc % n_chan);
+            const uint32_t rest = tile_ok ? t_idx / (uint32_t)tb_count : 0;
+            const int tb = tile_ok ? (int)(t_idx - rest * tb_count) : 0;
+            const uint32_t dc = rest / (uint32_t)nb_count;   // dump * n_chan + chan
+            const int nb = (int)(rest - dc * nb_count);
+            const int64_t d = dc / (uint32_t)n_chan;
+            const int c = (int)(dc - (uint32_t)d * n_chan);
             const int64_t valid = row_bytes - (int64_t)nb * F::kRowBytes;   // bytes of this block's row that exist
 #pragma unroll
             for (int u = 0; u < kPer; ++u) {
@@ -172,18 +171,20 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
                 if (tile_ok && tg < n_time && (int64_t)piece * 16 < valid) {
                     const int64_t off =
                         ((d * n_time + tg) * n_chan + c) * row_bytes + (int64_t)nb * F::kRowBytes + piece * 16;
-                    v[gi][u] = *reinterpret_cast<const uint4*>(packed + off);
+                    if constexpr (RAGGED)
+                        v[gi][u] = load_piece(packed, off, last_word, (int)(valid - piece * 16 < 16 ? valid - piece * 16 : 16));
+                    else v[gi][u] = *reinterpret_cast<const uint4*>(packed + off);
                 }
             }
         }
 #pragma unroll
         for (int gi = 0; gi < kGroup; ++gi) {
-            const int64_t t_idx = t_base + (int64_t)gi * gridDim.x;
+            const uint32_t t_idx = t_base + gi * gridDim.x;
             if (t_idx >= n_tiles) break;   // uniform across the block
-            const int tb = (int)(t_idx % tb_count);
-            const int64_t rest = t_idx / tb_count;
-            const int nb = (int)(rest % nb_count);
-            const int64_t dc = rest / nb_count;
+            const uint32_t rest = t_idx / (uint32_t)tb_count;
+            const int tb = (int)(t_idx - rest * tb_count);
+            const int64_t dc = rest / (uint32_t)nb_count;
+            const int nb = (int)(rest - (uint32_t)dc * nb_count);
 #pragma unroll
             for (int u = 0; u < kPer; ++u) {
                 const int k = tid + u * F::kThreads;
@@ -270,89 +271,97 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
     }
 }
 
-template <int BITS>
-cudaError_t launch_fast(const Plan& p, const void* d_packed, int n_dumps, void* planes, cudaStream_t s,
-                       int blocks_per_sm) {
+// The whole GPU: many blocks, one tile each at a time; or, beside a tensor-core launch, few blocks
+// with eight tiles of loads in flight each (blocks_per_sm > 0).  kp: samples of a plane row.
+template <int BITS, bool F8>
+cudaError_t launch_fast(const Plan& p, const void* d_packed, int n_dumps, void* planes, int kp, cudaStream_t s,
+                        int blocks_per_sm) {
     using F = FastTile<BITS>;
-    const int64_t n_tiles = (int64_t)n_dumps * p.n_chan * p.nb * (p.kp / kTimeBlock);
+    const int64_t n_tiles = (int64_t)n_dumps * p.n_chan * p.nb * (kp / kTimeBlock);
     if (n_tiles < 1) return cudaSuccess;
+    if (n_tiles >= (int64_t{1} << 31)) return cudaErrorInvalidValue;
     const auto* src = static_cast<const unsigned char*>(d_packed);
-    auto* out = static_cast<__half*>(planes);
-    if (blocks_per_sm > 0) {   // few blocks: each keeps eight tiles of loads in flight
-        const int64_t cap = (int64_t)p.n_sm * blocks_per_sm;
-        const int grid = (int)(n_tiles < cap ? n_tiles : cap);
-        unpack_fast_kernel<BITS, 8><<<grid, F::kThreads, 0, s>>>(src, p.n_inputs, p.n_chan, p.n_time, p.nb, p.kp,
-                                                                 n_tiles, out);
-    } else {                   // the whole GPU: many blocks, one tile each at a time
-        const int64_t cap = (int64_t)p.n_sm * (BITS == 8 ? 8 : 16);
-        const int grid = (int)(n_tiles < cap ? n_tiles : cap);
-        unpack_fast_kernel<BITS, 1><<<grid, F::kThreads, 0, s>>>(src, p.n_inputs, p.n_chan, p.n_time, p.nb, p.kp,
-                                                                 n_tiles, out);
-    }
-    return cudaGetLastError();
+    const int64_t bytes = (int64_t)n_dumps * p.n_time * p.n_chan * p.n_inputs * (BITS == 8 ? 2 : 1);
+    const bool ragged = (int64_t)p.n_inputs * (BITS == 8 ? 2 : 1) % 16 != 0;
+    const int64_t cap = (int64_t)p.n_sm * (blocks_per_sm > 0 ? blocks_per_sm : BITS == 8 ? 8 : 16);
+    const dim3 grid((unsigned)(n_tiles < cap ? n_tiles : cap));
+    auto kern = ragged ? unpack_fast_kernel<BITS, 1, F8, true>
+                       : blocks_per_sm > 0 ? unpack_fast_kernel<BITS, 8, F8> : unpack_fast_kernel<BITS, 1, F8>;
+    return launch_kernel(kern, grid, F::kThreads, 0, s, 1, false, src, p.n_inputs, p.n_chan, p.n_time, p.nb, kp,
+                          (uint32_t)n_tiles, planes, (bytes + 3) / 4 - 1);
 }
 
-// 4-bit samples into e4m3 planes with rows of kp8 bytes (n_time rounded up to 128 samples);
-// blocks_per_sm as for launch_fast
-cudaError_t launch_fast_e4m3(const Plan& p, const void* d_packed, int n_dumps, void* planes, int kp8,
-                             cudaStream_t s, int blocks_per_sm) {
-    using F = FastTile<4>;
-    const int64_t n_tiles = (int64_t)n_dumps * p.n_chan * p.nb * (kp8 / kTimeBlock);
-    if (n_tiles < 1) return cudaSuccess;
-    const auto* src = static_cast<const unsigned char*>(d_packed);
-    if (blocks_per_sm > 0) {
-        const int64_t cap = (int64_t)p.n_sm * blocks_per_sm;
-        const int grid = (int)(n_tiles < cap ? n_tiles : cap);
-        unpack_fast_kernel<4, 8, true><<<grid, F::kThreads, 0, s>>>(src, p.n_inputs, p.n_chan, p.n_time, p.nb, kp8,
-                                                                    n_tiles, planes);
-    } else {
-        const int64_t cap = (int64_t)p.n_sm * 16;
-        const int grid = (int)(n_tiles < cap ? n_tiles : cap);
-        unpack_fast_kernel<4, 1, true><<<grid, F::kThreads, 0, s>>>(src, p.n_inputs, p.n_chan, p.n_time, p.nb, kp8,
-                                                                    n_tiles, planes);
+// Packed rows [row][row_bytes] -> [row][pitch], pitch a multiple of 16 bytes: rows that TMA can
+// address (what lies between a row's end and the next row is never read).  A copy at the price of
+// the packed samples twice over, where planes cost their two to four times as many bytes twice
+// (75 inputs, 8-bit: 78 MB in, 83 out, against 284 MB of planes).
+__global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __restrict__ packed,
+                                                     unsigned char* __restrict__ out, uint32_t rows, int row_bytes,
+                                                     int pieces, uint32_t rows_per_block, int64_t last_word) {
+    for (uint32_t r0 = blockIdx.x * rows_per_block; r0 < rows; r0 += gridDim.x * rows_per_block) {
+        const uint32_t n = min(rows_per_block, rows - r0) * (uint32_t)pieces;
+        uint4* dst = reinterpret_cast<uint4*>(out) + (int64_t)r0 * pieces;
+        const int64_t base = (int64_t)r0 * row_bytes;
+#pragma unroll 4
+        for (uint32_t e = threadIdx.x; e < n; e += 256) {
+            const uint32_t r = e / (uint32_t)pieces;
+            dst[e] = load_piece(packed, base + (int64_t)r * row_bytes + (e - r * pieces) * 16, last_word, 16);
+        }
     }
-    return cudaGetLastError();
 }
 
-template <int BITS, int OUT>
+template <int OUT>
 cudaError_t launch(const Plan& p, const void* d_packed, int n_dumps, void* o0, void* o1, cudaStream_t s) {
     const int64_t n_tiles = (int64_t)n_dumps * p.n_chan * p.nb * (p.kp / kTimeBlock);
     const int64_t cap = (int64_t)p.n_sm * 8;
     const int grid = (int)(n_tiles < cap ? n_tiles : cap);
-    unpack_kernel<BITS, OUT><<<grid, kThreads, 0, s>>>(static_cast<const unsigned char*>(d_packed), p.n_inputs,
-                                                        p.n_chan, p.n_time, p.nb, p.kp, n_tiles, o0, o1);
-    return cudaGetLastError();
+    return launch_kernel(unpack_kernel<OUT>, dim3((unsigned)grid), kThreads, 0, s, 1, false,
+                          static_cast<const float2*>(d_packed), p.n_inputs, p.n_chan, p.n_time, p.nb, p.kp,
+                          n_tiles, o0, o1);
 }
 
 }  // namespace
 
 cudaError_t launch_unpack_fp16(const Plan& p, const void* d_packed, int n_dumps, void* d_planes, cudaStream_t s,
                                int blocks_per_sm) {
-    // packed rows of whole 16-byte pieces (and a 16-byte aligned base) take the vectorised kernel
-    const int64_t row = (int64_t)p.n_inputs * (p.sample_bits == 8 ? 2 : 1);
-    const bool fast = row % 16 == 0 && (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0 &&
-                      (reinterpret_cast<uintptr_t>(d_planes) & 15u) == 0;
-    if (p.sample_bits == 4)
-        return fast ? launch_fast<4>(p, d_packed, n_dumps, d_planes, s, blocks_per_sm)
-                    : launch<4, kOutF16>(p, d_packed, n_dumps, d_planes, nullptr, s);
-    return fast ? launch_fast<8>(p, d_packed, n_dumps, d_planes, s, blocks_per_sm)
-                : launch<8, kOutF16>(p, d_packed, n_dumps, d_planes, nullptr, s);
+    if (((reinterpret_cast<uintptr_t>(d_packed) | reinterpret_cast<uintptr_t>(d_planes)) & 15u) != 0)
+        return cudaErrorInvalidValue;
+    return p.sample_bits == 4 ? launch_fast<4, false>(p, d_packed, n_dumps, d_planes, p.kp, s, blocks_per_sm)
+                              : launch_fast<8, false>(p, d_packed, n_dumps, d_planes, p.kp, s, blocks_per_sm);
 }
 
 cudaError_t launch_unpack_e4m3(const Plan& p, const void* d_packed, int n_dumps, void* d_planes, cudaStream_t s,
                                int blocks_per_sm) {
-    if (!tc_planes_e4m3(p) || (reinterpret_cast<uintptr_t>(d_packed) & 15u) || (reinterpret_cast<uintptr_t>(d_planes) & 15u))
+    if (p.sample_bits != 4 || (reinterpret_cast<uintptr_t>(d_packed) & 15u) || (reinterpret_cast<uintptr_t>(d_planes) & 15u))
         return cudaErrorInvalidValue;
-    return launch_fast_e4m3(p, d_packed, n_dumps, d_planes, tc_kp_e4m3(p), s, blocks_per_sm);
+    return launch_fast<4, true>(p, d_packed, n_dumps, d_planes, tc_kp_e4m3(p), s, blocks_per_sm);
+}
+
+int64_t repack_pitch(const Plan& p) {
+    return ((int64_t)p.n_inputs * (p.sample_bits == 8 ? 2 : 1) + 15) / 16 * 16;
+}
+
+cudaError_t launch_repack(const Plan& p, const void* d_packed, int n_dumps, void* d_out, cudaStream_t s) {
+    const int64_t rows = (int64_t)n_dumps * p.n_time * p.n_chan;
+    const int row_bytes = p.n_inputs * (p.sample_bits == 8 ? 2 : 1);
+    if (rows >= (int64_t{1} << 31) ||
+        ((reinterpret_cast<uintptr_t>(d_packed) | reinterpret_cast<uintptr_t>(d_out)) & 15u) != 0)
+        return cudaErrorInvalidValue;
+    const int pieces = (int)(repack_pitch(p) / 16);
+    const int per = 2048 / pieces > 0 ? 2048 / pieces : 1;
+    const int64_t want = (rows + per - 1) / per, cap = (int64_t)p.n_sm * 8;
+    return launch_kernel(repack_kernel, dim3((unsigned)(want < cap ? want : cap)), 256, 0, s, 1, false,
+                          static_cast<const unsigned char*>(d_packed), static_cast<unsigned char*>(d_out), (uint32_t)rows,
+                          row_bytes, pieces, (uint32_t)per, (rows * row_bytes + 3) / 4 - 1);
 }
 
 cudaError_t launch_unpack_f32(const Plan& p, const void* d_packed, int n_dumps, void* d_planes, cudaStream_t s) {
-    return launch<32, kOutF32>(p, d_packed, n_dumps, d_planes, nullptr, s);
+    return launch<kOutF32>(p, d_packed, n_dumps, d_planes, nullptr, s);
 }
 
 cudaError_t launch_unpack_bf16x2(const Plan& p, const void* d_packed, int n_dumps, void* d_hi, void* d_lo,
                                  cudaStream_t s) {
-    return launch<32, kOutBF16Split>(p, d_packed, n_dumps, d_hi, d_lo, s);
+    return launch<kOutBF16Split>(p, d_packed, n_dumps, d_hi, d_lo, s);
 }
 
 }  // namespace corr

@@ -59,6 +59,7 @@
 #include <new>
 
 #include "corr_internal.h"
+#include "launch.cuh"
 #include "sample_convert.cuh"
 #include "tc_ptx.cuh"
 
@@ -1340,11 +1341,11 @@ bool make_plane_map(CUtensorMap* map, const void* base, int kp, int64_t rows, CU
 // runs over whole time samples (all channels' inputs as one row) and a box of one or two tiles
 // starts at the first channel's input 0, a multiple of 16 bytes.
 bool make_raw_map(CUtensorMap* map, const void* base, int n_inputs, int n_chan, int n_time, int n_dumps, int bps,
-                  int box_chans, int box_t, int pack) {
+                  int box_chans, int box_t, int pack, int64_t pitch) {
     auto enc = get_encode();
     if (!enc) return false;
-    const cuuint64_t row = (cuuint64_t)n_inputs * bps;
-    cuuint64_t dims[4] = {row, (cuuint64_t)n_chan, (cuuint64_t)n_time, (cuuint64_t)n_dumps};
+    const cuuint64_t row = pitch > 0 ? (cuuint64_t)pitch : (cuuint64_t)n_inputs * bps;
+    cuuint64_t dims[4] = {(cuuint64_t)n_inputs * bps, (cuuint64_t)n_chan, (cuuint64_t)n_time, (cuuint64_t)n_dumps};
     cuuint64_t strides[3] = {row, row * n_chan, row * n_chan * n_time};
     cuuint32_t box[4] = {(cuuint32_t)(kBlockInputs * bps), (cuuint32_t)box_chans, (cuuint32_t)box_t, 1};
     if (pack > 1) {
@@ -1506,19 +1507,9 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e == cudaSuccess && items > 0) {
-        const int per_item = pair ? 2 : 1, slots = n_sm / per_item;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)(items < slots ? items : slots) * per_item);
-        cfg.blockDim = dim3(C::kThreads);
-        cfg.dynamicSmemBytes = (size_t)smem_bytes;
-        cfg.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = pair ? 1 : 0;
-        e = cudaLaunchKernelEx(&cfg, kern, *prm);
+        const int ctas = pair ? 2 : 1, slots = n_sm / ctas;
+        e = launch_kernel(kern, dim3((unsigned)(items < slots ? items : slots) * ctas), C::kThreads, (size_t)smem_bytes,
+                          s, ctas, false, *prm);
     }
     delete prm;
     return e;
@@ -1575,7 +1566,7 @@ bool tc_use_pairs(const Plan& p, bool packed) {
 // inputs 310 -> 311 / 405 -> 451 / 992 -> 1185 (256 samples: 374 -> 344, 360 -> 343).  4-bit (e4m3
 // planes): 256 inputs 89 -> 84 / 125 -> 109 / 303 -> 320, 512 inputs 342 -> 346 at 512 samples.
 bool tc_packed_pairs(const Plan& p) {
-    if (p.tc_operands != 0 || p.nb % 2 || !tc_use_pairs(p, true) || !tc_raw_supported(p)) return false;
+    if (p.tc_operands != 0 || p.nb % 2 || !tc_use_pairs(p, true)) return false;
     return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= 256 : p.nb == 4 && p.kp <= 512;
 }
 
@@ -1586,7 +1577,7 @@ int tc_kp_e4m3(const Plan& p) { return (p.n_time + 127) / 128 * 128; }
 cudaError_t launch_xeng_tc_e4m3_planes(const Plan& p, const void* d_planes, int n_dumps, void* d_vis, int accumulate,
                                        cudaStream_t s) {
     const int64_t rows = (int64_t)n_dumps * p.n_chan * p.nb * kBlockRows;
-    if (rows >= (int64_t)1 << 31 || !tc_planes_e4m3(p)) return cudaErrorInvalidValue;
+    if (rows >= (int64_t)1 << 31 || p.sample_bits != 4) return cudaErrorInvalidValue;
     const int kp8 = tc_kp_e4m3(p);
     CUtensorMap mh, mw;
     TcJobSpec sp{p.n_inputs, p.n_chan, p.n_time, n_dumps, p.sample_bits, d_planes, d_vis, 1};
@@ -1602,18 +1593,6 @@ cudaError_t launch_xeng_tc_e4m3_planes(const Plan& p, const void* d_planes, int 
         return launch_jobs<kPlanesF8, 1>(&sp, 1, &mh, nullptr, accumulate, p.d_status, p.n_sm, tune, s, &mw);
     }
     return launch_jobs<kPlanesF8, 1>(&sp, 1, &mh, nullptr, accumulate, p.d_status, p.n_sm, tune, s);
-}
-
-cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
-                                 int accumulate, cudaStream_t s) {
-    if (tc_packed_pairs(p) && (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0)
-        return launch_xeng_tc_raw(p, d_packed, n_dumps, d_vis, accumulate, s);
-    if (tc_planes_e4m3(p)) {
-        const cudaError_t e = launch_unpack_e4m3(p, d_packed, n_dumps, d_ws, s);
-        return e == cudaSuccess ? launch_xeng_tc_e4m3_planes(p, d_ws, n_dumps, d_vis, accumulate, s) : e;
-    }
-    const cudaError_t e = launch_unpack_fp16(p, d_packed, n_dumps, d_ws, s);
-    return e == cudaSuccess ? launch_xeng_tc(p, d_ws, nullptr, n_dumps, d_vis, accumulate, s) : e;
 }
 
 bool tc_use_planes(const Plan& p) {
@@ -1670,7 +1649,7 @@ int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm
 bool tc_make_raw_map(CUtensorMap* map, const TcJobSpec& sp, bool f8) {
     const int bps = sp.sample_bits == 8 ? 2 : 1;
     return make_raw_map(map, sp.data, sp.n_inputs, sp.n_chan, sp.n_time, sp.n_dumps, bps, sp.cpi,
-                        f8 ? Cfg<kRaw4F8>::kStageT : kTimeBlock, sp.pack);
+                        f8 ? Cfg<kRaw4F8>::kStageT : kTimeBlock, sp.pack, sp.row_pitch);
 }
 
 cudaError_t launch_xeng_tc_raw_jobs(const TcJobSpec* specs, const CUtensorMap* maps, int n_jobs, int accumulate,
@@ -1680,7 +1659,8 @@ cudaError_t launch_xeng_tc_raw_jobs(const TcJobSpec* specs, const CUtensorMap* m
     for (int j = 0; j < n_jobs; ++j)
         if (specs[j].sample_bits != bits || specs[j].pack < 1 ||
             (specs[j].pack > 1 ? specs[j].pack * specs[j].n_inputs > kBlockInputs
-                               : !tc_raw_supported(specs[j].n_inputs, bits)) ||
+             : specs[j].row_pitch ? specs[j].row_pitch % 16 != 0
+                                  : !tc_raw_supported(specs[j].n_inputs, bits)) ||
             (specs[j].cpi != 1 && specs[j].cpi != 2) || (specs[j].cpi == 2 && specs[j].n_inputs > kBlockInputs))
             return cudaErrorInvalidValue;
     if (tune.f8_operands) {   // e4m3 operands: 4-bit samples (maps with 128-sample boxes)
@@ -1741,9 +1721,10 @@ cudaError_t launch_xeng_tc_plane_jobs(const TcJobSpec* specs, const CUtensorMap*
 
 namespace {
 cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, void* d_vis, int accumulate,
-                            cudaStream_t s, const TcTuning* tune, int out_mode, const void* phasor, float inv_n) {
+                            cudaStream_t s, const TcTuning* tune, int out_mode, const void* phasor, float inv_n,
+                            int64_t pitch = 0) {
     const int bps = p.sample_bits == 8 ? 2 : 1;
-    const int pack = tc_channel_pack(p.n_inputs, bps, p.n_chan, n_dumps, p.n_sm);
+    const int pack = pitch ? 1 : tc_channel_pack(p.n_inputs, bps, p.n_chan, n_dumps, p.n_sm);
     if ((p.sample_bits != 4 && p.sample_bits != 8) || pack < 1 || (reinterpret_cast<uintptr_t>(d_packed) & 15u))
         return cudaErrorInvalidValue;
     TcTuning plan_tune;
@@ -1760,7 +1741,7 @@ cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, vo
     const int64_t items_per_dump = (int64_t)((chan_tiles + cpi - 1) / cpi) * (p.nb * (p.nb + 1) / 2);
     const int64_t max_dumps = ((int64_t{1} << 31) - 1) / items_per_dump;
     if (max_dumps < 1) return cudaErrorInvalidValue;
-    const size_t packed_dump = (size_t)p.n_time * p.n_chan * p.n_inputs * bps;
+    const size_t packed_dump = (size_t)p.n_time * p.n_chan * (pitch ? (size_t)pitch : (size_t)p.n_inputs * bps);
     const size_t vis_dump = (size_t)p.n_chan * (size_t)p.n_baselines * (out_mode ? 8 : 16);
     for (int d0 = 0; d0 < n_dumps;) {
         const int nd = (int)((n_dumps - d0) < max_dumps ? (n_dumps - d0) : max_dumps);
@@ -1768,6 +1749,7 @@ cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, vo
                      static_cast<const uint8_t*>(d_packed) + (size_t)d0 * packed_dump,
                      static_cast<uint8_t*>(d_vis) + (size_t)d0 * vis_dump, cpi};
         sp.pack = pack;
+        sp.row_pitch = pitch;
         sp.out_mode = out_mode;
         sp.phasor = phasor;
         sp.inv_n = inv_n;
@@ -1821,6 +1803,32 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
 cudaError_t launch_xeng_tc_raw(const Plan& p, const void* d_packed, int n_dumps, void* d_vis, int accumulate,
                                cudaStream_t s, const TcTuning* tune) {
     return launch_raw_impl(p, d_packed, n_dumps, d_vis, accumulate, s, tune, 0, nullptr, 1.0f);
+}
+
+// Rows that TMA cannot address (and channels that do not pack into tiles it can) go into the
+// workspace as rows of whole 16-byte pieces where the packed feed is the better one, and else
+// straight into planes (e4m3 for 4-bit samples: the workspace holds fp16 ones, twice as large).
+// Measured, 8-bit, 75 inputs x 333 channels x 777 samples x 2 dumps: 215 us with a general unpack into
+// fp16 planes (147 us of it the unpack), 109 us repacked.
+cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
+                                 int accumulate, cudaStream_t s) {
+    const bool ragged = !tc_raw_supported(p), aligned = (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0;
+    const bool packed = tc_packed_pairs(p) || (ragged && p.tc_operands == 0 &&
+                                               p.nb < (p.sample_bits == 4 ? kPlaneMinBlocksE4m3 : kPlaneMinBlocks));
+    if (packed && aligned) {
+        if (!ragged) return launch_xeng_tc_raw(p, d_packed, n_dumps, d_vis, accumulate, s);
+        if ((int64_t)n_dumps * p.n_time * p.n_chan < (int64_t{1} << 31)) {
+            const cudaError_t e = launch_repack(p, d_packed, n_dumps, d_ws, s);
+            if (e != cudaSuccess) return e;
+            return launch_raw_impl(p, d_ws, n_dumps, d_vis, accumulate, s, nullptr, 0, nullptr, 1.0f, repack_pitch(p));
+        }
+    }
+    if (p.sample_bits == 4) {
+        const cudaError_t e = launch_unpack_e4m3(p, d_packed, n_dumps, d_ws, s);
+        return e == cudaSuccess ? launch_xeng_tc_e4m3_planes(p, d_ws, n_dumps, d_vis, accumulate, s) : e;
+    }
+    const cudaError_t e = launch_unpack_fp16(p, d_packed, n_dumps, d_ws, s);
+    return e == cudaSuccess ? launch_xeng_tc(p, d_ws, nullptr, n_dumps, d_vis, accumulate, s) : e;
 }
 
 cudaError_t launch_xeng_tc_raw_dump(const Plan& p, const void* d_packed, int n_dumps, void* d_out, const void* phasor,
