@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "corr_internal.h"
+#include "launch.cuh"
 
 namespace corr {
 namespace {
@@ -24,6 +25,7 @@ constexpr int kDumpThreads = 256;
 
 __global__ void phasor_kernel(const double* __restrict__ tau, const double* __restrict__ nu, int N, int C,
                               float2* __restrict__ g) {
+    grid_release();
     const int64_t total = (int64_t)N * C;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
@@ -117,8 +119,8 @@ cudaError_t launch_phasors(const Plan& p, const double* d_delays, const double* 
     const int64_t total = (int64_t)p.n_inputs * p.n_chan;
     const int64_t want = (total + kDumpThreads - 1) / kDumpThreads;
     const int blocks = (int)(want < 4096 ? want : 4096);
-    phasor_kernel<<<blocks, kDumpThreads, 0, s>>>(d_delays, d_freqs, p.n_inputs, p.n_chan, static_cast<float2*>(d_g));
-    return cudaGetLastError();
+    return launch_kernel(phasor_kernel, dim3(blocks), kDumpThreads, 0, s, 1, false, d_delays, d_freqs, p.n_inputs, p.n_chan,
+                          static_cast<float2*>(d_g));
 }
 
 }  // namespace corr

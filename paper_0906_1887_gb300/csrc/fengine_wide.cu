@@ -37,6 +37,7 @@
 #include "corr_internal.h"
 #include "fengine_wide.h"
 #include "fft_reg.cuh"
+#include "launch.cuh"
 
 namespace corr {
 namespace {
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, 0>::T, 1024 / FW<KIND, LGL, 0>::
     const int n0 = blockIdx.x * F::G;
     const int g_n = min(F::G, N - n0);
     for (int k = threadIdx.x; k < F::TWN; k += F::T) tws[k] = tw[k];
+    grid_release();
     const int n_batches = (n_frames + F::FB - 1) / F::FB;
     const size_t frame_bytes = (size_t)F::L * N * F::BPS;
     const uint8_t* const in0 = in + (size_t)n0 * F::BPS;
@@ -442,6 +444,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
         }
     };
     Raw w[4][SPP];
+    grid_release();
     if (f0 < f1) {
         for (int t = f0; t < f0 + MT - 1; ++t) {   // the run's first sums
             float2 y[4];
@@ -510,9 +513,8 @@ cudaError_t launch_plain(const FWideArgs& p, cudaStream_t s) {
     const int rows = fw_rows(groups, (p.n_frames + F::FB - 1) / F::FB, p.n_sm * kPerSm);
     const int vec = F::PIECE >= 4 && (size_t)p.n_inputs * F::BPS % F::PIECE == 0 &&
                     reinterpret_cast<uintptr_t>(p.d_in) % F::PIECE == 0;
-    kern<<<dim3(groups, rows), F::T, F::SMEM, s>>>(static_cast<const uint8_t*>(p.d_in), static_cast<float2*>(p.d_out),
-                                                   static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames, vec);
-    return cudaGetLastError();
+    return launch_kernel(kern, dim3(groups, rows), F::T, F::SMEM, s, 1, false, static_cast<const uint8_t*>(p.d_in),
+                          static_cast<float2*>(p.d_out), static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames, vec);
 }
 
 template <int KIND, int LGL, int MT>
@@ -526,10 +528,9 @@ cudaError_t launch_pfb(const FWideArgs& p, cudaStream_t s) {
     const int rows = fw_rows(groups, batches, p.n_sm * (512 / F::T));
     const int run = (batches + rows - 1) / rows * 4;
     const int vec = (size_t)p.n_inputs % 4 == 0 && reinterpret_cast<uintptr_t>(p.d_in) % (4 * F::BPS) == 0;
-    kern<<<dim3(groups, rows), F::T, F::SMEM, s>>>(static_cast<const uint8_t*>(p.d_in), static_cast<float2*>(p.d_out),
-                                                   static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames, run,
-                                                   p.d_taps, p.n_taps, vec);
-    return cudaGetLastError();
+    return launch_kernel(kern, dim3(groups, rows), F::T, F::SMEM, s, 1, false, static_cast<const uint8_t*>(p.d_in),
+                          static_cast<float2*>(p.d_out), static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames, run,
+                          p.d_taps, p.n_taps, vec);
 }
 
 template <int KIND, int LGL>

@@ -298,6 +298,7 @@ cudaError_t launch_fast(const Plan& p, const void* d_packed, int n_dumps, void* 
 __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __restrict__ packed,
                                                      unsigned char* __restrict__ out, uint32_t rows, int row_bytes,
                                                      int pieces, uint32_t rows_per_block, int64_t last_word) {
+    grid_release();
     for (uint32_t r0 = blockIdx.x * rows_per_block; r0 < rows; r0 += gridDim.x * rows_per_block) {
         const uint32_t n = min(rows_per_block, rows - r0) * (uint32_t)pieces;
         uint4* dst = reinterpret_cast<uint4*>(out) + (int64_t)r0 * pieces;

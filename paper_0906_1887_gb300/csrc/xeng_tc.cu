@@ -592,6 +592,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     }
     ptx::tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    grid_wait();   // samples and outputs may be the preceding kernel's
+    grid_release();
 
 
     if (warp == 0) {
@@ -1509,7 +1511,7 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     if (e == cudaSuccess && items > 0) {
         const int ctas = pair ? 2 : 1, slots = n_sm / ctas;
         e = launch_kernel(kern, dim3((unsigned)(items < slots ? items : slots) * ctas), C::kThreads, (size_t)smem_bytes,
-                          s, ctas, false, *prm);
+                          s, ctas, C::kRaw, *prm);
     }
     delete prm;
     return e;
