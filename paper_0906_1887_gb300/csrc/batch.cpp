@@ -42,6 +42,7 @@ struct TuneChoice {
     int order = 0;       // 0: items of the costliest jobs first; 1: jobs in the caller's order
     int plane_min_nb = 0;   // jobs of at least this many 64-input blocks read fp16 planes (0: none)
     int wide = 1;           // plane jobs: wide items (block I against J, J + 1 in one MMA)
+    int pair = 1;           // arrays of several blocks: CTA pairs on squares of tiles
     int plane_splits = 1;   // plane jobs in this many launches, each next one's unpack beside the last
     float ms = 0.f;
 };
@@ -61,6 +62,7 @@ std::map<std::string, TuneChoice> g_tune_cache;
 struct ModeGroup {
     int bits = 0;
     bool planes = false;                  // jobs read fp16 planes the unpack kernel writes first
+    bool multi = false;                   // arrays of several blocks (a launch of CTA pairs takes no others)
     std::vector<int> job_index;           // caller's job indices in this group
     std::vector<TcJobSpec> specs;         // launch order
     std::vector<CUtensorMap> maps;
@@ -130,12 +132,19 @@ bool build_groups(corr_batch_s* b, const TuneChoice& ch) {
     b->groups.clear();
     b->items = 0;
     for (int bits : {8, 4}) {
-        for (bool planes : {false, true}) {
+        // packed samples: one launch for arrays of several blocks and one for the single-block ones
+        // where the former run in CTA pairs, else one for both; then the plane jobs
+        for (int form = 0; form < 3; ++form) {
+            const bool planes = form == 2;
+            if (form == 1 && !ch.pair) continue;
             ModeGroup g;
             g.bits = bits;
             g.planes = planes;
+            g.multi = planes || (ch.pair && form == 0);
             for (int k = 0; k < (int)b->jobs.size(); ++k)
-                if (b->jobs[k].sample_bits == bits && takes_planes(b, ch, k) == planes) g.job_index.push_back(k);
+                if (b->jobs[k].sample_bits == bits && takes_planes(b, ch, k) == planes &&
+                    (planes || !ch.pair || (blocks_of(b->jobs[k]) > 1) == g.multi))
+                    g.job_index.push_back(k);
             if (g.job_index.empty()) continue;
             auto cpi_of = [&](const corr_job& j) { return !planes && j.n_inputs <= kBlockInputs ? ch.pair_cpi : 1; };
             if (ch.order == 0)
@@ -159,16 +168,18 @@ bool build_groups(corr_batch_s* b, const TuneChoice& ch) {
                 CUtensorMap m, mw{};
                 if (!(planes ? tc_make_plane_map(&m, sp, f8) : tc_make_raw_map(&m, sp, f8))) return false;
                 const int nb = blocks_of(j);
-                if (planes && ch.wide && nb >= 2 && tc_make_plane_map_wide(&mw, sp, f8)) sp.tw = 2;
+                if (planes && ch.wide && !ch.pair && nb >= 2 && tc_make_plane_map_wide(&mw, sp, f8)) sp.tw = 2;
                 g.specs.push_back(sp);
                 g.maps.push_back(m);
                 g.maps_wide.push_back(mw);
-                const int per_chan = sp.tw == 2 ? ((nb + 1) / 2) * ((nb + 2) / 2) : nb * (nb + 1) / 2;
+                const int ng = (nb + 1) / 2;
+                const int per_chan = g.multi && ch.pair ? ng * (ng + 1) / 2 : sp.tw == 2 ? ((nb + 1) / 2) * ((nb + 2) / 2) : nb * (nb + 1) / 2;
                 const int chan_tiles = (j.n_chan + sp.pack - 1) / sp.pack;
                 b->items += (int64_t)((chan_tiles + sp.cpi - 1) / sp.cpi) * per_chan;
             }
             g.tune.op_stages = ch.op_stages;
             g.tune.f8_operands = f8 ? 1 : 0;
+            g.tune.pair = g.multi && ch.pair ? 1 : 0;
             b->groups.push_back(std::move(g));
         }
     }
@@ -312,6 +323,7 @@ void load_cache_file(const char* path) {
         if ((p = strstr(k1, "\"order\": "))) c.order = atoi(p + 9);
         if ((p = strstr(k1, "\"plane_min_nb\": "))) c.plane_min_nb = atoi(p + 16);
         if ((p = strstr(k1, "\"wide\": "))) c.wide = atoi(p + 8);
+        if ((p = strstr(k1, "\"pair\": "))) c.pair = atoi(p + 8);
         if ((p = strstr(k1, "\"plane_splits\": "))) c.plane_splits = atoi(p + 16);
         if ((p = strstr(k1, "\"ms\": "))) c.ms = (float)atof(p + 6);
         if (c.pair_cpi != 1 && c.pair_cpi != 2) continue;
@@ -327,8 +339,8 @@ void append_cache_file(const char* path, const std::string& key, const TuneChoic
     if (!f) return;
     fprintf(f,
             "{\"key\": \"%s\", \"op_stages\": %d, \"pair_cpi\": %d, \"order\": %d, \"plane_min_nb\": %d, "
-            "\"wide\": %d, \"plane_splits\": %d, \"ms\": %.6f}\n",
-            key.c_str(), c.op_stages, c.pair_cpi, c.order, c.plane_min_nb, c.wide, c.plane_splits, c.ms);
+            "\"wide\": %d, \"pair\": %d, \"plane_splits\": %d, \"ms\": %.6f}\n",
+            key.c_str(), c.op_stages, c.pair_cpi, c.order, c.plane_min_nb, c.wide, c.pair, c.plane_splits, c.ms);
     fclose(f);
 }
 
@@ -382,24 +394,10 @@ corr_status autotune(corr_batch_s* b, const char* cache_path) {
     if (b->d_planes)
         for (int nb : {2, 4, 8, 16})
             if (nb <= max_nb) plane_opts.push_back(nb);
-    std::vector<TuneChoice> cands;
-    for (int order : {0, 1})
-        for (int cpi : any_small ? std::vector<int>{2, 1} : std::vector<int>{2})
-            for (int ops : {3, 4, 5})
-                for (int pm : plane_opts)
-                    for (int wide : pm ? std::vector<int>{1, 0} : std::vector<int>{1}) {
-                        TuneChoice c;
-                        c.op_stages = ops;
-                        c.pair_cpi = cpi;
-                        c.order = order;
-                        c.plane_min_nb = pm;
-                        c.wide = wide;
-                        cands.push_back(c);
-                    }
     TuneChoice best;
     float best_ms = 1e30f;
     cudaStream_t s = b->own_stream;
-    for (auto& c : cands) {
+    auto trial = [&](TuneChoice c) {   // time one shape and keep the fastest
         b->choice = c;
         if (!build_groups(b, c)) return set_error(CORR_EINVAL, "tensor map encoding failed");
         cudaError_t err;
@@ -410,24 +408,36 @@ corr_status autotune(corr_batch_s* b, const char* cache_path) {
             best_ms = ms;
             best = c;
         }
-    }
+        return CORR_OK;
+    };
+    corr_status st = CORR_OK;
+    for (int pair : max_nb > 1 ? std::vector<int>{1, 0} : std::vector<int>{0})
+        for (int order : {0, 1})
+            for (int cpi : any_small ? std::vector<int>{2, 1} : std::vector<int>{2})
+                for (int ops : {3, 4, 5})
+                    for (int pm : plane_opts)
+                        for (int wide : pm && !pair ? std::vector<int>{1, 0} : std::vector<int>{1}) {
+                            // single CTAs: only around the shape that pairs chose
+                            if (!pair && max_nb > 1 && (order != best.order || cpi != best.pair_cpi)) continue;
+                            TuneChoice c;
+                            c.op_stages = ops;
+                            c.pair_cpi = cpi;
+                            c.order = order;
+                            c.plane_min_nb = pm;
+                            c.wide = wide;
+                            c.pair = pair;
+                            if (st == CORR_OK) st = trial(c);
+                        }
     // second stage: the best shape with its plane jobs split into overlapped launches
     if (best.plane_min_nb > 0) {
+        const TuneChoice base = best;
         for (int splits : {2, 3, 4}) {
-            TuneChoice c = best;
+            TuneChoice c = base;
             c.plane_splits = splits;
-            b->choice = c;
-            if (!build_groups(b, c)) return set_error(CORR_EINVAL, "tensor map encoding failed");
-            cudaError_t err;
-            const float ms = time_groups(b, s, 3, &err);
-            if (err != cudaSuccess) return cuda_error(err, "autotune run");
-            c.ms = ms;
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = c;
-            }
+            if (st == CORR_OK) st = trial(c);
         }
     }
+    if (st != CORR_OK) return st;
     b->choice = best;
     b->tuned = true;
     {
@@ -536,6 +546,10 @@ corr_status corr_batch_create(corr_batch* out, const corr_job* jobs, int n_jobs,
     } else {
         TuneChoice def;
         if (b->d_planes) def.plane_min_nb = 4;   // untuned: arrays of 256 inputs and more read planes
+        // untuned: CTA pairs where they need no launch of their own
+        def.pair = 1;
+        for (const auto& j : b->jobs)
+            if (blocks_of(j) < 2) def.pair = 0;
         b->choice = def;
         if (!build_groups(b, def)) st = set_error(CORR_EINVAL, "tensor map encoding failed");
     }
@@ -569,6 +583,7 @@ corr_status corr_batch_set_shape(corr_batch b, int op_stages, int pair_cpi, int 
     c.order = order;
     c.plane_min_nb = plane_min_nb;
     c.wide = wide;
+    c.pair = wide;   // the single tiles of wide = 0 are single CTAs'
     c.plane_splits = plane_splits;
     if (!build_groups(b, c)) return set_error(CORR_EINVAL, "tensor map encoding failed");
     b->choice = c;
