@@ -98,7 +98,8 @@ bool tc_raw_by_packing(const Plan& p);
 // public planes calls (corr_unpack, corr_xengine_run_planes) keep fp16 planes.
 bool tc_planes_e4m3(const Plan& p);
 bool tc_use_pairs(const Plan& p, bool packed);   // CTA pairs (PAIR in xeng_tc.cu) rather than single CTAs
-bool tc_packed_pairs(const Plan& p);             // packed feed with pairs although the plan has a plane workspace
+// the packed feed although the plan has a plane workspace
+bool tc_packed_pairs(const Plan& p, int accumulate);
 int tc_kp_e4m3(const Plan& p);
 size_t tc_workspace_planes_bytes(const Plan& p, int n_dumps);
 cudaError_t launch_unpack_e4m3(const Plan& p, const void* d_packed, int n_dumps, void* d_planes, cudaStream_t s,

@@ -1567,8 +1567,16 @@ bool tc_use_pairs(const Plan& p, bool packed) {
 // 512 inputs 273 -> 255 / 427 -> 392 / 998 -> 936, 768 inputs 321 -> 313 / 432 -> 446 / 990 -> 1085, 1024
 // inputs 310 -> 311 / 405 -> 451 / 992 -> 1185 (256 samples: 374 -> 344, 360 -> 343).  4-bit (e4m3
 // planes): 256 inputs 89 -> 84 / 125 -> 109 / 303 -> 320, 512 inputs 342 -> 346 at 512 samples.
-bool tc_packed_pairs(const Plan& p) {
-    if (p.tc_operands != 0 || p.nb % 2 || !tc_use_pairs(p, true)) return false;
+// Accumulating dumps gain more: the read-modify-write of the sums leaves the packed feed's port and
+// the memory system less to share than planes do.  8-bit, 400 inputs x 512 / 1024 samples 424 -> 358 /
+// 702 -> 642, 1024 x 512 / 768 / 1024 536 -> 446 / 579 -> 549 / 666 -> 695; 4-bit, 192 x 384 94 -> 77,
+// 400 x 512 320 -> 308, 1024 x 512 / 768 527 -> 488 / 505 -> 457, but 400 x 768 356 -> 417.
+bool tc_packed_pairs(const Plan& p, int accumulate) {
+    if (p.tc_operands != 0 || p.tc_items != 0 || p.nb < 2) return false;
+    const bool even = p.nb % 2 == 0;
+    if (accumulate)
+        return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= (p.nb <= 12 ? 1024 : 768) : p.kp <= (even ? 768 : 512);
+    if (!even || !tc_use_pairs(p, true)) return false;
     return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= 256 : p.nb == 4 && p.kp <= 512;
 }
 
@@ -1815,7 +1823,7 @@ cudaError_t launch_xeng_tc_raw(const Plan& p, const void* d_packed, int n_dumps,
 cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
                                  int accumulate, cudaStream_t s) {
     const bool ragged = !tc_raw_supported(p), aligned = (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0;
-    const bool packed = tc_packed_pairs(p) || (ragged && p.tc_operands == 0 &&
+    const bool packed = tc_packed_pairs(p, accumulate) || (ragged && p.tc_operands == 0 &&
                                                p.nb < (p.sample_bits == 4 ? kPlaneMinBlocksE4m3 : kPlaneMinBlocks));
     if (packed && aligned) {
         if (!ragged) return launch_xeng_tc_raw(p, d_packed, n_dumps, d_vis, accumulate, s);

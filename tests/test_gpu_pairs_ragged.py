@@ -44,7 +44,8 @@ def test_pairs_bit_exact(feed, n, c, t, bits):
     _check(n, c, t, bits, PLANES if feed == "planes" else (PACKED if bits == 8 else PACKED_F8))
 
 
-@pytest.mark.parametrize("n,c,t,bits,n_dumps", [(96, 5, 400, 8, 3), (128, 7, 1100, 8, 1), (256, 3, 600, 4, 2), (512, 2, 200, 8, 2)])
+@pytest.mark.parametrize("n,c,t,bits,n_dumps", [(96, 5, 400, 8, 3), (128, 7, 1100, 8, 1), (256, 3, 600, 4, 2), (512, 2, 200, 8, 2),
+                                                (192, 3, 500, 4, 1), (320, 2, 300, 4, 2), (400, 2, 260, 8, 1)])
 def test_pairs_dumps_and_accumulate(n, c, t, bits, n_dumps):
     _check(n, c, t, bits, n_dumps=n_dumps)
     _check(n, c, t, bits, n_dumps=n_dumps, accumulate=True)
