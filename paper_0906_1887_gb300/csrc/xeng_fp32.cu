@@ -635,11 +635,14 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
 //
 // Float samples need no conversion: 16-byte pieces (two inputs' (re, im)) go from the packed rows
 // into the float2 rows with cp.async, into one of two row buffers while the block computes on the
-// other (16-sample chunks, so both buffers of four diagonal or two off-diagonal channel-dumps fit
-// two blocks per SM).  Accuracy as in the kernels above: fp32 partials over 64 samples, each added
-// into the float32 output (the first stored unless accumulating or split over sample ranges,
-// later ones by vector float2 reductions, one writing thread per element).
-constexpr int kFChunk = 16;
+// other.  Accuracy as in the kernels above: fp32 partials over 64 samples.  Their totals stay in
+// shared memory, thread-private 16-byte pieces, and reach the output once per item (a store, or a
+// float2 reduction when accumulating or split over sample ranges); adding every partial into the
+// output took one scattered reduction per element and 64 samples, a quarter of the time (64 inputs x
+// 768 channels x 1000 samples: 391 -> 300 us with the fuller waves of sample_ranges, 0.57 of the FFMA
+// rate; what is left is issue and dispatch in the FFMA stream).  Chunks of 8 samples leave both row buffers of four diagonal
+// or two off-diagonal channel-dumps (40 KB) and the totals (64 KB) room for two blocks per SM.
+constexpr int kFChunk = 8;
 constexpr int kFSeg = 64;
 
 template <int NBLK, int KCH, int NT>
@@ -679,9 +682,10 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
     constexpr int kThreads = DIAG ? kIDiagThreads : kIOffThreads;
     constexpr int NBLK = DIAG ? 1 : 2;
     constexpr int kBuf = kCh * NBLK * kFChunk * kIRow;   // float2 slots of one row buffer
-    // two row buffers [kCh][NBLK][kFChunk][kIRow], then the item
+    // two row buffers [kCh][NBLK][kFChunk][kIRow], the totals [16][kThreads] of 16 bytes, the item
     extern __shared__ __align__(16) float2 s_dyn[];
-    IItem<kCh>* item_s = reinterpret_cast<IItem<kCh>*>(s_dyn + 2 * kBuf);
+    float4* const tot = reinterpret_cast<float4*>(s_dyn + 2 * kBuf) + threadIdx.x;
+    IItem<kCh>* item_s = reinterpret_cast<IItem<kCh>*>(s_dyn + 2 * kBuf + 32 * kThreads);
     const volatile IItem<kCh>* info = item_s;
     const int tid = threadIdx.x;
     const float2 *sa, *sb;
@@ -749,10 +753,10 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
                 const float2* pa = sa + buf * kBuf;
                 const float2* pb = sb + buf * kBuf;
                 if (DIAG && tri) {   // warp-uniform
-#pragma unroll 1
+#pragma unroll 2
                     for (int t = 0; t < kFChunk; ++t) itri(acc, ild4(pa + t * kIRow), ild4(pa + t * kIRow + 4));
                 } else {
-#pragma unroll 1
+#pragma unroll 2
                     for (int t = 0; t < kFChunk; ++t) {
                         const IRows a = ild4(pa + t * kIRow), b0 = ild4(pb + t * kIRow), b1 = ild4(pb + t * kIRow + 4);
                         icmac(acc, a, b0, 0);
@@ -760,10 +764,27 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
                     }
                 }
             }
+            // the segment's partials into the totals, in the order of the segments
+            if (s0 > sbeg) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const float4 o = tot[k * kThreads];
+                    acc[4 * k] = o.x + acc[4 * k];
+                    acc[4 * k + 1] = o.y + acc[4 * k + 1];
+                    acc[4 * k + 2] = o.z + acc[4 * k + 2];
+                    acc[4 * k + 3] = o.w + acc[4 * k + 3];
+                }
+            }
+            if (s1 < info->s_end) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k)
+                    tot[k * kThreads] = make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+                continue;
+            }
             const ISub<DIAG> u(tid);
             const int64_t dc = info->dc0 + u.q;
             if (dc >= n_dc) continue;
-            const bool add = accumulate || s0 > sbeg || ts > 1;
+            const bool add = accumulate || ts > 1;
             const int I = info->I, J = info->J;
             const int64_t row0 = dc * P;
             auto row_of = [&](int i) { return row0 + (int64_t)i * n_inputs - (int64_t)i * (i - 1) / 2 - i; };
@@ -801,18 +822,28 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
 }
 
 // Sample ranges per item for a launch of base_items items: with fewer than two waves of two
-// blocks per SM, the sample axis is split (whole chunks, at least 64 samples a range).
+// blocks per SM, the sample axis is split (whole chunks, at least 64 samples a range) so that the
+// waves are full: the number of ranges with the smallest waves x (range + some 24 samples an item
+// costs besides).  768 channels of 64 inputs (192 items, 304 blocks), 1000 samples: 3 ranges run
+// in 2 waves of 352 samples where 4 took 3 waves of 256.
 void sample_ranges(const Plan& p, int64_t base_items, int* ts, int* range_len) {
-    const int64_t target = 4LL * p.n_sm;
-    int64_t t = 1;
-    if (base_items > 0 && base_items < target) t = (target + base_items - 1) / base_items;
-    const int64_t t_max = (p.n_time + 63) / 64;
-    if (t > t_max) t = t_max;
-    if (t < 1) t = 1;
-    int len = (int)((p.n_time + t - 1) / t);
-    len = (len + kIChunk - 1) / kIChunk * kIChunk;
-    *range_len = len;
-    *ts = (p.n_time + len - 1) / len;
+    const int64_t slots = 2LL * p.n_sm;
+    int best_len = (p.n_time + kIChunk - 1) / kIChunk * kIChunk;
+    if (base_items > 0 && base_items < 2 * slots) {
+        int64_t best = INT64_MAX;
+        const int t_max = (p.n_time + 63) / 64 < 64 ? (p.n_time + 63) / 64 : 64;
+        for (int t = 1; t <= t_max; ++t) {
+            const int len = ((p.n_time + t - 1) / t + kIChunk - 1) / kIChunk * kIChunk;
+            const int n = (p.n_time + len - 1) / len;
+            const int64_t cost = (base_items * n + slots - 1) / slots * (len + 24);
+            if (cost < best) {
+                best = cost;
+                best_len = len;
+            }
+        }
+    }
+    *range_len = best_len;
+    *ts = (p.n_time + best_len - 1) / best_len;
 }
 
 template <int BITS, bool VEC>
@@ -867,9 +898,11 @@ cudaError_t launch_float_feed(const Plan& p, const float2* src, int64_t n_dc, fl
     sample_ranges(p, diag_base, &ts_d, &len_d);
     sample_ranges(p, off_base, &ts_o, &len_o);
     const int64_t diag_items = diag_base * ts_d, off_items = off_base * ts_o;
-    // two row buffers (10 KB per channel-dump and block each) and the item: 80 KB
-    const int smem_diag = 2 * kIDiagCh * kFChunk * kIRow * (int)sizeof(float2) + (int)sizeof(IItem<kIDiagCh>);
-    const int smem_off = 2 * kIOffCh * 2 * kFChunk * kIRow * (int)sizeof(float2) + (int)sizeof(IItem<kIOffCh>);
+    // two row buffers (5 KB per channel-dump and block each), 256 bytes of totals per thread, the item
+    const int smem_diag = 2 * kIDiagCh * kFChunk * kIRow * (int)sizeof(float2) + 256 * kIDiagThreads +
+                          (int)sizeof(IItem<kIDiagCh>);
+    const int smem_off = 2 * kIOffCh * 2 * kFChunk * kIRow * (int)sizeof(float2) + 256 * kIOffThreads +
+                         (int)sizeof(IItem<kIOffCh>);
     const int64_t P = p.n_baselines, tstride = (int64_t)p.n_chan * p.n_inputs;
     cudaError_t e = cudaFuncSetAttribute(xeng_fp32_float_kernel<true, VEC>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem_diag);
