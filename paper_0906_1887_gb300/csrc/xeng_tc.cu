@@ -449,12 +449,15 @@ __device__ __forceinline__ void convert_words4_f8(const uint32_t (&w)[16], uint3
 // rows l + 32 kk (kk = 0..3) of samples 8q .. 8q + 7 and writes each row's 16-byte chunk q of
 // the hi tile and of the lo tile (kTileBytes further).  A quarter-warp's rows differ in
 // (row & 7), so its swizzled chunks fall in distinct banks.
+__device__ __forceinline__ uint32_t bf16x2_bits(float a, float b) {   // a in the low half
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
 __device__ __forceinline__ uint32_t bf16_pair(float a, float b, uint32_t& lo) {
-    const __nv_bfloat16 ha = __float2bfloat16_rn(a), hb = __float2bfloat16_rn(b);
-    const __nv_bfloat16 la = __float2bfloat16_rn(a - __bfloat162float(ha));
-    const __nv_bfloat16 lb = __float2bfloat16_rn(b - __bfloat162float(hb));
-    lo = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
-    return (uint32_t)__bfloat16_as_ushort(ha) | ((uint32_t)__bfloat16_as_ushort(hb) << 16);
+    const uint32_t h = bf16x2_bits(a, b);   // one conversion for both, and again for what it dropped
+    lo = bf16x2_bits(a - __uint_as_float(h << 16), b - __uint_as_float(h & 0xFFFF0000u));
+    return h;
 }
 
 __device__ __forceinline__ void convert_slice_f32(uint32_t raw_tile, uint32_t dst_hi, int q, int lane) {
