@@ -231,7 +231,10 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, uint32_t m, int s) {
 // against blocks J = 2 b and J + 1.
 template <int MAXJ, bool PAIR>
 __device__ __forceinline__ void decode_item(const TcLaunch<MAXJ>& L, int64_t item, int& j, ItemCtx& it, int rank) {
-    while (j + 1 < L.n_jobs && item >= L.jobs[j + 1].item_begin) ++j;
+    // single-job launches: a constant index, so the job's fields are plain parameter operands
+    if constexpr (MAXJ == 1) j = 0;
+    else
+        while (j + 1 < L.n_jobs && item >= L.jobs[j + 1].item_begin) ++j;
     const TcJob& jb = L.jobs[j];
     const uint32_t local = (uint32_t)(item - jb.item_begin);   // < 2^31 per job (host-checked)
     const uint32_t dg = fast_div(local, jb.tiles_m, jb.tiles_s);
@@ -614,7 +617,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
                 ItemCtx it;
                 decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
-                const TcJob& jb = prm.jobs[it.j];
+                const TcJob& jb = prm.jobs[MAXJ == 1 ? 0 : it.j];
                 const int I = it.I, J = it.J;
                 const bool same = it.same;
                 const int nkb = jb.kp / C::kStageT;
@@ -700,7 +703,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
                     ItemCtx it;
                     decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
-                    const int nkb = prm.jobs[it.j].kp / C::kStageT;
+                    const int nkb = prm.jobs[MAXJ == 1 ? 0 : it.j].kp / C::kStageT;
                     for (int kb = 0; kb < nkb; ++kb) {
                         if (!ptx::mbar_wait_bounded(bar_op_full + 8 * s, ph, abort_flag, prm.wait_limit_ns)) {
                             record_error(prm.status, abort_flag, kDevTimeoutFull, kb);
@@ -740,7 +743,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
                 ItemCtx it;
                 decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
-                const TcJob& jb = prm.jobs[it.j];
+                const TcJob& jb = prm.jobs[MAXJ == 1 ? 0 : it.j];
                 const uint32_t idesc = jb.idesc;
                 const bool same = it.same;
                 const int nkb = jb.kp / C::kStageT;
@@ -854,7 +857,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
             ItemCtx it;
             decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
-            const TcJob& jb = prm.jobs[it.j];
+            const TcJob& jb = prm.jobs[MAXJ == 1 ? 0 : it.j];
             const int n_in = jb.n_inputs;
             const int P = n_in * (n_in + 1) / 2;
             const int I = it.I, J = it.J;
@@ -1191,10 +1194,10 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         for (int64_t item = item0; ok && item < prm.n_items; item += item_step) {
             ItemCtx it;
             decode_item<MAXJ, PAIR>(prm, item, jc, it, rank);
-            const int cpi = prm.jobs[it.j].cpi;
-            const uint32_t pair_off = (uint32_t)prm.jobs[it.j].pair_off;
+            const int cpi = prm.jobs[MAXJ == 1 ? 0 : it.j].cpi;
+            const uint32_t pair_off = (uint32_t)prm.jobs[MAXJ == 1 ? 0 : it.j].pair_off;
             const bool same = it.same;
-            const int nkb = prm.jobs[it.j].kp / C::kStageT;
+            const int nkb = prm.jobs[MAXJ == 1 ? 0 : it.j].kp / C::kStageT;
             // The stage holds n_tl packed tiles: cpi channels side by side in each sample row
             // (diagonal items, row pitch cpi x kRow), or blocks I and J (off-diagonal items,
             // pitch kRow).  Each tile splits into warp-sized slices (8 for 8-bit, 4 for 4-bit);
