@@ -218,29 +218,17 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
                 }
             } else if constexpr (F8) {
                 // as below, each row's 8 samples written as 8 e4m3 bytes (rows of kp bytes)
-                const __half2 bias = conv::bias4();
                 unsigned char* out8 = static_cast<unsigned char*>(planes_out) + row0 * kp +
                                       (int64_t)tb * kTimeBlock + 8 * q;
-                uint32_t hi[8], lo[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    hi[e] = (w[e] >> 4) & 0x0F0F0F0Fu;
-                    lo[e] = w[e] & 0x0F0F0F0Fu;
-                }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const uint32_t sel = conv::lane_selector(k);
-                    uint2 o;
-                    o.x = conv::e4m3x4(conv::pair_to_half2(hi[0], hi[1], sel, conv::kFlip4, bias),
-                                       conv::pair_to_half2(hi[2], hi[3], sel, conv::kFlip4, bias));
-                    o.y = conv::e4m3x4(conv::pair_to_half2(hi[4], hi[5], sel, conv::kFlip4, bias),
-                                       conv::pair_to_half2(hi[6], hi[7], sel, conv::kFlip4, bias));
-                    *reinterpret_cast<uint2*>(out8 + (int64_t)(8 * pw + 2 * k) * kp) = o;
-                    o.x = conv::e4m3x4(conv::pair_to_half2(lo[0], lo[1], sel, conv::kFlip4, bias),
-                                       conv::pair_to_half2(lo[2], lo[3], sel, conv::kFlip4, bias));
-                    o.y = conv::e4m3x4(conv::pair_to_half2(lo[4], lo[5], sel, conv::kFlip4, bias),
-                                       conv::pair_to_half2(lo[6], lo[7], sel, conv::kFlip4, bias));
-                    *reinterpret_cast<uint2*>(out8 + (int64_t)(8 * pw + 2 * k + 1) * kp) = o;
+                    constexpr uint32_t kSel[4] = {conv::gather_selector(0), conv::gather_selector(1),
+                                                  conv::gather_selector(2), conv::gather_selector(3)};
+                    uint2 re, im;
+                    conv::e4m3_of_nibbles(conv::gather4(w[0], w[1], w[2], w[3], kSel[k]), re.x, im.x);
+                    conv::e4m3_of_nibbles(conv::gather4(w[4], w[5], w[6], w[7], kSel[k]), re.y, im.y);
+                    *reinterpret_cast<uint2*>(out8 + (int64_t)(8 * pw + 2 * k) * kp) = re;
+                    *reinterpret_cast<uint2*>(out8 + (int64_t)(8 * pw + 2 * k + 1) * kp) = im;
                 }
             } else {
                 // word pw = inputs 4pw .. 4pw + 3, high nibble re, low nibble im -> rows 8pw + 2k (+1)

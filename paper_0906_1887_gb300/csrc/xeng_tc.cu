@@ -52,7 +52,6 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
-#include <cuda_fp8.h>
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -397,9 +396,9 @@ __device__ __forceinline__ void convert_words4(const uint32_t (&w)[8], uint32_t 
 
 // The e4m3 converter's lane constants: input 4m + k at step kk with k = (kk + m) & 3, its re row
 // 2(4m + k) first and the im row after it.  Its stores are half as many as the fp16 ones and
-// conflict in pairs; the conflict-free order of conv_lane4 and its loads (a variable shift per
-// word, permuted row addresses) measured slower here (1.51-1.55 against 1.45 ms on a 4-bit
-// stream of 64 inputs x 768 channels x 50 dumps) though faster for the fp16 converter.
+// conflict in pairs; the conflict-free order of conv_lane4 and its loads (permuted row addresses,
+// a lane-dependent order of the two rows) measured slower here (99 against 97 us on a 4-bit
+// stream of 64 inputs x 768 channels x 4 dumps, 75 against 71 on 128 x 512 x 2048).
 __device__ __forceinline__ ConvLane conv_lane4_f8(int l) {
     ConvLane c;
     const int m = l & 15;
@@ -407,7 +406,7 @@ __device__ __forceinline__ ConvLane conv_lane4_f8(int l) {
     for (int kk = 0; kk < 4; ++kk) {
         const int k = (kk + m) & 3;
         const int row = 2 * (4 * m + k);
-        c.sel[kk] = lane_selector(k);
+        c.sel[kk] = conv::gather_selector(k);
         c.rowoff[kk] = (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
         c.r7x16[kk] = (uint32_t)((row & 7) << 4);
     }
@@ -420,14 +419,6 @@ __device__ __forceinline__ ConvLane conv_lane4_f8(int l) {
 // w[e] = inputs 4m .. 4m+3 (m = l & 15) of sample 16c + e, e = 0..15, and writes, for the re
 // and im rows of each of its four inputs, the row's 16-byte chunk c (16 samples).
 __device__ __forceinline__ void convert_words4_f8(const uint32_t (&w)[16], uint32_t dst, int c, const ConvLane& cl) {
-    const __half2 bias = conv::bias4();
-    const uint32_t flip = conv::kFlip4;
-    uint32_t a[16], b[16];                // re and im nibbles, one per byte (conv_lane4_f8)
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        a[e] = (w[e] >> 4) & 0x0F0F0F0Fu;
-        b[e] = w[e] & 0x0F0F0F0Fu;
-    }
     const uint32_t c16 = (uint32_t)c << 4;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
@@ -435,12 +426,8 @@ __device__ __forceinline__ void convert_words4_f8(const uint32_t (&w)[16], uint3
         const uint32_t at = dst + cl.rowoff[kk];
         uint32_t r[4], m[4];
 #pragma unroll
-        for (int o = 0; o < 4; ++o) {
-            r[o] = conv::e4m3x4(pair_to_half2(a[4 * o], a[4 * o + 1], sel, flip, bias),
-                          pair_to_half2(a[4 * o + 2], a[4 * o + 3], sel, flip, bias));
-            m[o] = conv::e4m3x4(pair_to_half2(b[4 * o], b[4 * o + 1], sel, flip, bias),
-                          pair_to_half2(b[4 * o + 2], b[4 * o + 3], sel, flip, bias));
-        }
+        for (int o = 0; o < 4; ++o)
+            conv::e4m3_of_nibbles(conv::gather4(w[4 * o], w[4 * o + 1], w[4 * o + 2], w[4 * o + 3], sel), r[o], m[o]);
         st_shared_v4(at + (c16 ^ cl.r7x16[kk]), r[0], r[1], r[2], r[3]);
         st_shared_v4(at + 128u + (c16 ^ (cl.r7x16[kk] + 16u)), m[0], m[1], m[2], m[3]);   // the im row
     }
