@@ -119,10 +119,26 @@ def _ptr(x):
     return x.data_ptr()
 
 
+_raw_stream = None
+
+
+def _current_stream_handle():
+    """Handle of the current device's current stream.  torch.cuda.current_stream() builds a Stream
+    object around it, 2.9 us of a call whose launch takes 3.4; torch's raw getters take 0.2."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()   # initialises CUDA, or raises as it always did
+        get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if get is None or dev is None:
+            return torch.cuda.current_stream().cuda_stream
+        _raw_stream = lambda: get(dev())   # noqa: E731
+    return _raw_stream()
+
+
 def _stream_handle(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream_handle()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
