@@ -492,14 +492,23 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
     }
 }
 
-// rows of CTAs along the frames: one wave of resident CTAs, each with the same number of batches
+// rows of CTAs along the frames, each with the same number of batches: the number of waves whose
+// waves x (batches of a CTA + 1) is least, the 1 being what a CTA spends before its first batch.  One
+// wave alone leaves up to half the chip idle when the groups are more than half of it.
 int fw_rows(int groups, int n_batches, int slots) {
-    int rows = slots / groups;
-    if (rows < 1) rows = 1;
-    if (rows > n_batches) rows = n_batches;
-    const int per = (n_batches + rows - 1) / rows;
-    rows = (n_batches + per - 1) / per;
-    return rows > 65535 ? 65535 : rows;
+    const int w0 = (groups + slots - 1) / slots;
+    long long best_cost = 0;
+    int best = 1;
+    for (int w = w0; w < w0 + 8; ++w) {
+        long long rows = (long long)w * slots / groups;
+        if (rows > n_batches) rows = n_batches;
+        const long long per = (n_batches + rows - 1) / rows, cost = w * (per + 1);
+        if (w == w0 || cost < best_cost) {
+            best_cost = cost;
+            best = (int)((n_batches + per - 1) / per);
+        }
+    }
+    return best > 65535 ? 65535 : best;
 }
 
 template <int KIND, int LGL>
@@ -569,12 +578,15 @@ cudaError_t launch_kind(const FWideArgs& p, cudaStream_t s) {
 // 755 -> 166; their error against 64 bits is that of the full-length transform (1.0e-7 at 1024
 // points).  Shorter ones keep fengine.cu: at half length their error would be 5% larger.
 // Filterbanks of up to 8 taps where four frames of at least four inputs fit: 8 taps, c8, L = 32 ..
-// 512: 403 -> 158, 302 -> 163, 313 -> 178, 421 -> 218, 515 -> 356; r8, L = 32 .. 1024: 308 -> 88,
-// 244 -> 94, 252 -> 112, 342 -> 125, 442 -> 200, 938 -> 248 (error 1.0e-7 .. 1.2e-7, within 5%).
+// 512: 403 -> 158, 302 -> 163, 313 -> 178, 421 -> 218, 515 -> 340; r8, L = 32 .. 1024: 308 -> 88,
+// 244 -> 94, 252 -> 112, 342 -> 125, 442 -> 200, 938 -> 238 (error 1.0e-7 .. 1.2e-7, within 5%).
+// The few taps of a long complex transform stay with fengine.cu, which pays for each tap: c8 of 128
+// inputs, L = 512, 2 / 3 / 4 taps: 267 / 304 / 335 there, 313 here; c4, L = 256, 2 / 4 taps: 193 / 258
+// there, 205 / 200 here.
 bool fwide_takes(int kind, int log2L, int n_inputs, int n_taps) {
     const bool real = kind == CORR_F_REAL8;
     if (log2L < 5) return false;
-    if (n_taps > 0) return n_taps <= 8 && log2L <= (real ? 10 : 9);
+    if (n_taps > 0) return n_taps <= 8 && log2L <= (real ? 10 : 9) && (real || log2L < 8 || n_taps >= log2L - 5);
     return real ? log2L >= 8 : log2L != 6 || n_inputs % 64 != 0;
 }
 

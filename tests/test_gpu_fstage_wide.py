@@ -90,3 +90,16 @@ def test_samples_off_the_vector_alignment(kind, n_chan, n_taps):
     n, f = 16, 6
     p = _samples(3 + n_chan, (f + max(0, n_taps - 1)) * L, n, kind)
     assert np.array_equal(_run(p, n, n_chan, f, kind, n_taps, offset=2), _run(p, n, n_chan, f, kind, n_taps))
+
+
+# groups of inputs that are more than half of the chip, or more than all of it: several waves of runs
+@pytest.mark.parametrize("kind,n_chan,n_taps,n_inputs,n_frames", [
+    ("c4", 512, 4, 336, 29), ("c4", 512, 4, 1300, 9), ("r8", 512, 8, 700, 21), ("c8", 2048, 0, 680, 7)])
+def test_runs_in_several_waves(kind, n_chan, n_taps, n_inputs, n_frames):
+    L = fstage.transform_length(n_chan, kind)
+    p = _samples(n_chan + n_inputs, (n_frames + max(0, n_taps - 1)) * L, n_inputs, kind)
+    taps = np.random.default_rng(n_inputs).normal(size=n_taps * L).astype(np.float32) if n_taps else None
+    got = _run(p, n_inputs, n_chan, n_frames, kind, n_taps, taps)
+    ref = (fstage.pfb(p, n_inputs, n_chan, n_frames, kind, taps.astype(np.float64)) if n_taps else
+           fstage.fstage(p, n_inputs, n_chan, n_frames, kind))
+    _check(got, ref, (4 * math.log2(L) + 4 * n_taps) * EPS)
