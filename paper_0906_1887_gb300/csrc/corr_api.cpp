@@ -224,7 +224,9 @@ corr_status corr_xengine_run_batch(corr_plan plan, const void* d_packed, int n_d
     } else if (engine == CORR_ENGINE_BF16X3) {
         if (p->sample_bits != 32)
             return set_error(CORR_EUNSUPPORTED, "CORR_ENGINE_BF16X3 takes float samples (sample_bits=32)");
-        if (need == 0) {   // fused: TMA loads the floats, the converter warps split them
+        // fused: TMA loads the floats, the converter warps split them
+        if (need == 0 || (tc_rawf32_pairs(*p) && aligned16(d_packed) &&
+                          (int64_t)n_dumps * p->n_chan < (int64_t{1} << 31))) {
             e = launch_xeng_tc_rawf32(*p, d_packed, n_dumps, d_vis, accumulate, s);
         } else {
             char* hi = static_cast<char*>(d_workspace);

@@ -758,9 +758,14 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                         if constexpr (PAIR) {
                             const uint32_t b0 = same ? a0 : a0 + boff16;
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                ptx::mma_pair_lo<C::kF8>(dset, a0 + 2u * k, b0 + 2u * k, desc_hi, idesc_wide,
-                                                         (k > 0) | acc0);
+                            for (int k = 0; k < 4; ++k) {
+                                const uint32_t ak = a0 + 2u * k, bk = b0 + 2u * k;
+                                ptx::mma_pair_lo<C::kF8>(dset, ak, bk, desc_hi, idesc_wide, (k > 0) | acc0);
+                                if constexpr (C::kSplit) {
+                                    ptx::mma_pair_lo<false>(dset, ak, bk + 1024u, desc_hi, idesc_wide, 1u);   // h_i l_j
+                                    ptx::mma_pair_lo<false>(dset, ak + 1024u, bk, desc_hi, idesc_wide, 1u);   // l_i h_j
+                                }
+                            }
                         } else if (!C::kRaw && !C::kSplit && it.wide) {
                             // one M = 128, N = 256 MMA covers tiles (I, J) and (I, J + 1); on the
                             // diagonal A is the first half of the B box
@@ -1207,7 +1212,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 const uint32_t raw = ptx::smem_u32(rawring + rs * prm.raw_stage_bytes) + lane_byte;
                 const uint32_t dst = ptx::smem_u32(ring + os * prm.op_stage_bytes);
                 if constexpr (C::kFloat) {
-                    // single-block arrays only (one tile, B = A): slice q of the tile per warp
+                    // B = A: one block, or the diagonal square of a pair's two (the CTA's own block):
+                    // slice q of the tile per warp
                     const uint32_t raw_tile = ptx::smem_u32(rawring + rs * prm.raw_stage_bytes);
                     for (int sl = cwarp; sl < kTimeBlock / 8; sl += C::kGroupWarps)
                         convert_slice_f32(raw_tile, dst, sl, lane);
@@ -1385,8 +1391,9 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     if (map_lo) prm->map_lo = *map_lo;
     int64_t items = 0;
     int op_tiles = 1, raw_tiles = 1;
-    bool any_pair = false, pair = tune.pair != 0 && !C::kSplit && MODE != kRaw4;
-    for (int j = 0; j < n_jobs; ++j) pair = pair && specs[j].n_inputs > kBlockInputs;
+    bool any_pair = false, pair = tune.pair != 0 && MODE != kPlanesBF16x3 && MODE != kRaw4;
+    for (int j = 0; j < n_jobs; ++j)
+        pair = pair && specs[j].n_inputs > kBlockInputs && (!C::kFloat || specs[j].n_inputs <= 2 * kBlockInputs);
     for (int j = 0; j < n_jobs; ++j) {
         const TcJobSpec& sp = specs[j];
         TcJob& jb = prm->jobs[j];
@@ -1433,8 +1440,9 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
         fast_div_make((uint32_t)jb.n_tiles, jb.tiles_m, jb.tiles_s);
         fast_div_make((uint32_t)jb.n_groups, jb.groups_m, jb.groups_s);
         items += job_items;
-        // operand tiles one stage needs: A + a two-block B box for wide items
-        const int tiles = jb.tw == 2 ? 3 : (jb.nb == 1 ? jb.cpi : 2);
+        // operand tiles one stage needs: A + a two-block B box for wide items; float pairs only ever
+        // work on their diagonal square
+        const int tiles = jb.tw == 2 ? 3 : (jb.nb == 1 ? jb.cpi : C::kFloat && pair ? 1 : 2);
         op_tiles = tiles > op_tiles ? tiles : op_tiles;
         raw_tiles = tiles > raw_tiles ? tiles : raw_tiles;
         any_pair = any_pair || jb.cpi == 2 || jb.tw == 2 || pair;   // two 256-column accumulator sets
@@ -1488,7 +1496,7 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     prm->bar_offset = prm->staging_offset + stage_space;
     const int smem_bytes = prm->bar_offset + kBarBytes + 1024;
     auto kern = xeng_tc_kernel<MODE, MAXJ, false, false>;
-    if constexpr (!C::kSplit && MODE != kRaw4) {
+    if constexpr (MODE != kPlanesBF16x3 && MODE != kRaw4) {
         if (pair) kern = xeng_tc_kernel<MODE, MAXJ, false, true>;
     }
     if constexpr (C::kRaw && !C::kFloat && MAXJ == 1) {
@@ -1772,9 +1780,20 @@ bool tc_rawf32_supported(const Plan& p) {
     return p.sample_bits == 32 && p.n_inputs <= kBlockInputs && (p.n_inputs % 2) == 0;
 }
 
+// Arrays of two blocks: a CTA pair splits one block in each CTA and works on their diagonal square, whose
+// stages are no larger than a single block's.  (Larger arrays have squares off the diagonal, of twice
+// the samples and operands a stage: they take the planes.)  Measured, planes -> pairs: 128 inputs x
+// 512 channels x 64 / 128 / 256 / 512 samples 50 -> 27 / 69 -> 31 / 99 -> 38 / 173 -> 63 us (45 us for
+// the bytes of 512), 1024 channels x 1024 634 -> 227, 80 inputs x 139 x 1222 112 -> 43, 20 x 100 16 -> 9.
+bool tc_rawf32_pairs(const Plan& p) {
+    return p.sample_bits == 32 && p.nb == 2 && (p.n_inputs % 2) == 0 && !p.tc_float_planes &&
+           p.tc_op_stages != 1;   // one operand stage: the plane feed ignores it, this one could not run
+}
+
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,
                                   cudaStream_t s) {
-    if (!tc_rawf32_supported(p) || (reinterpret_cast<uintptr_t>(d_samples) & 15u)) return cudaErrorInvalidValue;
+    const bool pairs = tc_rawf32_pairs(p);
+    if ((!pairs && !tc_rawf32_supported(p)) || (reinterpret_cast<uintptr_t>(d_samples) & 15u)) return cudaErrorInvalidValue;
     if ((int64_t)n_dumps * p.n_chan >= (int64_t{1} << 31)) return cudaErrorInvalidValue;   // 32-bit item indices
     auto enc = get_encode();
     if (!enc) return cudaErrorInvalidValue;
@@ -1800,6 +1819,7 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
     sp.pack = pack;
     TcTuning tune;
     tune.op_stages = p.tc_op_stages;
+    tune.pair = pairs;
     return launch_jobs<kRawF32, 1>(&sp, 1, &m, nullptr, accumulate, p.d_status, p.n_sm, tune, s);
 }
 
