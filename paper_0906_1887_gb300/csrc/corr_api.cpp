@@ -228,6 +228,8 @@ corr_status corr_xengine_run_batch(corr_plan plan, const void* d_packed, int n_d
         if (need == 0 || (tc_rawf32_pairs(*p) && aligned16(d_packed) &&
                           (int64_t)n_dumps * p->n_chan < (int64_t{1} << 31))) {
             e = launch_xeng_tc_rawf32(*p, d_packed, n_dumps, d_vis, accumulate, s);
+        } else if (tc_rawf32_odd(*p, n_dumps)) {
+            e = launch_xeng_tc_rawf32_odd(*p, d_packed, n_dumps, d_workspace, d_vis, accumulate, s);
         } else {
             char* hi = static_cast<char*>(d_workspace);
             char* lo = hi + need / 2;

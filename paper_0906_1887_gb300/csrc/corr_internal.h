@@ -142,7 +142,10 @@ int tc_default_cpi(int n_inputs, int64_t channels, int n_sm);   // channels = du
 bool tc_rawf32_supported(const Plan& p);
 bool tc_rawf32_pairs(const Plan& p);   // float samples of two blocks that CTA pairs split in the kernel
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,
-                                  cudaStream_t s);
+                                  cudaStream_t s, int64_t pitch = 0);   // pitch: bytes of a padded row, 0: dense
+bool tc_rawf32_odd(const Plan& p, int n_dumps);
+cudaError_t launch_xeng_tc_rawf32_odd(const Plan& p, const void* d_samples, int n_dumps, void* d_ws, void* d_vis,
+                                      int accumulate, cudaStream_t s);
 // Fused dump mode: float32 [n_dumps][C][P][2] = V / n_accum * phasor_i conj(phasor_j) (phasor
 // float2 [C][N] or nullptr); every dump must fit one exact chunk.
 cudaError_t launch_xeng_tc_raw_dump(const Plan& p, const void* d_packed, int n_dumps, void* d_out, const void* phasor,

@@ -283,6 +283,8 @@ cudaError_t launch_fast(const Plan& p, const void* d_packed, int n_dumps, void* 
 // address (what lies between a row's end and the next row is never read).  A copy at the price of
 // the packed samples twice over, where planes cost their two to four times as many bytes twice
 // (75 inputs, 8-bit: 78 MB in, 83 out, against 284 MB of planes).
+// FLOAT: rows of an odd number of 8-byte samples.
+template <bool FLOAT>
 __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __restrict__ packed,
                                                      unsigned char* __restrict__ out, uint32_t rows, int row_bytes,
                                                      int pieces, uint32_t rows_per_block, int64_t last_word) {
@@ -294,7 +296,14 @@ __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __rest
 #pragma unroll 4
         for (uint32_t e = threadIdx.x; e < n; e += 256) {
             const uint32_t r = e / (uint32_t)pieces;
-            dst[e] = load_piece(packed, base + (int64_t)r * row_bytes + (e - r * pieces) * 16, last_word, 16);
+            const int64_t off = base + (int64_t)r * row_bytes + (e - r * pieces) * 16;
+            if constexpr (FLOAT) {
+                const uint2 a = *reinterpret_cast<const uint2*>(packed + off);
+                const uint2 b = (off >> 2) + 3 <= last_word ? *reinterpret_cast<const uint2*>(packed + off + 8) : uint2{};
+                dst[e] = make_uint4(a.x, a.y, b.x, b.y);
+            } else {
+                dst[e] = load_piece(packed, off, last_word, 16);
+            }
         }
     }
 }
@@ -327,19 +336,19 @@ cudaError_t launch_unpack_e4m3(const Plan& p, const void* d_packed, int n_dumps,
 }
 
 int64_t repack_pitch(const Plan& p) {
-    return ((int64_t)p.n_inputs * (p.sample_bits == 8 ? 2 : 1) + 15) / 16 * 16;
+    return ((int64_t)p.n_inputs * (p.sample_bits == 32 ? 8 : p.sample_bits == 8 ? 2 : 1) + 15) / 16 * 16;
 }
 
 cudaError_t launch_repack(const Plan& p, const void* d_packed, int n_dumps, void* d_out, cudaStream_t s) {
     const int64_t rows = (int64_t)n_dumps * p.n_time * p.n_chan;
-    const int row_bytes = p.n_inputs * (p.sample_bits == 8 ? 2 : 1);
+    const int row_bytes = p.n_inputs * (p.sample_bits == 32 ? 8 : p.sample_bits == 8 ? 2 : 1);
     if (rows >= (int64_t{1} << 31) ||
         ((reinterpret_cast<uintptr_t>(d_packed) | reinterpret_cast<uintptr_t>(d_out)) & 15u) != 0)
         return cudaErrorInvalidValue;
     const int pieces = (int)(repack_pitch(p) / 16);
     const int per = 2048 / pieces > 0 ? 2048 / pieces : 1;
     const int64_t want = (rows + per - 1) / per, cap = (int64_t)p.n_sm * 8;
-    return launch_kernel(repack_kernel, dim3((unsigned)(want < cap ? want : cap)), 256, 0, s, 1, false,
+    return launch_kernel(p.sample_bits == 32 ? repack_kernel<true> : repack_kernel<false>, dim3((unsigned)(want < cap ? want : cap)), 256, 0, s, 1, false,
                           static_cast<const unsigned char*>(d_packed), static_cast<unsigned char*>(d_out), (uint32_t)rows,
                           row_bytes, pieces, (uint32_t)per, (rows * row_bytes + 3) / 4 - 1);
 }

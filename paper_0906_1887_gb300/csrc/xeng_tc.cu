@@ -1790,18 +1790,38 @@ bool tc_rawf32_pairs(const Plan& p) {
            p.tc_op_stages != 1;   // one operand stage: the plane feed ignores it, this one could not run
 }
 
+// Odd counts of inputs, whose rows TMA cannot address: several channels of at most 32 inputs packed into
+// a tile start at 16-byte multiples again; other rows go into the workspace one sample longer.
+// Measured, planes -> this: packed channels 9 / 31 inputs x 512 channels x 1000 samples 139 -> 25 / 147 -> 33
+// us; repacked 9 / 31 x 513 x 1000 137 -> 56 / 150 -> 88, 41 x 762 x 318 x 3 dumps 211 -> 153, 75 x 139 x
+// 1222 113 -> 73, 127 x 512 x 512 181 -> 145, x 20 x 100 15 -> 13.
+bool tc_rawf32_odd(const Plan& p, int n_dumps) {
+    return p.sample_bits == 32 && p.nb <= 2 && p.n_inputs % 2 && !p.tc_float_planes && p.tc_op_stages != 1 &&
+           (int64_t)n_dumps * p.n_time * p.n_chan < (int64_t{1} << 31);
+}
+
+cudaError_t launch_xeng_tc_rawf32_odd(const Plan& p, const void* d_samples, int n_dumps, void* d_ws, void* d_vis,
+                                      int accumulate, cudaStream_t s) {
+    if (!accumulate && tc_channel_pack(p.n_inputs, 8, p.n_chan, n_dumps, p.n_sm) > 1)
+        return launch_xeng_tc_rawf32(p, d_samples, n_dumps, d_vis, accumulate, s);
+    const cudaError_t e = launch_repack(p, d_samples, n_dumps, d_ws, s);
+    if (e != cudaSuccess) return e;
+    return launch_xeng_tc_rawf32(p, d_ws, n_dumps, d_vis, accumulate, s, repack_pitch(p));
+}
+
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,
-                                  cudaStream_t s) {
-    const bool pairs = tc_rawf32_pairs(p);
-    if ((!pairs && !tc_rawf32_supported(p)) || (reinterpret_cast<uintptr_t>(d_samples) & 15u)) return cudaErrorInvalidValue;
+                                  cudaStream_t s, int64_t pitch) {
+    const int pack = accumulate || pitch ? 1 : tc_channel_pack(p.n_inputs, 8, p.n_chan, n_dumps, p.n_sm);
+    if (p.sample_bits != 32 || p.nb > 2 || (p.n_inputs % 2 && !pitch && pack < 2) ||
+        (reinterpret_cast<uintptr_t>(d_samples) & 15u))
+        return cudaErrorInvalidValue;
     if ((int64_t)n_dumps * p.n_chan >= (int64_t{1} << 31)) return cudaErrorInvalidValue;   // 32-bit item indices
     auto enc = get_encode();
     if (!enc) return cudaErrorInvalidValue;
     // [dump][time][chan][input] of 8-byte complex floats; box = 64 inputs x 1 channel x 64 samples.
     // The register epilogue that adds float sums in place takes one channel per tile.
     CUtensorMap m;
-    const int pack = accumulate ? 1 : tc_channel_pack(p.n_inputs, 8, p.n_chan, n_dumps, p.n_sm);
-    const cuuint64_t row = (cuuint64_t)p.n_inputs * 8;
+    const cuuint64_t row = pitch ? (cuuint64_t)pitch : (cuuint64_t)p.n_inputs * 8;
     cuuint64_t dims[4] = {(cuuint64_t)p.n_inputs, (cuuint64_t)p.n_chan, (cuuint64_t)p.n_time, (cuuint64_t)n_dumps};
     cuuint64_t strides[3] = {row, row * p.n_chan, row * p.n_chan * p.n_time};
     if (pack > 1) {   // whole time samples as rows, as in make_raw_map
@@ -1809,6 +1829,7 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
         dims[1] = 1;
         strides[0] = row * p.n_chan;
     }
+    // (an odd count of a padded row: what lies past it reads as zero)
     cuuint32_t box[4] = {(cuuint32_t)kBlockInputs, 1, (cuuint32_t)kTimeBlock, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     if (enc(&m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(d_samples), dims, strides, box, estr,
@@ -1819,7 +1840,7 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
     sp.pack = pack;
     TcTuning tune;
     tune.op_stages = p.tc_op_stages;
-    tune.pair = pairs;
+    tune.pair = p.nb == 2;
     return launch_jobs<kRawF32, 1>(&sp, 1, &m, nullptr, accumulate, p.d_status, p.n_sm, tune, s);
 }
 
