@@ -99,7 +99,7 @@ struct FW {
     static constexpr int PS = fw_lgr(LGH, kReal, 0);           // one pad row after every first radix of rows
     // row pitch: the filterbank's 16-byte stores of a quarter-warp (2 x 4 rows, 1 x 8 rows for
     // few inputs) then fall in distinct banks
-    static constexpr int CP = C + (MT && G == 8 ? 8 : MT && G == 4 ? 4 : 0);
+    static constexpr int CP = C + (MT && G == 8 ? 8 : MT && G == 4 ? 4 : MT && G == 2 ? 2 : 0);
     static constexpr int NOUT = kReal ? H + 1 : H;
     static constexpr int TWN = fw_tw_entries(LGH, kReal);
     static constexpr int ROWB = G * BPS;                       // packed bytes of a sample row
@@ -363,14 +363,17 @@ __global__ void __launch_bounds__(FW<KIND, LGL, 0>::T, 1024 / FW<KIND, LGL, 0>::
 }
 
 // Filterbank of at most MT taps: CTA (x, y) takes inputs n0 .. n0 + G - 1 and the frames of run y.
-// Thread: the four points i of inputs n0 + 4 gv .. + 3 (real samples: rows 2 i and 2 i + 1).
+// Thread: the four points i of inputs n0 + 4 gv .. + 3 (real samples: rows 2 i and 2 i + 1); where a CTA
+// has room for two inputs only, points i and i + T of both.
 template <int KIND, int LGL, int MT>
 __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>::T)
     fengine_pfb_kernel(const uint8_t* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tw, int N,
                        int n_frames, int run, const float* __restrict__ taps, int M, int vec) {
     using F = FW<KIND, LGL, MT>;
     constexpr int SPP = F::kReal ? 2 : 1;                    // samples per point
-    constexpr int VB = 4 * F::BPS;                           // bytes of four inputs of a sample
+    constexpr int QV = F::G < 4 ? F::G : 4, NI = 4 / QV;                   // inputs and points of each of a thread
+    constexpr int NR = NI * SPP;                             // its sample rows
+    constexpr int VB = QV * F::BPS;                          // bytes of QV inputs of a sample
     extern __shared__ __align__(16) uint8_t fw_smem[];
     float2* const buf = reinterpret_cast<float2*>(fw_smem);
     float2* const tws = buf + F::DATA;
@@ -379,23 +382,25 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
     const int g_n = min(F::G, N - n0);
     const int f0 = blockIdx.y * run, f1 = min(n_frames, f0 + run);
     const int n_in = n_frames + M - 1;                       // input frames
-    const int gv = threadIdx.x % (F::G / 4), i = threadIdx.x / (F::G / 4);
+    const int gv = threadIdx.x % (F::G / QV), i = threadIdx.x / (F::G / QV);
     const size_t frame_bytes = (size_t)F::L * N * F::BPS;
-    const uint8_t* const src = in + ((size_t)SPP * i * N + n0 + 4 * gv) * F::BPS;
-    const int g_left = g_n - 4 * gv;                         // inputs of the thread's four that exist
+    const uint8_t* const src = in + ((size_t)SPP * i * N + n0 + QV * gv) * F::BPS;
+    const int g_left = g_n - QV * gv;                        // inputs of the thread's that exist
     using Raw = std::conditional_t<VB == 8, uint2, uint32_t>;
-    auto load = [&](int t, Raw (&w)[SPP]) {                  // input frame t: its packed samples, or zeros
+    using Load = std::conditional_t<VB == 2, unsigned short, Raw>;
+    auto row = [](int s) { return s / SPP * F::T * SPP + s % SPP; };   // sample row s of the thread, from its first
+    auto load = [&](int t, Raw (&w)[NR]) {                   // input frame t: its packed samples, or zeros
 #pragma unroll
-        for (int s = 0; s < SPP; ++s) {
+        for (int s = 0; s < NR; ++s) {
             w[s] = Raw{};
             if (t >= n_in || g_left <= 0) continue;
-            const uint8_t* p = src + (size_t)t * frame_bytes + (size_t)s * N * F::BPS;
+            const uint8_t* p = src + (size_t)t * frame_bytes + (size_t)row(s) * N * F::BPS;
             if (vec) {
-                w[s] = *reinterpret_cast<const Raw*>(p);
+                w[s] = *reinterpret_cast<const Load*>(p);
             } else {
                 uint32_t u[2] = {0u, 0u};
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
+                for (int k = 0; k < QV; ++k)
                     if (k < g_left) {
                         const uint32_t x = F::BPS == 2 ? (uint32_t)*reinterpret_cast<const unsigned short*>(p + 2 * k)
                                                        : (uint32_t)p[k];
@@ -406,44 +411,48 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
             }
         }
     };
-    auto point = [&](const Raw (&w)[SPP], int k) -> float2 {   // point of input k of the four
+    auto point = [&](const Raw (&w)[NR], int q) -> float2 {   // point q: input q % QV, row q / QV
+        const int k = q % QV, s = q / QV * SPP;
         if constexpr (KIND == CORR_F_COMPLEX8) {
-            const uint32_t u = (k < 2 ? w[0].x : w[0].y) ^ 0x80808080u;
+            uint32_t u;
+            if constexpr (VB == 8) u = (k < 2 ? w[s].x : w[s].y) ^ 0x80808080u;
+            else u = w[s] ^ 0x80808080u;
             const uint32_t b0 = 2u * (k & 1);
             return make_float2(f_byte(u, 0x7540u | b0, kBias8), f_byte(u, 0x7541u + b0, kBias8));
         } else if constexpr (KIND == CORR_F_COMPLEX4) {
-            const uint32_t u = w[0] ^ 0x88888888u;
+            const uint32_t u = w[s] ^ 0x88888888u;
             return make_float2(f_byte((u >> 4) & 0x0F0F0F0Fu, 0x7540u | (uint32_t)k, kBias4),
                                f_byte(u & 0x0F0F0F0Fu, 0x7540u | (uint32_t)k, kBias4));
         } else {
-            return make_float2(f_byte(w[0] ^ 0x80808080u, 0x7540u | (uint32_t)k, kBias8),
-                               f_byte(w[1] ^ 0x80808080u, 0x7540u | (uint32_t)k, kBias8));
+            return make_float2(f_byte(w[s] ^ 0x80808080u, 0x7540u | (uint32_t)k, kBias8),
+                               f_byte(w[s + 1] ^ 0x80808080u, 0x7540u | (uint32_t)k, kBias8));
         }
     };
-    float h[MT][SPP];
+    float h[MT][NR];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
-        for (int s = 0; s < SPP; ++s) h[m][s] = m < M ? taps[m * F::L + SPP * i + s] : 0.f;
+        for (int s = 0; s < NR; ++s) h[m][s] = m < M ? taps[m * F::L + SPP * i + row(s)] : 0.f;
     float2 a[MT - 1][4];   // a[k]: partial sum of the output frame that k + 1 more samples complete
 #pragma unroll
     for (int k = 0; k < MT - 1; ++k)
 #pragma unroll
         for (int q = 0; q < 4; ++q) a[k][q] = make_float2(0.f, 0.f);
     // taps past M are zero, so frame f completes with input frame f + MT - 1 (zeros past the last)
-    auto step = [&](const Raw (&w)[SPP], float2 (&y)[4]) {
+    auto step = [&](const Raw (&w)[NR], float2 (&y)[4]) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float2 x = point(w, q);
-            y[q] = make_float2(fmaf(h[MT - 1][0], x.x, a[0][q].x), fmaf(h[MT - 1][SPP - 1], x.y, a[0][q].y));
+            const int s0 = q / QV * SPP, s1 = s0 + SPP - 1;
+            y[q] = make_float2(fmaf(h[MT - 1][s0], x.x, a[0][q].x), fmaf(h[MT - 1][s1], x.y, a[0][q].y));
 #pragma unroll
             for (int k = 0; k < MT - 2; ++k)
-                a[k][q] = make_float2(fmaf(h[MT - 2 - k][0], x.x, a[k + 1][q].x),
-                                      fmaf(h[MT - 2 - k][SPP - 1], x.y, a[k + 1][q].y));
-            a[MT - 2][q] = make_float2(h[0][0] * x.x, h[0][SPP - 1] * x.y);
+                a[k][q] = make_float2(fmaf(h[MT - 2 - k][s0], x.x, a[k + 1][q].x),
+                                      fmaf(h[MT - 2 - k][s1], x.y, a[k + 1][q].y));
+            a[MT - 2][q] = make_float2(h[0][s0] * x.x, h[0][s1] * x.y);
         }
     };
-    Raw w[4][SPP];
+    Raw w[4][NR];
     grid_release();
     if (f0 < f1) {
         for (int t = f0; t < f0 + MT - 1; ++t) {   // the run's first sums
@@ -454,7 +463,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
     }
     const int c = threadIdx.x & (F::C - 1), cg = c % F::G, cf = c / F::G;
     const bool second = (threadIdx.x >> 2) & 1;   // which half of the four goes first (distinct banks)
-    float2* const wr = buf + F::pad(i) * F::CP + 4 * gv;
+    float2* const wr = buf + F::pad(i) * F::CP + QV * gv;
 #pragma unroll
     for (int fb = 0; fb < 4; ++fb) load(f0 + MT - 1 + fb, w[fb]);
     for (int f = f0; f < f1; f += 4) {
@@ -466,8 +475,13 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
             const float4 lo = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
             const float4 hi = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
             float4* const d = reinterpret_cast<float4*>(wr + fb * F::G);
-            d[second ? 1 : 0] = second ? hi : lo;
-            d[second ? 0 : 1] = second ? lo : hi;
+            if constexpr (QV == 4) {
+                d[second ? 1 : 0] = second ? hi : lo;
+                d[second ? 0 : 1] = second ? lo : hi;
+            } else {
+                d[0] = lo;
+                d[F::pad(F::T) * F::CP / 2] = hi;   // point i + T (pad(i + T) = pad(i) + pad(T))
+            }
         }
 #pragma unroll
         for (int fb = 0; fb < 4; ++fb) load(f + 4 + MT - 1 + fb, w[fb]);
@@ -536,7 +550,8 @@ cudaError_t launch_pfb(const FWideArgs& p, cudaStream_t s) {
     const int batches = (p.n_frames + 3) / 4;
     const int rows = fw_rows(groups, batches, p.n_sm * (512 / F::T));
     const int run = (batches + rows - 1) / rows * 4;
-    const int vec = (size_t)p.n_inputs % 4 == 0 && reinterpret_cast<uintptr_t>(p.d_in) % (4 * F::BPS) == 0;
+    constexpr int kVec = F::G < 4 ? F::G : 4;
+    const int vec = (size_t)p.n_inputs % kVec == 0 && reinterpret_cast<uintptr_t>(p.d_in) % (kVec * F::BPS) == 0;
     return launch_kernel(kern, dim3(groups, rows), F::T, F::SMEM, s, 1, false, static_cast<const uint8_t*>(p.d_in),
                           static_cast<float2*>(p.d_out), static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames, run,
                           p.d_taps, p.n_taps, vec);
@@ -544,7 +559,7 @@ cudaError_t launch_pfb(const FWideArgs& p, cudaStream_t s) {
 
 template <int KIND, int LGL>
 cudaError_t launch_len(const FWideArgs& p, cudaStream_t s) {
-    if constexpr (LGL <= (KIND == CORR_F_REAL8 ? 10 : 9)) {
+    if constexpr (LGL <= (KIND == CORR_F_REAL8 ? 11 : 10)) {
         if (p.d_taps) return p.n_taps <= 4 ? launch_pfb<KIND, LGL, 4>(p, s) : launch_pfb<KIND, LGL, 8>(p, s);
     }
     if constexpr (KIND != CORR_F_REAL8 || LGL >= 8) {
@@ -577,16 +592,18 @@ cudaError_t launch_kind(const FWideArgs& p, cudaStream_t s) {
 // Plain real transforms of 256 points and more: 112 -> 87, 194 -> 94, 226 -> 108, 339 -> 119,
 // 755 -> 166; their error against 64 bits is that of the full-length transform (1.0e-7 at 1024
 // points).  Shorter ones keep fengine.cu: at half length their error would be 5% larger.
-// Filterbanks of up to 8 taps where four frames of at least four inputs fit: 8 taps, c8, L = 32 ..
-// 512: 403 -> 158, 302 -> 163, 313 -> 178, 421 -> 218, 515 -> 340; r8, L = 32 .. 1024: 308 -> 88,
-// 244 -> 94, 252 -> 112, 342 -> 125, 442 -> 200, 938 -> 238 (error 1.0e-7 .. 1.2e-7, within 5%).
+// Filterbanks of up to 8 taps where four frames of at least two inputs fit: 8 taps, c8, L = 32 ..
+// 512: 403 -> 158, 302 -> 163, 313 -> 178, 421 -> 212, 515 -> 331; r8, L = 32 .. 1024: 308 -> 88,
+// 244 -> 94, 252 -> 112, 342 -> 127, 442 -> 169, 938 -> 242 (error 1.0e-7 .. 1.2e-7, within 5%).  With
+// two inputs, 8 taps, 128 / 336 inputs: c8, L = 1024: 1025 -> 577 / 1411 -> 582; r8, L = 2048: 1590 ->
+// 434, 481 inputs 1659 -> 585, 4 taps 908 -> 373 / 882 -> 364 (error 1.28e-7, 1.25e-7 before).
 // The few taps of a long complex transform stay with fengine.cu, which pays for each tap: c8 of 128
 // inputs, L = 512, 2 / 3 / 4 taps: 267 / 304 / 335 there, 313 here; c4, L = 256, 2 / 4 taps: 193 / 258
-// there, 205 / 200 here.
+// there, 205 / 200 here; L = 1024, 4 / 6 taps: 476 / 823 there, 544 / 577 here.
 bool fwide_takes(int kind, int log2L, int n_inputs, int n_taps) {
     const bool real = kind == CORR_F_REAL8;
     if (log2L < 5) return false;
-    if (n_taps > 0) return n_taps <= 8 && log2L <= (real ? 10 : 9) && (real || log2L < 8 || n_taps >= log2L - 5);
+    if (n_taps > 0) return n_taps <= 8 && log2L <= (real ? 11 : 10) && (real || log2L < 8 || n_taps >= log2L - 5);
     return real ? log2L >= 8 : log2L != 6 || n_inputs % 64 != 0;
 }
 

@@ -103,3 +103,16 @@ def test_runs_in_several_waves(kind, n_chan, n_taps, n_inputs, n_frames):
     ref = (fstage.pfb(p, n_inputs, n_chan, n_frames, kind, taps.astype(np.float64)) if n_taps else
            fstage.fstage(p, n_inputs, n_chan, n_frames, kind))
     _check(got, ref, (4 * math.log2(L) + 4 * n_taps) * EPS)
+
+
+# CTAs with room for two inputs: a thread takes two points of each
+@pytest.mark.parametrize("n_inputs,n_frames", [(1, 5), (3, 9), (34, 18)])
+@pytest.mark.parametrize("n_taps", [2, 4, 5, 8])
+@pytest.mark.parametrize("kind,n_chan", [("c8", 1024), ("c4", 1024), ("r8", 1024)])
+def test_long_filterbank(kind, n_chan, n_taps, n_inputs, n_frames):
+    L = fstage.transform_length(n_chan, kind)
+    p = _samples(5 * n_chan + n_inputs, (n_frames + n_taps - 1) * L, n_inputs, kind)
+    taps = np.random.default_rng(n_chan + n_taps).normal(size=n_taps * L).astype(np.float32)
+    got = _run(p, n_inputs, n_chan, n_frames, kind, n_taps, taps)
+    ref = fstage.pfb(p, n_inputs, n_chan, n_frames, kind, taps.astype(np.float64))
+    _check(got, ref, (4 * math.log2(L) + 4 * n_taps) * EPS)
