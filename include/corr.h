@@ -133,10 +133,13 @@ corr_status corr_plan_set_tuning(corr_plan plan, int op_stages, int float_planes
  * kernel wrote into the workspace first (each block converted once; the planes cost HBM
  * traffic; fp16 planes, or e4m3 ones for 4-bit samples of rows that are 16-byte multiples --
  * the workspace's own format, not the fp16 exchange format of corr_unpack).  operands:
- *   CORR_OPERANDS_AUTO    planes for arrays of at least 256 inputs (4 blocks; 192 inputs, 3
- *                         blocks, for 4-bit samples, whose planes are e4m3) when a workspace
- *                         is given, and always where the packed rows are not 16-byte multiples;
- *                         otherwise the fused conversion, into e4m3 operands for 4-bit samples;
+ *   CORR_OPERANDS_AUTO    arrays of at least 256 inputs (4 blocks; 192 inputs, 3 blocks, for
+ *                         4-bit samples) when a workspace is given, and rows that are not 16-byte
+ *                         multiples: planes, or the fused conversion where pairs of CTAs convert
+ *                         faster than planes are read (shorter and accumulating dumps) and, for
+ *                         smaller arrays of unaligned rows, where the rows are copied to 16-byte
+ *                         multiples in the workspace; otherwise the fused conversion, into e4m3
+ *                         operands for 4-bit samples;
  *   CORR_OPERANDS_PACKED  always the fused conversion into fp16 operands (CORR_EUNSUPPORTED
  *                         where rows are not 16-byte multiples);
  *   CORR_OPERANDS_PLANES  always planes (the workspace is then required);
@@ -148,9 +151,9 @@ corr_status corr_plan_set_tuning(corr_plan plan, int op_stages, int float_planes
  *                         multiples).
  * items (plane feed): CORR_ITEMS_WIDE = work items of block I against blocks J and J + 1 in one
  * M = 128, N = 256 MMA (a quarter fewer operand loads per tile); CORR_ITEMS_TILES = one 64 x 64
- * input tile per item; CORR_ITEMS_AUTO = wide, except single tiles for accumulating dumps of
- * fewer than 1024 samples (bound by their read-modify-write of the output).  CORR_EINVAL on
- * unknown values.
+ * input tile per item; CORR_ITEMS_AUTO = pairs of CTAs on 2 x 2 squares of tiles for most arrays
+ * (both feeds), else wide items, except single tiles for accumulating dumps of fewer than 1024
+ * samples (bound by their read-modify-write of the output).  CORR_EINVAL on unknown values.
  */
 enum { CORR_OPERANDS_AUTO = 0, CORR_OPERANDS_PACKED = 1, CORR_OPERANDS_PLANES = 2, CORR_OPERANDS_PACKED_F8 = 3 };
 enum { CORR_ITEMS_AUTO = 0, CORR_ITEMS_TILES = 1, CORR_ITEMS_WIDE = 2 };
@@ -159,7 +162,7 @@ corr_status corr_plan_set_operands(corr_plan plan, int operands, int items);
 /* Device workspace (bytes) corr_xengine_run_batch uses for `engine` and n_dumps dumps.  0 means
  * the engine needs none (d_workspace may be NULL).  For CORR_ENGINE_TC on arrays whose packed
  * rows are 16-byte multiples the workspace is optional unless CORR_OPERANDS_PLANES is set: a
- * NULL workspace runs the fused conversion, a workspace of this size the plane feed. */
+ * NULL workspace runs the fused conversion, a workspace of this size the feed chosen above. */
 corr_status corr_workspace_size(corr_plan plan, int engine, int n_dumps, size_t *bytes);
 
 /*
