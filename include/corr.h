@@ -118,8 +118,8 @@ corr_status corr_plan_info(corr_plan plan, int64_t *n_baselines, size_t *packed_
  * sample ring is reduced to what fits; the plane feed uses the requested depth when it is
  * smaller than what fits (by default as deep as fits).  float_planes (CORR_ENGINE_BF16X3 on float samples): 0 = the
  * default, the tensor-core kernel loads the floats and splits them into bf16 hi + lo itself
- * where it can (an even count of inputs: at most 64, needing no workspace, or up to 128, whose
- * workspace stays unused); 1 = always split into hi/lo planes in the workspace first.  Results are
+ * where it can (an even count of inputs, at most 64, needs no workspace; larger arrays leave theirs
+ * unused, odd counts copy their rows into it); 1 = always split into hi/lo planes in the workspace first.  Results are
  * identical for every setting.
  * CORR_EINVAL when op_stages is outside [0, 16] or float_planes outside [0, 1].
  */

@@ -140,7 +140,7 @@ int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm
 int tc_default_cpi(int n_inputs, int64_t channels, int n_sm);   // channels = dumps x n_chan of the launch
 // BF16x3 on float samples with the hi/lo split done in the tensor-core kernel (single-block arrays)
 bool tc_rawf32_supported(const Plan& p);
-bool tc_rawf32_pairs(const Plan& p);   // float samples of two blocks that CTA pairs split in the kernel
+bool tc_rawf32_pairs(const Plan& p);   // float samples of several blocks that CTA pairs split in the kernel
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,
                                   cudaStream_t s, int64_t pitch = 0);   // pitch: bytes of a padded row, 0: dense
 bool tc_rawf32_odd(const Plan& p, int n_dumps);

@@ -515,7 +515,9 @@ __device__ __forceinline__ void mma_op(uint32_t d, uint32_t a_lo, uint32_t b_lo,
 // its two tiles -- one, on the diagonal -- where single tiles take two per tile, and its shared
 // memory feeds 8 KB instead of 16 KB of operands per tile and K step.  The even CTA's MMA thread
 // issues for both; converters and epilogue warps of the odd CTA arrive on its barriers, and its
-// commits arrive in both.  On planes the odd CTA's MMA thread relays "stage loaded".
+// commits arrive in both.  On planes the odd CTA's MMA thread relays "stage loaded".  Float
+// pairs have 64 KB of operands (two blocks, hi and lo) in a stage off the diagonal: two such stages
+// and two raw slots of one 32 KB tile each fit, and the converter groups take a tile each.
 template <int MODE, int MAXJ, bool DUMP, bool PAIR>
 __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const __grid_constant__ TcLaunch<MAXJ> prm) {
     using C = Cfg<MODE>;
@@ -547,7 +549,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < OS; ++s) {
-            ptx::mbar_init(bar_op_full + 8 * s, C::kRaw ? C::kGroupWarps * kCtas : 1);
+            ptx::mbar_init(bar_op_full + 8 * s, C::kRaw ? C::kGroupWarps * kCtas * (C::kFloat && PAIR ? 2 : 1) : 1);
             ptx::mbar_init(bar_op_empty + 8 * s, 1);
             ptx::mbar_init(bar_peer_full + 8 * s, 1);
         }
@@ -608,14 +610,17 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 const int I = it.I, J = it.J;
                 const bool same = it.same;
                 const int nkb = jb.kp / C::kStageT;
-                for (int kb = 0; kb < nkb; ++kb) {
+                // float pairs: the two blocks of a square off the diagonal take a raw slot each
+                const int units = C::kFloat && PAIR && !same ? 2 : 1;
+                for (int ku = 0; ku < nkb * units; ++ku) {
+                    const int kb = units == 2 ? ku >> 1 : ku;
                     if (!ptx::mbar_wait_bounded(bar_empty + 8 * s, ph ^ 1u, abort_flag, prm.wait_limit_ns)) {
                         record_error(prm.status, abort_flag, kDevTimeoutEmpty, kb);
                         ok = false;
                         break;
                     }
                     const uint32_t fb = bar_full + 8 * s;
-                    if (item == prm.stall_item && kb == 0) {
+                    if (item == prm.stall_item && ku == 0) {
                         // self-test of the bounded waits: nothing will complete this stage
                         withheld = n_slots++;
                         if (++s == S) {
@@ -626,6 +631,11 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     }
                     if constexpr (C::kRaw) {
                         const uint32_t st = ptx::smem_u32(rawring + s * prm.raw_stage_bytes);
+                        if constexpr (C::kFloat && PAIR) {
+                            const int block = units == 2 && (ku & 1) ? J + rank : I;
+                            ptx::mbar_expect_tx(fb, (uint32_t)C::kRawTileBytes);
+                            tma_load_4d(st, &jb.map, block * C::kMapX, it.c0, kb * C::kStageT, (int)it.d, fb);
+                        } else {
                         // one box covers cpi adjacent channels (cpi x 64 inputs per sample row)
                         ptx::mbar_expect_tx(fb, (same ? (uint32_t)jb.cpi : 2u) * (uint32_t)C::kRawTileBytes);
                         tma_load_4d(st, &jb.map, I * C::kMapX + it.c0 * jb.x_step, it.c0 * jb.y_step,
@@ -633,6 +643,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                         if (!same)
                             tma_load_4d(st + C::kRawTileBytes, &jb.map, (J + rank) * C::kMapX, it.c0, kb * C::kStageT,
                                         (int)it.d, fb);
+                        }
                     } else {
                         const uint32_t st = ptx::smem_u32(ring + s * prm.op_stage_bytes);
                         const int64_t dc = it.d * jb.n_chan + it.c0;   // planes: one channel per item
@@ -1197,7 +1208,9 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             constexpr int kSlices = C::kBits8 ? 8 : 4;
             const int n_tl = same ? cpi : 2;
             const bool pair_pitch = same && cpi == 2;
-            for (int kb = 0; kb < nkb; ++kb) {
+            const int units = C::kFloat && PAIR && !same ? 2 : 1;
+            for (int ku = 0; ku < nkb * units; ++ku) {
+                const int kb = units == 2 ? ku >> 1 : ku;
                 const bool mine = turn == group;
                 if (++turn == C::kConvGroups) turn = 0;
                 if (mine) {
@@ -1212,11 +1225,11 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 const uint32_t raw = ptx::smem_u32(rawring + rs * prm.raw_stage_bytes) + lane_byte;
                 const uint32_t dst = ptx::smem_u32(ring + os * prm.op_stage_bytes);
                 if constexpr (C::kFloat) {
-                    // B = A: one block, or the diagonal square of a pair's two (the CTA's own block):
-                    // slice q of the tile per warp
+                    // one tile a visit (B = A, or a square off the diagonal, whose two tiles go to the
+                    // two groups): slice q of the tile per warp
                     const uint32_t raw_tile = ptx::smem_u32(rawring + rs * prm.raw_stage_bytes);
                     for (int sl = cwarp; sl < kTimeBlock / 8; sl += C::kGroupWarps)
-                        convert_slice_f32(raw_tile, dst, sl, lane);
+                        convert_slice_f32(raw_tile, units == 2 && (ku & 1) ? dst + prm.b_offset : dst, sl, lane);
                 } else if constexpr (C::kF8) {
                     // e4m3 operands, a slice per warp: 32 samples of one tile, lanes 0..15 chunk
                     // c = 2 part (samples 16c .. 16c + 15) and 16..31 chunk c + 1.  (The fp16
@@ -1271,8 +1284,13 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                 fence_async_shared();   // generic-proxy writes -> visible to the tensor core
                 __syncwarp();
                 if (lane == 0) {
-                    if constexpr (PAIR) ptx::mbar_arrive_cluster(ptx::map_shared(bar_op_full + 8 * os, 0));
-                    else ptx::mbar_arrive(bar_op_full + 8 * os);
+                    if constexpr (PAIR) {
+                        const uint32_t full = ptx::map_shared(bar_op_full + 8 * os, 0);
+                        ptx::mbar_arrive_cluster(full);
+                        if (C::kFloat && units == 1) ptx::mbar_arrive_cluster(full);   // for the tile it has not
+                    } else {
+                        ptx::mbar_arrive(bar_op_full + 8 * os);
+                    }
                     ptx::mbar_arrive(bar_raw_empty + 8 * rs);
                 }
                 }   // the group's stage
@@ -1280,6 +1298,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     rs = 0;
                     rph ^= 1u;
                 }
+                if (units == 2 && !(ku & 1)) continue;   // the stage's second tile follows
                 if (++os == OS) {
                     os = 0;
                     oph ^= 1u;
@@ -1393,7 +1412,7 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     int op_tiles = 1, raw_tiles = 1;
     bool any_pair = false, pair = tune.pair != 0 && MODE != kPlanesBF16x3 && MODE != kRaw4;
     for (int j = 0; j < n_jobs; ++j)
-        pair = pair && specs[j].n_inputs > kBlockInputs && (!C::kFloat || specs[j].n_inputs <= 2 * kBlockInputs);
+        pair = pair && specs[j].n_inputs > kBlockInputs;
     for (int j = 0; j < n_jobs; ++j) {
         const TcJobSpec& sp = specs[j];
         TcJob& jb = prm->jobs[j];
@@ -1440,11 +1459,11 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
         fast_div_make((uint32_t)jb.n_tiles, jb.tiles_m, jb.tiles_s);
         fast_div_make((uint32_t)jb.n_groups, jb.groups_m, jb.groups_s);
         items += job_items;
-        // operand tiles one stage needs: A + a two-block B box for wide items; float pairs only ever
-        // work on their diagonal square
-        const int tiles = jb.tw == 2 ? 3 : (jb.nb == 1 ? jb.cpi : C::kFloat && pair ? 1 : 2);
+        // operand tiles one stage needs: A + a two-block B box for wide items; float pairs of two
+        // blocks have their diagonal square only, and float pairs' raw slots hold one tile
+        const int tiles = jb.tw == 2 ? 3 : (jb.nb == 1 ? jb.cpi : C::kFloat && pair && jb.nb == 2 ? 1 : 2);
         op_tiles = tiles > op_tiles ? tiles : op_tiles;
-        raw_tiles = tiles > raw_tiles ? tiles : raw_tiles;
+        raw_tiles = C::kFloat && pair ? 1 : tiles > raw_tiles ? tiles : raw_tiles;
         any_pair = any_pair || jb.cpi == 2 || jb.tw == 2 || pair;   // two 256-column accumulator sets
     }
     prm->n_items = items;
@@ -1472,8 +1491,10 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
         int raw_space = kSmemBudget - stage_space - prm->op_stages * prm->op_stage_bytes;
         prm->raw_stages = raw_space / prm->raw_stage_bytes;
         if (prm->raw_stages > kMaxRawStages) prm->raw_stages = kMaxRawStages;
-        // two converter groups on a shallower raw ring need an even one (see the converters' waits)
-        if (C::kConvGroups == 2 && prm->raw_stages < prm->op_stages) prm->raw_stages &= ~1;
+        // two converter groups on a shallower raw ring, or one whose slots are parts of stages, need an
+        // even one (see the converters' waits)
+        if (C::kConvGroups == 2 && (prm->raw_stages < prm->op_stages || (C::kFloat && pair && op_tiles == 2)))
+            prm->raw_stages &= ~1;
         if (prm->raw_stages < 2) {
             delete prm;
             return cudaErrorInvalidValue;
@@ -1780,13 +1801,16 @@ bool tc_rawf32_supported(const Plan& p) {
     return p.sample_bits == 32 && p.n_inputs <= kBlockInputs && (p.n_inputs % 2) == 0;
 }
 
-// Arrays of two blocks: a CTA pair splits one block in each CTA and works on their diagonal square, whose
-// stages are no larger than a single block's.  (Larger arrays have squares off the diagonal, of twice
-// the samples and operands a stage: they take the planes.)  Measured, planes -> pairs: 128 inputs x
-// 512 channels x 64 / 128 / 256 / 512 samples 50 -> 27 / 69 -> 31 / 99 -> 38 / 173 -> 63 us (45 us for
-// the bytes of 512), 1024 channels x 1024 634 -> 227, 80 inputs x 139 x 1222 112 -> 43, 20 x 100 16 -> 9.
+// Arrays of several blocks: the CTAs of a pair split the blocks of a square themselves, where the plane
+// feed writes hi and lo planes (half of its time) and reads them back.  Measured, planes -> pairs: 128
+// inputs x 512 channels x 64 / 128 / 256 / 512 samples 50 -> 27 / 69 -> 31 / 99 -> 38 / 173 -> 63 us (45
+// us for the bytes of 512), 1024 channels x 1024 634 -> 227, 80 inputs x 139 x 1222 112 -> 43, 20 x 100
+// 16 -> 9; squares off the diagonal too: 256 x 512 x 128 / 512 162 -> 81 / 402 -> 201, 256 x 76 x 4096
+// 433 -> 238, 192 x 202 x 506 116 -> 78, 130 x 139 x 1222 180 -> 136, 512 x 128 x 512 283 -> 178, 1024 x 64
+// x 256 / 1024 281 -> 180 / 780 -> 602.  Odd block counts above one compute half-empty squares and gain
+// nothing on long dumps (320 x 200 x 500 220 -> 167, but 320 x 30 x 2000 126 -> 127).
 bool tc_rawf32_pairs(const Plan& p) {
-    return p.sample_bits == 32 && p.nb == 2 && (p.n_inputs % 2) == 0 && !p.tc_float_planes &&
+    return p.sample_bits == 32 && p.nb >= 2 && (p.nb % 2 == 0 || p.kp <= 1536) && (p.n_inputs % 2) == 0 && !p.tc_float_planes &&
            p.tc_op_stages != 1;   // one operand stage: the plane feed ignores it, this one could not run
 }
 
@@ -1794,9 +1818,11 @@ bool tc_rawf32_pairs(const Plan& p) {
 // a tile start at 16-byte multiples again; other rows go into the workspace one sample longer.
 // Measured, planes -> this: packed channels 9 / 31 inputs x 512 channels x 1000 samples 139 -> 25 / 147 -> 33
 // us; repacked 9 / 31 x 513 x 1000 137 -> 56 / 150 -> 88, 41 x 762 x 318 x 3 dumps 211 -> 153, 75 x 139 x
-// 1222 113 -> 73, 127 x 512 x 512 181 -> 145, x 20 x 100 15 -> 13.
+// 1222 113 -> 73, 127 x 512 x 512 181 -> 145, x 20 x 100 15 -> 13, 255 x 202 x 506 177 -> 149, 1023 x 64 x
+// 256 289 -> 227; odd block counts, whose squares are half empty, stay with the planes (141 x 179 x 833 172
+// there, 182 here).
 bool tc_rawf32_odd(const Plan& p, int n_dumps) {
-    return p.sample_bits == 32 && p.nb <= 2 && p.n_inputs % 2 && !p.tc_float_planes && p.tc_op_stages != 1 &&
+    return p.sample_bits == 32 && p.n_inputs % 2 && (p.nb == 1 || p.nb % 2 == 0) && !p.tc_float_planes && p.tc_op_stages != 1 &&
            (int64_t)n_dumps * p.n_time * p.n_chan < (int64_t{1} << 31);
 }
 
@@ -1812,7 +1838,7 @@ cudaError_t launch_xeng_tc_rawf32_odd(const Plan& p, const void* d_samples, int 
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,
                                   cudaStream_t s, int64_t pitch) {
     const int pack = accumulate || pitch ? 1 : tc_channel_pack(p.n_inputs, 8, p.n_chan, n_dumps, p.n_sm);
-    if (p.sample_bits != 32 || p.nb > 2 || (p.n_inputs % 2 && !pitch && pack < 2) ||
+    if (p.sample_bits != 32 || (p.n_inputs % 2 && !pitch && pack < 2) ||
         (reinterpret_cast<uintptr_t>(d_samples) & 15u))
         return cudaErrorInvalidValue;
     if ((int64_t)n_dumps * p.n_chan >= (int64_t{1} << 31)) return cudaErrorInvalidValue;   // 32-bit item indices
@@ -1840,7 +1866,7 @@ cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_du
     sp.pack = pack;
     TcTuning tune;
     tune.op_stages = p.tc_op_stages;
-    tune.pair = p.nb == 2;
+    tune.pair = p.nb >= 2;
     return launch_jobs<kRawF32, 1>(&sp, 1, &m, nullptr, accumulate, p.d_status, p.n_sm, tune, s);
 }
 

@@ -53,3 +53,18 @@ def test_odd_float_rows_match_planes(n, c, t, n_dumps, accumulate):
     chans = sorted({0, c // 2, c - 1})
     for d in range(n_dumps):
         check_bf16x3(v[d][chans], x[d], n, c, t, chans)
+
+
+# more than two blocks: squares off the diagonal, whose stages are two tiles; even and odd block counts
+@pytest.mark.parametrize("accumulate", [False, True])
+@pytest.mark.parametrize("n,c,t,n_dumps,op_stages", [
+    (130, 1, 1, 1, 0), (192, 3, 65, 2, 2), (140, 90, 130, 1, 0), (254, 2, 400, 1, 16), (256, 80, 64, 1, 0),
+    (129, 3, 100, 1, 0), (300, 2, 200, 2, 0), (513, 1, 130, 1, 0), (640, 2, 65, 1, 3)])
+def test_float_squares_off_the_diagonal_match_planes(n, c, t, n_dumps, op_stages, accumulate):
+    rng = np.random.default_rng(n + c + t)
+    x = rng.normal(size=(n_dumps, t, c, n, 2)).astype(np.float32)
+    init = np.zeros((n_dumps, c, n * (n + 1) // 2, 2), np.float32) if accumulate else None
+    v = run_engine(x, n, c, t, 32, BF16X3, n_dumps=n_dumps, accumulate=accumulate, vis_init=init, tuning=(op_stages, 0))
+    planes = run_engine(x, n, c, t, 32, BF16X3, n_dumps=n_dumps, tuning=(0, 1))
+    assert np.array_equal(v, planes)
+    check_bf16x3(v[0][:1], x[0], n, c, t, [0])
