@@ -432,7 +432,7 @@ def run_large(args):
                           "separate_x_plus_dump_ms": ms_one + ms_dump, "dump_step_ms": ms_dump,
                           "output": "float32 V / n_accum, phase-corrected (8 B per baseline)",
                           "achieved_gbs": (per_dump + P * c * 8) / (ms_fused / 1e3) / 1e9},
-           "roofline": {"bound": "hbm", "kernel": "unpack_fast_kernel<8> + xeng_tc_kernel<planes, wide items>",
+           "roofline": {"bound": "hbm", "kernel": "xeng_tc_kernel<raw8, CTA pairs>",
                         "achieved": gbs, "peak": hbm,
                         "unit": "GB/s", "frac": gbs / hbm, "algorithmic_bytes_per_launch": bytes_launch,
                         "kernel_ms": ms_one, "tensor_tflops_algorithmic": 8.0 * P * c * t / (ms_one / 1e3) / 1e12,
@@ -611,12 +611,12 @@ def run_fx(args):
            # Table 4's actual column: the 1.28 MHz band processed in this time per second of data
            "processed_bandwidth_mhz": {"fp32_chain": 1.28 / (ms / 1e3), "bf16x3_chain": 1.28 / (res["bf16x3"] / 1e3),
                                        "paper_c1060_gp4_mhz": 6.9},
-           "fstage": {"kernel": "fengine_kernel<complex8>", "ms": f_ms, "bound": "hbm", "achieved": gbs,
+           "fstage": {"kernel": "fengine_wide_kernel<complex8>", "ms": f_ms, "bound": "hbm", "achieved": gbs,
                       "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "algorithmic_bytes": f_bytes,
                       "peak_source": src},
            "pfb_fstage": {"taps": taps, "ms": pfb_ms, "achieved": pfb_bytes / (pfb_ms / 1e3) / 1e9,
                           "frac": pfb_bytes / (pfb_ms / 1e3) / 1e9 / hbm, "algorithmic_bytes": pfb_bytes,
-                          "note": "each input frame is read by 8 output frames (through L2); bytes counted once"},
+                          "note": "the window stays in registers: each sample is read once"},
            "err_vs_fp64": err,
            "err_sample": "1000-frame slice, all 128 channels, against the oracle's complex128 F and float64 X stages",
            "paper_context": "C1060 (Table 3): unpack 53 + FFT 53 + CMAC (GP, G=4) 185 = 291 ms per second of data",
