@@ -1810,7 +1810,8 @@ bool tc_rawf32_supported(const Plan& p) {
 // x 256 / 1024 281 -> 180 / 780 -> 602.  Odd block counts above one compute half-empty squares and gain
 // nothing on long dumps (320 x 200 x 500 220 -> 167, but 320 x 30 x 2000 126 -> 127).
 bool tc_rawf32_pairs(const Plan& p) {
-    return p.sample_bits == 32 && p.nb >= 2 && (p.nb % 2 == 0 || p.kp <= 1536) && (p.n_inputs % 2) == 0 && !p.tc_float_planes &&
+    return p.sample_bits == 32 && p.nb >= 2 && (p.nb % 2 == 0 || p.kp <= 1536) && (p.n_inputs % 2) == 0 &&
+           !p.tc_float_planes &&
            p.tc_op_stages != 1;   // one operand stage: the plane feed ignores it, this one could not run
 }
 
