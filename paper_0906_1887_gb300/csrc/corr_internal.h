@@ -138,7 +138,8 @@ struct TcTuning {
 };
 int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm);   // n_sm = 0: as many as fit
 int tc_default_cpi(int n_inputs, int64_t channels, int n_sm);   // channels = dumps x n_chan of the launch
-// BF16x3 on float samples with the hi/lo split done in the tensor-core kernel (single-block arrays)
+// BF16x3 on float samples with the hi/lo split done in the tensor-core kernel: without a workspace
+// (single-block arrays of an even count), by pairs of CTAs, and for odd counts
 bool tc_rawf32_supported(const Plan& p);
 bool tc_rawf32_pairs(const Plan& p);   // float samples of several blocks that CTA pairs split in the kernel
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,

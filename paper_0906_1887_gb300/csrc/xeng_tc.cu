@@ -1796,7 +1796,7 @@ cudaError_t launch_raw_impl(const Plan& p, const void* d_packed, int n_dumps, vo
 }  // namespace
 
 bool tc_rawf32_supported(const Plan& p) {
-    // single-block arrays (the float raw stage and hi/lo operand tiles fill the ring), and a
+    // the arrays that ask for no workspace: single-block ones (single CTAs), and a
     // row of N complex floats a multiple of 16 bytes (TMA strides)
     return p.sample_bits == 32 && p.n_inputs <= kBlockInputs && (p.n_inputs % 2) == 0;
 }
