@@ -15,6 +15,7 @@
 
 #include "corr_internal.h"
 #include "launch.cuh"
+#include "ragged_piece.h"
 #include "sample_convert.cuh"
 
 namespace corr {
@@ -111,29 +112,12 @@ struct FastTile {
 // block per SM beside a tensor-core launch, 64 KB in flight per block).  F8 (4-bit only): the
 // planes hold e4m3 bytes instead of fp16 (rows of kp bytes), for the e4m3 plane feed.
 // RAGGED: rows that are no whole 16-byte pieces; a piece is put together from the aligned words
-// around it, and bytes past the row are zero.  Tiles are counted in 32 bits (2^31 tiles of planes are
+// around it (load_piece), and bytes past the row are zero.  Tiles are counted in 32 bits (2^31 tiles of planes are
 // 17 TB); 64-bit divisions of the tile index took a tenth of the time.
-__device__ __forceinline__ uint4 load_piece(const unsigned char* __restrict__ base, int64_t off, int64_t last_word,
-                                            int n_valid) {
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(base);
-    const int64_t i = off >> 2;
-    const uint32_t sh = (uint32_t)(off & 3) * 8;
-    uint32_t x[5], v[4];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) x[k] = w[i + k < last_word ? i + k : last_word];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int left = n_valid - 4 * k;   // bytes of this word inside the row
-        v[k] = __funnelshift_r(x[k], x[k + 1], sh);
-        if (left < 4) v[k] = left <= 0 ? 0u : v[k] & ((1u << (8 * left)) - 1u);
-    }
-    return make_uint4(v[0], v[1], v[2], v[3]);
-}
-
 template <int BITS, int kGroup, bool F8 = false, bool RAGGED = false>
 __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
     const unsigned char* __restrict__ packed, int n_inputs, int n_chan, int n_time, int nb_count, int kp,
-    uint32_t n_tiles, void* __restrict__ planes_out, int64_t last_word) {
+    uint32_t n_tiles, void* __restrict__ planes_out, int64_t n_bytes) {
     static_assert(!F8 || BITS == 4, "e4m3 planes hold 4-bit samples only");
     __half* __restrict__ planes = static_cast<__half*>(planes_out);
     using F = FastTile<BITS>;
@@ -171,9 +155,13 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
                 if (tile_ok && tg < n_time && (int64_t)piece * 16 < valid) {
                     const int64_t off =
                         ((d * n_time + tg) * n_chan + c) * row_bytes + (int64_t)nb * F::kRowBytes + piece * 16;
-                    if constexpr (RAGGED)
-                        v[gi][u] = load_piece(packed, off, last_word, (int)(valid - piece * 16 < 16 ? valid - piece * 16 : 16));
-                    else v[gi][u] = *reinterpret_cast<const uint4*>(packed + off);
+                    if constexpr (RAGGED) {
+                        uint32_t x[4];
+                        load_piece(packed, off, n_bytes, (int)(valid - piece * 16 < 16 ? valid - piece * 16 : 16), x);
+                        v[gi][u] = make_uint4(x[0], x[1], x[2], x[3]);
+                    } else {
+                        v[gi][u] = *reinterpret_cast<const uint4*>(packed + off);
+                    }
                 }
             }
         }
@@ -276,7 +264,7 @@ cudaError_t launch_fast(const Plan& p, const void* d_packed, int n_dumps, void* 
     auto kern = ragged ? unpack_fast_kernel<BITS, 1, F8, true>
                        : blocks_per_sm > 0 ? unpack_fast_kernel<BITS, 8, F8> : unpack_fast_kernel<BITS, 1, F8>;
     return launch_kernel(kern, grid, F::kThreads, 0, s, 1, false, src, p.n_inputs, p.n_chan, p.n_time, p.nb, kp,
-                          (uint32_t)n_tiles, planes, (bytes + 3) / 4 - 1);
+                          (uint32_t)n_tiles, planes, bytes);
 }
 
 // Packed rows [row][row_bytes] -> [row][pitch], pitch a multiple of 16 bytes: rows that TMA can
@@ -287,7 +275,7 @@ cudaError_t launch_fast(const Plan& p, const void* d_packed, int n_dumps, void* 
 template <bool FLOAT>
 __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __restrict__ packed,
                                                      unsigned char* __restrict__ out, uint32_t rows, int row_bytes,
-                                                     int pieces, uint32_t rows_per_block, int64_t last_word) {
+                                                     int pieces, uint32_t rows_per_block, int64_t n_bytes) {
     grid_release();
     for (uint32_t r0 = blockIdx.x * rows_per_block; r0 < rows; r0 += gridDim.x * rows_per_block) {
         const uint32_t n = min(rows_per_block, rows - r0) * (uint32_t)pieces;
@@ -299,10 +287,12 @@ __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __rest
             const int64_t off = base + (int64_t)r * row_bytes + (e - r * pieces) * 16;
             if constexpr (FLOAT) {
                 const uint2 a = *reinterpret_cast<const uint2*>(packed + off);
-                const uint2 b = (off >> 2) + 3 <= last_word ? *reinterpret_cast<const uint2*>(packed + off + 8) : uint2{};
+                const uint2 b = off + 16 <= n_bytes ? *reinterpret_cast<const uint2*>(packed + off + 8) : uint2{};
                 dst[e] = make_uint4(a.x, a.y, b.x, b.y);
             } else {
-                dst[e] = load_piece(packed, off, last_word, 16);
+                uint32_t x[4];
+                load_piece(packed, off, n_bytes, 16, x);
+                dst[e] = make_uint4(x[0], x[1], x[2], x[3]);
             }
         }
     }
@@ -350,7 +340,7 @@ cudaError_t launch_repack(const Plan& p, const void* d_packed, int n_dumps, void
     const int64_t want = (rows + per - 1) / per, cap = (int64_t)p.n_sm * 8;
     return launch_kernel(p.sample_bits == 32 ? repack_kernel<true> : repack_kernel<false>, dim3((unsigned)(want < cap ? want : cap)), 256, 0, s, 1, false,
                           static_cast<const unsigned char*>(d_packed), static_cast<unsigned char*>(d_out), (uint32_t)rows,
-                          row_bytes, pieces, (uint32_t)per, (rows * row_bytes + 3) / 4 - 1);
+                          row_bytes, pieces, (uint32_t)per, rows * row_bytes);
 }
 
 cudaError_t launch_unpack_f32(const Plan& p, const void* d_packed, int n_dumps, void* d_planes, cudaStream_t s) {
