@@ -716,8 +716,6 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
                     }
                 }
             }
-            // the issuing CTA's last commits must have arrived here before this CTA exits
-            if (lane == 0) ptx::mbar_wait_drain(bar_drain, 0, kDrainLimitNs);
         } else if (lane == 0) {
             constexpr uint32_t idesc_wide = ptx::idesc_f16(PAIR ? 256 : 128, 256, C::kSplit);
             auto wait = [&](uint32_t bar, uint32_t parity) {
@@ -830,6 +828,8 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
             if (any) {
                 commit(bar_drain);
                 ptx::mbar_wait_drain(bar_drain, 0, kDrainLimitNs);
+            } else if constexpr (PAIR) {
+                ptx::mbar_arrive_cluster(ptx::map_shared(bar_drain, 1));   // nothing to come for the peer
             }
         }
         __syncwarp();
@@ -1311,6 +1311,12 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
     if constexpr (PAIR) {
         __syncwarp();
         ptx::cluster_sync();   // neither CTA's memory goes while the other may still arrive there or read it
+        // The issuing CTA has seen its last commit; the same commits must have arrived here before
+        // this CTA exits.  The limit runs from here, not from the start of a launch that may take longer.
+        if (rank != 0 && warp == 1) {
+            if (lane == 0) ptx::mbar_wait_drain(bar_drain, 0, kDrainLimitNs);
+            __syncwarp();
+        }
     } else {
         __syncthreads();
     }
