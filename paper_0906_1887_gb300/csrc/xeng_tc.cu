@@ -1667,12 +1667,14 @@ int tc_default_cpi(int n_inputs, int64_t channels, int n_sm) {
 // after another, so `pack` adjacent channels of n inputs are pack n adjacent inputs of one tile, of
 // whose products the epilogue keeps each channel's own: TMA boxes, conversions and MMAs then carry
 // pack channels for the price of one padded one.  Tiles start at 16-byte multiples and time samples
-// are 16-byte multiples (TMA), which also admits rows of fewer than 16 bytes or odd ones.  A small
-// launch keeps one tile per SM rather than fewer fuller ones.
+// are 16-byte multiples (TMA), which also admits rows of fewer than 16 bytes or odd ones.  A tile's
+// place in the time sample is a 32-bit coordinate (in bytes, or in complex floats), so longer time
+// samples do not pack.  A small launch keeps one tile per SM rather than fewer fuller ones.
 int tc_channel_pack(int n_inputs, int bps, int n_chan, int64_t n_dumps, int n_sm) {
     const int64_t row = (int64_t)n_inputs * bps;
+    const int64_t extent = (bps == 8 ? n_inputs : row) * n_chan;
     const bool aligned = row % 16 == 0;
-    if (n_inputs > kBlockInputs / 2 || row * n_chan % 16 != 0) return aligned ? 1 : 0;
+    if (n_inputs > kBlockInputs / 2 || row * n_chan % 16 != 0 || extent >= (int64_t{1} << 31)) return aligned ? 1 : 0;
     int step = 1;   // smallest pack whose tiles are 16-byte multiples
     while (row * step % 16) ++step;
     const int most = kBlockInputs / n_inputs;
