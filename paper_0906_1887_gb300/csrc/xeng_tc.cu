@@ -1600,7 +1600,8 @@ bool tc_use_pairs(const Plan& p, bool packed) {
 // 702 -> 642, 1024 x 512 / 768 / 1024 536 -> 446 / 579 -> 549 / 666 -> 695; 4-bit, 192 x 384 94 -> 77,
 // 400 x 512 320 -> 308, 1024 x 512 / 768 527 -> 488 / 505 -> 457, but 400 x 768 356 -> 417.
 bool tc_packed_pairs(const Plan& p, int accumulate) {
-    if (p.tc_operands != 0 || p.tc_items != 0 || p.nb < 2) return false;
+    // one operand stage (set_tuning): the plane feed ignores it, the packed one could not run
+    if (p.tc_operands != 0 || p.tc_items != 0 || p.nb < 2 || p.tc_op_stages == 1) return false;
     const bool even = p.nb % 2 == 0;
     if (accumulate)
         return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= (p.nb <= 12 ? 1024 : 768) : p.kp <= (even ? 768 : 512);
@@ -1651,6 +1652,7 @@ bool tc_raw_supported(const Plan& p) { return tc_raw_supported(p.n_inputs, p.sam
 
 bool tc_raw_by_packing(const Plan& p) {
     return (p.sample_bits == 4 || p.sample_bits == 8) && !tc_raw_supported(p) && p.tc_operands == 0 &&
+           p.tc_op_stages != 1 &&   // as in tc_packed_pairs
            tc_channel_pack(p.n_inputs, p.sample_bits == 8 ? 2 : 1, p.n_chan, 1, p.n_sm) > 1;
 }
 
@@ -1892,7 +1894,7 @@ cudaError_t launch_xeng_tc_raw(const Plan& p, const void* d_packed, int n_dumps,
 cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
                                  int accumulate, cudaStream_t s) {
     const bool ragged = !tc_raw_supported(p), aligned = (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0;
-    const bool packed = tc_packed_pairs(p, accumulate) || (ragged && p.tc_operands == 0 &&
+    const bool packed = tc_packed_pairs(p, accumulate) || (ragged && p.tc_operands == 0 && p.tc_op_stages != 1 &&
                                                p.nb < (p.sample_bits == 4 ? kPlaneMinBlocksE4m3 : kPlaneMinBlocks));
     if (packed && aligned) {
         if (!ragged) return launch_xeng_tc_raw(p, d_packed, n_dumps, d_vis, accumulate, s);
