@@ -72,6 +72,8 @@ cudaError_t launch_unpack_bf16x2(const Plan& p, const void* d_packed, int n_dump
                                  void* d_lo, cudaStream_t s);
 cudaError_t launch_xeng_fp32(const Plan& p, const void* d_planes, int n_dumps, void* d_vis,
                              int accumulate, cudaStream_t s);
+// ranges of the sample axis the FP32 engine's items are split into: their count and length
+void fp32_sample_ranges(int n_time, int n_sm, int64_t base_items, int* ts, int* range_len);
 // FP32 engine on the packed samples themselves (4/8-bit or float32), no planes
 cudaError_t launch_xeng_fp32_packed(const Plan& p, const void* d_packed, int n_dumps, void* d_vis, int accumulate,
                                     cudaStream_t s);

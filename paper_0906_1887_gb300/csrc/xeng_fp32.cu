@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
 // shared memory, thread-private 16-byte pieces, and reach the output once per item (a store, or a
 // float2 reduction when accumulating or split over sample ranges); adding every partial into the
 // output took one scattered reduction per element and 64 samples, a quarter of the time (64 inputs x
-// 768 channels x 1000 samples: 391 -> 300 us with the fuller waves of sample_ranges, 0.57 of the FFMA
+// 768 channels x 1000 samples: 391 -> 300 us with the fuller waves of fp32_sample_ranges, 0.57 of the FFMA
 // rate; what is left is issue and dispatch in the FFMA stream).  Chunks of 8 samples leave both row buffers of four diagonal
 // or two off-diagonal channel-dumps (40 KB) and the totals (64 KB) room for two blocks per SM.
 constexpr int kFChunk = 8;
@@ -821,31 +821,6 @@ __global__ void __launch_bounds__(DIAG ? kIDiagThreads : kIOffThreads, 2)
     }
 }
 
-// Sample ranges per item for a launch of base_items items: with fewer than two waves of two
-// blocks per SM, the sample axis is split (whole chunks, at least 64 samples a range) so that the
-// waves are full: the number of ranges with the smallest waves x (range + some 24 samples an item
-// costs besides).  768 channels of 64 inputs (192 items, 304 blocks), 1000 samples: 3 ranges run
-// in 2 waves of 352 samples where 4 took 3 waves of 256.
-void sample_ranges(const Plan& p, int64_t base_items, int* ts, int* range_len) {
-    const int64_t slots = 2LL * p.n_sm;
-    int best_len = (p.n_time + kIChunk - 1) / kIChunk * kIChunk;
-    if (base_items > 0 && base_items < 2 * slots) {
-        int64_t best = INT64_MAX;
-        const int t_max = (p.n_time + 63) / 64 < 64 ? (p.n_time + 63) / 64 : 64;
-        for (int t = 1; t <= t_max; ++t) {
-            const int len = ((p.n_time + t - 1) / t + kIChunk - 1) / kIChunk * kIChunk;
-            const int n = (p.n_time + len - 1) / len;
-            const int64_t cost = (base_items * n + slots - 1) / slots * (len + 24);
-            if (cost < best) {
-                best = cost;
-                best_len = len;
-            }
-        }
-    }
-    *range_len = best_len;
-    *ts = (p.n_time + best_len - 1) / best_len;
-}
-
 template <int BITS, bool VEC>
 cudaError_t launch_int_feed(const Plan& p, const unsigned char* src, int64_t n_dc, longlong2* out, int accumulate,
                             cudaStream_t s) {
@@ -853,8 +828,8 @@ cudaError_t launch_int_feed(const Plan& p, const unsigned char* src, int64_t n_d
     const int64_t diag_base = (n_dc + kIDiagCh - 1) / kIDiagCh * p.nb;
     const int64_t off_base = (n_dc + kIOffCh - 1) / kIOffCh * (p.nb * (p.nb - 1) / 2);
     int ts_d, len_d, ts_o, len_o;
-    sample_ranges(p, diag_base, &ts_d, &len_d);
-    sample_ranges(p, off_base, &ts_o, &len_o);
+    fp32_sample_ranges(p.n_time, p.n_sm, diag_base, &ts_d, &len_d);
+    fp32_sample_ranges(p.n_time, p.n_sm, off_base, &ts_o, &len_o);
     const int64_t diag_items = diag_base * ts_d, off_items = off_base * ts_o;
     // rows (20 KB per channel-dump and block), one chunk of raw pieces, the item
     const int per = kIChunk * kIRow * (int)sizeof(float2) + kIChunk * 64 * bps;
@@ -895,8 +870,8 @@ cudaError_t launch_float_feed(const Plan& p, const float2* src, int64_t n_dc, fl
     const int64_t diag_base = (n_dc + kIDiagCh - 1) / kIDiagCh * p.nb;
     const int64_t off_base = (n_dc + kIOffCh - 1) / kIOffCh * (p.nb * (p.nb - 1) / 2);
     int ts_d, len_d, ts_o, len_o;
-    sample_ranges(p, diag_base, &ts_d, &len_d);
-    sample_ranges(p, off_base, &ts_o, &len_o);
+    fp32_sample_ranges(p.n_time, p.n_sm, diag_base, &ts_d, &len_d);
+    fp32_sample_ranges(p.n_time, p.n_sm, off_base, &ts_o, &len_o);
     const int64_t diag_items = diag_base * ts_d, off_items = off_base * ts_o;
     // two row buffers (5 KB per channel-dump and block each), 256 bytes of totals per thread, the item
     const int smem_diag = 2 * kIDiagCh * kFChunk * kIRow * (int)sizeof(float2) + 256 * kIDiagThreads +
@@ -953,6 +928,38 @@ cudaError_t launch_int(const Plan& p, const void* d_packed, int n_dumps, void* d
 }
 
 }  // namespace
+
+// Sample ranges per item for a launch of base_items items: with fewer than two waves of two
+// blocks per SM, the sample axis is split (whole chunks, at least 64 samples a range) so that the
+// waves are full: the number of ranges with the smallest waves x (range + some 24 samples an item
+// costs besides).  768 channels of 64 inputs (192 items, 304 blocks), 1000 samples: 3 ranges run
+// in 2 waves of 352 samples where 4 took 3 waves of 256.  Counts up to 64 are all tried; above, which
+// only few items with long dumps reach, the largest counts of one to four waves (up to 64 alone, 4
+// channels x 20000 samples ran on 64 blocks of 304).
+void fp32_sample_ranges(int n_time, int n_sm, int64_t base_items, int* ts, int* range_len) {
+    const int64_t slots = 2LL * n_sm;
+    int best_len = (int)(((int64_t)n_time + kIChunk - 1) / kIChunk * kIChunk);
+    if (base_items > 0 && base_items < 2 * slots) {
+        int64_t best = INT64_MAX;
+        auto consider = [&](int64_t t) {
+            const int len = (int)((((int64_t)n_time + t - 1) / t + kIChunk - 1) / kIChunk * kIChunk);
+            const int64_t n = ((int64_t)n_time + len - 1) / len;
+            const int64_t cost = (base_items * n + slots - 1) / slots * (len + 24);
+            if (cost < best) {
+                best = cost;
+                best_len = len;
+            }
+        };
+        const int64_t t_max = ((int64_t)n_time + 63) / 64;
+        for (int64_t t = 1; t <= (t_max < 64 ? t_max : 64); ++t) consider(t);
+        for (int waves = 1; waves <= 4; ++waves) {
+            const int64_t t = waves * slots / base_items < t_max ? waves * slots / base_items : t_max;
+            if (t > 64) consider(t);
+        }
+    }
+    *range_len = best_len;
+    *ts = (int)(((int64_t)n_time + best_len - 1) / best_len);
+}
 
 cudaError_t launch_xeng_fp32_packed(const Plan& p, const void* d_packed, int n_dumps, void* d_vis, int accumulate,
                                     cudaStream_t s) {
