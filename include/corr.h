@@ -387,7 +387,8 @@ typedef struct {
     float tune_ms;              /* the tuner's best time, ms (0 if not tuned) */
     int plane_min_nb;           /* jobs of at least this many blocks read planes (0: none) */
     size_t plane_bytes;         /* the batch's plane workspace */
-    int wide;                   /* plane jobs run wide work items (see CORR_ITEMS_WIDE) */
+    int wide;                   /* 1: plane jobs run wide work items (see CORR_ITEMS_WIDE); 0: single
+                                   tiles, or pairs of CTAs on 2 x 2 squares of tiles */
     int plane_splits;           /* plane jobs in this many launches, each run's unpack overlapping the
                                    previous run's tensor-core launch (1: unpacks, then one launch) */
 } corr_batch_stats;
@@ -411,7 +412,8 @@ corr_status corr_batch_create(corr_batch *out, const corr_job *jobs, int n_jobs,
  * pair_cpi (channels per work item of single-block arrays, 1 or 2), order (0: costliest jobs'
  * items first, 1: the caller's order), plane_min_nb (jobs of at least this many 64-input blocks
  * read fp16 planes; 0 = none; > 0 needs CORR_BATCH_PLANES), wide (plane jobs: 1 = wide work
- * items, 0 = single tiles), plane_splits (1..8: the plane jobs in this many launches of about
+ * items, 0 = single tiles; 2 = arrays of several blocks, packed or planes, by pairs of CTAs on 2 x 2
+ * squares of tiles, as the tuner may choose), plane_splits (1..8: the plane jobs in this many launches of about
  * equal products; the unpacks run back to back on the low-priority stream and each launch waits
  * for its own jobs' unpacks, so unpacking overlaps the tensor cores' work; each such launch
  * leaves 10 KB of shared memory per SM for an unpack block).  A captured graph is re-captured.

@@ -358,7 +358,8 @@ class Batch:
 
     def set_shape(self, op_stages: int = 0, pair_cpi: int = 2, order: int = 0, plane_min_nb: int = 0, wide: int = 1,
                   plane_splits: int = 1):
-        """Launch shape chosen by the caller instead of the tuner (results do not depend on it)."""
+        """Launch shape chosen by the caller instead of the tuner (results do not depend on it).  wide: plane
+        jobs as 0 single tiles or 1 wide items; 2 arrays of several blocks by pairs of CTAs."""
         check(lib().corr_batch_set_shape(self._h, op_stages, pair_cpi, order, plane_min_nb, wide, plane_splits),
               "corr_batch_set_shape")
 

@@ -572,9 +572,9 @@ corr_status corr_batch_set_shape(corr_batch b, int op_stages, int pair_cpi, int 
                                  int plane_splits) {
     if (!b) return set_error(CORR_EINVAL, "corr_batch_set_shape: NULL batch");
     if (op_stages < 0 || op_stages > 16 || (pair_cpi != 1 && pair_cpi != 2) || (order != 0 && order != 1) ||
-        plane_min_nb < 0 || (wide != 0 && wide != 1) || plane_splits < 1 || plane_splits > kMaxPlaneSplits)
+        plane_min_nb < 0 || wide < 0 || wide > 2 || plane_splits < 1 || plane_splits > kMaxPlaneSplits)
         return set_error(CORR_EINVAL, "corr_batch_set_shape: op_stages in [0, 16], pair_cpi 1 or 2, order 0 or 1, "
-                                      "plane_min_nb >= 0, wide 0 or 1, plane_splits in [1, %d]", kMaxPlaneSplits);
+                                      "plane_min_nb >= 0, wide 0, 1 or 2, plane_splits in [1, %d]", kMaxPlaneSplits);
     if (plane_min_nb > 0 && !b->d_planes)
         return set_error(CORR_EINVAL, "plane_min_nb > 0 needs a batch created with CORR_BATCH_PLANES");
     TuneChoice c;
@@ -582,8 +582,8 @@ corr_status corr_batch_set_shape(corr_batch b, int op_stages, int pair_cpi, int 
     c.pair_cpi = pair_cpi;
     c.order = order;
     c.plane_min_nb = plane_min_nb;
-    c.wide = wide;
-    c.pair = wide;   // the single tiles of wide = 0 are single CTAs'
+    c.wide = wide == 1;
+    c.pair = wide == 2;
     c.plane_splits = plane_splits;
     if (!build_groups(b, c)) return set_error(CORR_EINVAL, "tensor map encoding failed");
     b->choice = c;
@@ -624,7 +624,7 @@ corr_status corr_batch_info(corr_batch b, corr_batch_stats* st) {
     st->order = b->choice.order;
     st->tune_ms = b->choice.ms;
     st->plane_min_nb = b->choice.plane_min_nb;
-    st->wide = b->choice.wide;
+    st->wide = b->choice.wide && !b->choice.pair;
     st->plane_splits = b->choice.plane_splits;
     st->plane_bytes = b->plane_bytes;
     return CORR_OK;
