@@ -61,8 +61,9 @@ __host__ __device__ constexpr int fw_lgns(int lgh, bool real, int st) {   // log
     return o;
 }
 // twiddle tables: stage st (>= 1) holds exp(-2 pi i k r / (Ns R)) at k (R - 1) + r - 1; after the
-// stages, for real samples, exp(-2 pi i (p + q H / R) / L) at p R + q for p = 0 .. H / R / 2 of the
-// last stage (one rounding each: a task's root times a 16th root cost 5 to 20% in the error)
+// stages, for real samples, w = exp(-2 pi i (p + q H / R) / L) at p R + q for p = 0 .. H / R / 2 of the
+// last stage (one rounding each: a task's root times a 16th root cost 5 to 20% in the error), and in
+// the same order what w's rounding dropped (FW::kExact)
 __host__ __device__ constexpr int fw_tw_offset(int lgh, bool real, int st) {
     int o = 0;
     for (int u = 1; u < st; ++u) o += (1 << fw_lgns(lgh, real, u)) * ((1 << fw_lgr(lgh, real, u)) - 1);
@@ -101,7 +102,11 @@ struct FW {
     // few inputs) then fall in distinct banks
     static constexpr int CP = C + (MT && G == 8 ? 8 : MT && G == 4 ? 4 : MT && G == 2 ? 2 : 0);
     static constexpr int NOUT = kReal ? H + 1 : H;
-    static constexpr int TWN = fw_tw_entries(LGH, kReal);
+    // How far a real spectrum's split keeps its roundings (fw_split): as far as the error must not exceed that
+    // of the full-length transform, whose 0.97 to 1.08 a plain split has (least for plain transforms of
+    // 512 points and more, most for filterbanks of 64).
+    static constexpr int kExact = !kReal ? 0 : MT == 0 ? (LGL == 8 ? 1 : 0) : (LGL <= 8 || LGL == 11 ? 3 : 2);
+    static constexpr int TWN = fw_tw_entries(LGH, kReal) + (kExact > 0 ? fw_split_entries(LGH, kReal) : 0);
     static constexpr int ROWB = G * BPS;                       // packed bytes of a sample row
     static constexpr int PIECE = ROWB < 16 ? ROWB : 16;        // bytes of one asynchronous copy
     static constexpr int RAWB = MT ? 0 : FB * L * ROWB;        // packed bytes of a batch
@@ -154,17 +159,71 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {
     return s;
 }
 
-// X[k] and X[H - k] from Z[k] and Z[H - k]; w = exp(-2 pi i k / L).  The sums and differences keep
-// their rounding errors, so the split adds one rounding of the result to the transform's own error
-// (without: 2 to 10% more than the full-length complex transform has).
-__device__ __forceinline__ void fw_split(float2 z, float2 zp, float2 w, float2& xk, float2& xm) {
+// a b = p + e exactly
+__device__ __forceinline__ float two_prod(float a, float b, float& e) {
+    const float p = __fmul_rn(a, b);
+    e = fmaf(a, b, -p);
+    return p;
+}
+
+// X[k] and X[H - k] from Z[k] and Z[H - k]; w = exp(-2 pi i k / L), wl what its rounding dropped.  The sums
+// and differences 2 E and 2 O always keep their rounding errors.  EXACT = 1 adds wl and the errors
+// of one product each of 2 W O, 2 those of both and of their sum, 3 that of the last sum as well, which
+// leaves the rounding of the result.  Error relative to the full-length transform's, and time of 2^26
+// samples of 128 inputs, 0 -> the one chosen (FW::kExact): filterbanks of 8 taps, L = 32 1.05 -> 0.97, 94
+// -> 116 us; 64 1.06 -> 0.99, 97 -> 124; 128 1.05 -> 1.00, 116 -> 145; 256 1.03 -> 0.98, 127 -> 158; 512
+// 1.02 -> 0.99, 170 -> 180; 1024 1.02 -> 0.99, 242 -> 269; 2048 1.03 -> 0.99, 436 -> 465; plain, L = 256
+// 1.005 -> 0.97, 86 -> 89.
+template <int EXACT>
+__device__ __forceinline__ void fw_split(float2 z, float2 zp, float2 w, float2 wl, float2& xk, float2& xm) {
     float er, ei, fr, fi;
     const float sr = two_sum(z.x, zp.x, er), si = two_sum(z.y, -zp.y, ei);   // 2 E
     const float dr = two_sum(z.y, zp.y, fr), di = two_sum(zp.x, -z.x, fi);   // 2 O
-    const float pr = fmaf(fr, w.x, fmaf(-fi, w.y, fmaf(dr, w.x, -(di * w.y))));   // 2 W O
-    const float pi = fmaf(fr, w.y, fmaf(fi, w.x, fmaf(dr, w.y, di * w.x)));
-    xk = make_float2(0.5f * (sr + (pr + er)), 0.5f * (si + (pi + ei)));
-    xm = make_float2(0.5f * (sr - (pr - er)), 0.5f * ((pi - ei) - si));
+    if constexpr (EXACT == 0) {
+        const float pr = fmaf(fr, w.x, fmaf(-fi, w.y, fmaf(dr, w.x, -(di * w.y))));   // 2 W O
+        const float pi = fmaf(fr, w.y, fmaf(fi, w.x, fmaf(dr, w.y, di * w.x)));
+        xk = make_float2(0.5f * (sr + (pr + er)), 0.5f * (si + (pi + ei)));
+        xm = make_float2(0.5f * (sr - (pr - er)), 0.5f * ((pi - ei) - si));
+    } else {
+        float b, d, pr, pi, cr, ci;   // 2 W O = pr + cr, pi + ci
+        const float p1 = two_prod(di, w.y, b), q1 = two_prod(di, w.x, d);
+        if constexpr (EXACT == 1) {
+            pr = fmaf(dr, w.x, -p1);
+            pi = fmaf(dr, w.y, q1);
+            cr = -b;
+            ci = d;
+        } else {
+            float a, c, e, f;
+            const float p0 = two_prod(dr, w.x, a), q0 = two_prod(dr, w.y, c);
+            pr = two_sum(p0, -p1, e);
+            pi = two_sum(q0, q1, f);
+            cr = e + (a - b);
+            ci = f + (c + d);
+        }
+        cr = fmaf(dr, wl.x, fmaf(-di, wl.y, fmaf(fr, w.x, fmaf(-fi, w.y, cr))));
+        ci = fmaf(dr, wl.y, fmaf(di, wl.x, fmaf(fr, w.y, fmaf(fi, w.x, ci))));
+        if constexpr (EXACT < 3) {
+            xk = make_float2(0.5f * (sr + (pr + (cr + er))), 0.5f * (si + (pi + (ci + ei))));
+            xm = make_float2(0.5f * (sr - (pr + (cr - er))), 0.5f * ((pi + (ci - ei)) - si));
+        } else {
+            float g;
+            const float kr = two_sum(sr, pr, g);
+            xk.x = 0.5f * (kr + (g + (er + cr)));
+            const float ki = two_sum(si, pi, g);
+            xk.y = 0.5f * (ki + (g + (ei + ci)));
+            const float mr = two_sum(sr, -pr, g);
+            xm.x = 0.5f * (mr + (g + (er - cr)));
+            const float mi = two_sum(pi, -si, g);
+            xm.y = 0.5f * (mi + (g + (ci - ei)));
+        }
+    }
+}
+
+// the dropped part of the root at w, for FW::kExact
+template <class F>
+__device__ __forceinline__ float2 fw_low(const float2* w) {
+    if constexpr (F::kExact > 0) return w[fw_split_entries(F::LGH, true)];
+    else return float2{};
 }
 
 template <class F, int R, int Q>
@@ -173,7 +232,7 @@ __device__ __forceinline__ void fw_split_pairs(const float2 (&a)[R], const float
     if constexpr (Q < R) {   // channel p + q H / R and its mirror, output R - 1 - q of the mirror task
         constexpr int NS = F::H / R;
         float2 xk, xm;
-        fw_split(a[Q], b[R - 1 - Q], w[Q], xk, xm);
+        fw_split<F::kExact>(a[Q], b[R - 1 - Q], w[Q], fw_low<F>(w + Q), xk, xm);
         const int k = p + Q * NS;
         o[k * N] = xk;
         o[(F::H - k) * N] = xm;
@@ -186,7 +245,7 @@ __device__ __forceinline__ void fw_split_self(const float2 (&a)[R], const float2
     if constexpr (Q < R / 2) {   // task 0: channels q H / R, mirrored at R - q of the same task
         constexpr int NS = F::H / R;
         float2 xk, xm;
-        fw_split(a[Q], a[R - Q], w[Q], xk, xm);
+        fw_split<F::kExact>(a[Q], a[R - Q], w[Q], fw_low<F>(w + Q), xk, xm);
         o[Q * NS * N] = xk;
         o[(F::H - Q * NS) * N] = xm;
         fw_split_self<F, R, Q + 1>(a, w, o, N);
@@ -198,7 +257,7 @@ __device__ __forceinline__ void fw_split_mid(const float2 (&b)[R], const float2*
     if constexpr (Q < R / 2) {   // task H / R / 2: channels (q + 1/2) H / R, mirrored at R - 1 - q
         constexpr int NS = F::H / R;
         float2 xk, xm;
-        fw_split(b[Q], b[R - 1 - Q], w[Q], xk, xm);
+        fw_split<F::kExact>(b[Q], b[R - 1 - Q], w[Q], fw_low<F>(w + Q), xk, xm);
         o[(NS / 2 + Q * NS) * N] = xk;
         o[(F::H - NS / 2 - Q * NS) * N] = xm;
         fw_split_mid<F, R, Q + 1>(b, w, o, N);
@@ -589,14 +648,13 @@ cudaError_t launch_kind(const FWideArgs& p, cudaStream_t s) {
 // Plain complex transforms of 32 points and more: c8 of 128 inputs, L = 32 .. 4096: 138 -> 115,
 // (110 -> 116), 126 -> 119, 153 -> 123, 238 -> 163, 274 -> 179, 465 -> 216, 1067 -> 402; 16 inputs,
 // L = 64: 270 -> 115.  L = 64 of whole groups of 64 inputs stays with fengine.cu.
-// Plain real transforms of 256 points and more: 112 -> 87, 194 -> 94, 226 -> 108, 339 -> 119,
-// 755 -> 166; their error against 64 bits is that of the full-length transform (1.0e-7 at 1024
-// points).  Shorter ones keep fengine.cu: at half length their error would be 5% larger.
+// Plain real transforms of 256 points and more: 112 -> 89, 194 -> 94, 226 -> 108, 339 -> 119,
+// 755 -> 166.  Shorter ones keep fengine.cu.
 // Filterbanks of up to 8 taps where four frames of at least two inputs fit: 8 taps, c8, L = 32 ..
-// 512: 403 -> 158, 302 -> 163, 313 -> 178, 421 -> 212, 515 -> 331; r8, L = 32 .. 1024: 308 -> 88,
-// 244 -> 94, 252 -> 112, 342 -> 127, 442 -> 169, 938 -> 242 (error 1.0e-7 .. 1.2e-7, within 5%).  With
-// two inputs, 8 taps, 128 / 336 inputs: c8, L = 1024: 1025 -> 577 / 1411 -> 582; r8, L = 2048: 1590 ->
-// 434, 481 inputs 1659 -> 585, 4 taps 908 -> 373 / 882 -> 364 (error 1.28e-7, 1.25e-7 before).
+// 512: 403 -> 158, 302 -> 163, 313 -> 178, 421 -> 212, 515 -> 331; r8, L = 32 .. 1024: 308 -> 116,
+// 244 -> 124, 252 -> 145, 342 -> 158, 440 -> 180, 942 -> 269.  With two inputs, 8 taps, 128 / 336 inputs:
+// c8, L = 1024: 1025 -> 577 / 1411 -> 582; r8, L = 2048: 1604 -> 465 / 1418 -> 480, 4 taps 915 -> 404 /
+// 882 -> 394.  Real spectra of either kind have no more error than the full-length transform (fw_split).
 // The few taps of a long complex transform stay with fengine.cu, which pays for each tap: c8 of 128
 // inputs, L = 512, 2 / 3 / 4 taps: 267 / 304 / 335 there, 313 here; c4, L = 256, 2 / 4 taps: 193 / 258
 // there, 205 / 200 here; L = 1024, 4 / 6 taps: 476 / 823 there, 544 / 577 here.
@@ -622,8 +680,13 @@ std::vector<float2> fwide_tables(int kind, int log2L) {
     }
     if (real) {
         const int r_ = 1 << fw_lgr(lgh, real, fw_stages(lgh, real) - 1), ns = (1 << lgh) / r_;
-        for (int p = 0; p <= ns / 2; ++p)
-            for (int q = 0; q < r_; ++q) tw.push_back(root(p + q * ns, 1 << log2L));
+        for (int low = 0; low < 2; ++low)
+            for (int p = 0; p <= ns / 2; ++p)
+                for (int q = 0; q < r_; ++q) {
+                    const float2 w = root(p + q * ns, 1 << log2L);
+                    const double ang = -2.0 * M_PI * (double)(p + q * ns) / (double)(1 << log2L);
+                    tw.push_back(low ? make_float2((float)(cos(ang) - (double)w.x), (float)(sin(ang) - (double)w.y)) : w);
+                }
     }
     return tw;
 }
