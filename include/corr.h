@@ -301,7 +301,8 @@ corr_status corr_fengine_run(corr_fplan plan, const void *d_time, int n_frames, 
  * x L floats) must fit in shared memory beside the transform buffers (n_taps x L <= about
  * 28000; CORR_EINVAL otherwise).  For such a plan
  * corr_fengine_run's d_time must hold n_frames + n_taps - 1 frames of L samples; n_frames
- * spectra are produced.  Destroy with corr_fplan_destroy.
+ * spectra are produced.  Filterbanks of few frames run on another kernel than long ones, so the last bits of
+ * a frame's spectrum may depend on n_frames (those of plain transforms do not).  Destroy with corr_fplan_destroy.
  */
 corr_status corr_fplan_create_pfb(corr_fplan *out, int n_inputs, int n_chan, int kind, int n_taps, const float *h_taps);
 /* Taps of an F-stage plan (1 for a plain-transform plan). */

@@ -687,7 +687,7 @@ corr_status corr_fengine_run(corr_fplan plan, const void* d_time, int n_frames, 
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e;
     const bool pfb = p->d_taps != nullptr;
-    if (p->d_tw_wide && fwide_takes(p->kind, p->log2L, p->n_inputs, pfb ? p->n_taps : 0))
+    if (p->d_tw_wide && fwide_takes(p->kind, p->log2L, p->n_inputs, pfb ? p->n_taps : 0, n_frames, p->n_sm))
         e = launch_fwide({p->kind, p->log2L, p->n_inputs, n_frames, p->n_taps, p->n_sm, d_time, d_spectra,
                           p->d_tw_wide, p->d_taps}, s);
     else if (p->kind == CORR_F_COMPLEX8)

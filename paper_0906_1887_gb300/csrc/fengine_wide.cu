@@ -87,14 +87,16 @@ __host__ __device__ constexpr int fw_threads(int lgh, int mt) {
     return lgh <= 8 ? 256 : lgh == 9 ? 512 : 1024;
 }
 
-template <int KIND, int LGL, int MT>
+// ROW < 16: plain transforms in CTAs of 4096 points, with rows of at most ROW inputs (plain_row).  A column's
+// arithmetic is the same in every geometry, and so are its bits.
+template <int KIND, int LGL, int MT, int ROW = 16>
 struct FW {
     static constexpr bool kReal = KIND == CORR_F_REAL8;
     static constexpr int BPS = f_bps<KIND>();
     static constexpr int L = 1 << LGL, LGH = LGL - (kReal ? 1 : 0), H = 1 << LGH;
-    static constexpr int T = fw_threads(LGH, MT);
+    static constexpr int T = ROW < 16 ? 256 : fw_threads(LGH, MT);
     static constexpr int C = 16 * T / H;                       // columns
-    static constexpr int G = MT ? C / 4 : (C < 16 ? C : 16);   // inputs (16: whole 128-byte lines out)
+    static constexpr int G = MT ? C / 4 : (C < ROW ? C : ROW);   // inputs (16: whole 128-byte lines out)
     static constexpr int FB = C / G;                           // frames per batch
     static constexpr int NST = fw_stages(LGH, kReal);
     static constexpr int PS = fw_lgr(LGH, kReal, 0);           // one pad row after every first radix of rows
@@ -108,7 +110,7 @@ struct FW {
     static constexpr int kExact = !kReal ? 0 : MT == 0 ? (LGL == 8 ? 1 : 0) : (LGL <= 8 || LGL == 11 ? 3 : 2);
     static constexpr int TWN = fw_tw_entries(LGH, kReal) + (kExact > 0 ? fw_split_entries(LGH, kReal) : 0);
     static constexpr int ROWB = G * BPS;                       // packed bytes of a sample row
-    static constexpr int PIECE = ROWB < 16 ? ROWB : 16;        // bytes of one asynchronous copy
+    static constexpr int PIECE = ROWB < 16 ? ROWB : 16;        // bytes of one asynchronous copy, at most
     static constexpr int RAWB = MT ? 0 : FB * L * ROWB;        // packed bytes of a batch
     static constexpr int DATA = ((H - 1) + ((H - 1) >> PS) + 1) * CP;   // float2
     static constexpr int SMEM = (DATA + TWN) * 8 + RAWB + 16;
@@ -339,26 +341,36 @@ __device__ __forceinline__ void cp_async(uint32_t dst, const void* src, int byte
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// packed samples of `rows` sample rows of the CTA's inputs -> shared memory [row][G]
+// packed samples of `rows` sample rows of the CTA's inputs -> shared memory [row][G], in pieces of P bytes
+// where rows and their first byte are multiples of that (plain_piece), else sample by sample
+template <class F, int P>
+__device__ __forceinline__ void fw_fetch_pieces(uint8_t* raw, const uint8_t* src, int rows, int N, int g_n) {
+    constexpr int PP = F::ROWB / P;
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(raw));
+    for (int e = threadIdx.x; e < rows * PP; e += F::T) {
+        const int row = e / PP, pc = e % PP;
+        if (pc * (P / F::BPS) < g_n) cp_async(dst + (uint32_t)e * P, src + (size_t)row * N * F::BPS + pc * P, P);
+    }
+}
+
 template <class F>
-__device__ __forceinline__ void fw_fetch(uint8_t* raw, const uint8_t* src, int rows, int N, int g_n, bool vec) {
-    if (vec) {   // whole pieces: rows and their first byte are multiples of the piece
-        constexpr int PP = F::ROWB / F::PIECE;
-        const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(raw));
-        for (int e = threadIdx.x; e < rows * PP; e += F::T) {
-            const int row = e / PP, pc = e % PP;
-            if (pc * (F::PIECE / F::BPS) < g_n)
-                cp_async(dst + (uint32_t)e * F::PIECE, src + (size_t)row * N * F::BPS + pc * F::PIECE, F::PIECE);
-        }
-    } else {
-        for (int e = threadIdx.x; e < rows * F::G; e += F::T) {
-            const int row = e / F::G, g = e % F::G;
-            if (g >= g_n) continue;
-            const uint8_t* s = src + ((size_t)row * N + g) * F::BPS;
-            if constexpr (F::BPS == 2)
-                reinterpret_cast<unsigned short*>(raw)[e] = *reinterpret_cast<const unsigned short*>(s);
-            else raw[e] = *s;
-        }
+__device__ __forceinline__ void fw_fetch(uint8_t* raw, const uint8_t* src, int rows, int N, int g_n, int piece) {
+    if (F::PIECE >= 16 && piece == 16) return fw_fetch_pieces<F, F::PIECE >= 16 ? 16 : F::ROWB>(raw, src, rows, N, g_n);
+    if (F::PIECE >= 8 && piece == 8) return fw_fetch_pieces<F, F::PIECE >= 8 ? 8 : F::ROWB>(raw, src, rows, N, g_n);
+    if (F::PIECE >= 4 && piece == 4) return fw_fetch_pieces<F, F::PIECE >= 4 ? 4 : F::ROWB>(raw, src, rows, N, g_n);
+    // a thread's samples are rows apart: eight loads in flight
+    using S = std::conditional_t<F::BPS == 2, unsigned short, uint8_t>;
+    const int g = threadIdx.x % F::G;
+    const S* in = reinterpret_cast<const S*>(src) + g;
+    S* out = reinterpret_cast<S*>(raw) + g;
+    constexpr int STEP = F::T / F::G;
+    for (int row = threadIdx.x / F::G; row < rows; row += 8 * STEP) {
+        S x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = g < g_n && row + u * STEP < rows ? in[(size_t)(row + u * STEP) * N] : S{};
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (row + u * STEP < rows) out[(row + u * STEP) * F::G] = x[u];
     }
 }
 
@@ -371,11 +383,11 @@ __device__ __forceinline__ float2 fw_point(const uint8_t* raw, int i) {
     else return make_float2(unpack1<KIND>(raw[2 * i * F::ROWB]).x, unpack1<KIND>(raw[(2 * i + 1) * F::ROWB]).x);
 }
 
-template <int KIND, int LGL>
-__global__ void __launch_bounds__(FW<KIND, LGL, 0>::T, 1024 / FW<KIND, LGL, 0>::T)
+template <int KIND, int LGL, int ROW>
+__global__ void __launch_bounds__(FW<KIND, LGL, 0, ROW>::T, 1024 / FW<KIND, LGL, 0, ROW>::T)
     fengine_wide_kernel(const uint8_t* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tw, int N,
-                        int n_frames, int vec) {
-    using F = FW<KIND, LGL, 0>;
+                        int n_frames, int piece) {
+    using F = FW<KIND, LGL, 0, ROW>;
     extern __shared__ __align__(16) uint8_t fw_smem[];
     float2* const buf = reinterpret_cast<float2*>(fw_smem);
     float2* const tws = buf + F::DATA;
@@ -391,7 +403,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, 0>::T, 1024 / FW<KIND, LGL, 0>::
     const uint8_t* const col = raw + cf * F::L * F::ROWB + cg * F::BPS;
     int b = blockIdx.y;
     if (b < n_batches)
-        fw_fetch<F>(raw, in0 + (size_t)b * F::FB * frame_bytes, min(F::FB, n_frames - b * F::FB) * F::L, N, g_n, vec != 0);
+        fw_fetch<F>(raw, in0 + (size_t)b * F::FB * frame_bytes, min(F::FB, n_frames - b * F::FB) * F::L, N, g_n, piece);
     for (; b < n_batches; b += gridDim.y) {
         cp_async_wait();
         __syncthreads();   // this batch's samples are here, and the last one's columns are read
@@ -414,7 +426,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, 0>::T, 1024 / FW<KIND, LGL, 0>::
         const int bn = b + gridDim.y;
         if (bn < n_batches)
             fw_fetch<F>(raw, in0 + (size_t)bn * F::FB * frame_bytes, min(F::FB, n_frames - bn * F::FB) * F::L, N, g_n,
-                        vec != 0);
+                        piece);
         const int f = b * F::FB + cf;
         float2* const o = (cg < g_n && f < n_frames) ? out + (size_t)f * F::NOUT * N + n0 + cg : nullptr;
         fw_rest<F>(buf, tws, o, N);
@@ -568,7 +580,8 @@ __global__ void __launch_bounds__(FW<KIND, LGL, MT>::T, 512 / FW<KIND, LGL, MT>:
 // rows of CTAs along the frames, each with the same number of batches: the number of waves whose
 // waves x (batches of a CTA + 1) is least, the 1 being what a CTA spends before its first batch.  One
 // wave alone leaves up to half the chip idle when the groups are more than half of it.
-int fw_rows(int groups, int n_batches, int slots) {
+// *walk: the batches that a slot then takes one after another.
+int fw_rows(int groups, int n_batches, int slots, long long* walk = nullptr) {
     const int w0 = (groups + slots - 1) / slots;
     long long best_cost = 0;
     int best = 1;
@@ -579,24 +592,60 @@ int fw_rows(int groups, int n_batches, int slots) {
         if (w == w0 || cost < best_cost) {
             best_cost = cost;
             best = (int)((n_batches + per - 1) / per);
+            if (walk) *walk = w * per;
         }
     }
     return best > 65535 ? 65535 : best;
 }
 
-template <int KIND, int LGL>
+template <class F>
+constexpr int plain_per_sm() {
+    return 1024 / F::T < 227 * 1024 / (F::SMEM + 1024) ? 1024 / F::T : 227 * 1024 / (F::SMEM + 1024);
+}
+
+// bytes of the pieces a sample row can be fetched in (0: single samples)
+template <class F>
+int plain_piece(const FWideArgs& p) {
+    for (int piece = 16; piece >= 4; piece /= 2)
+        if (piece <= F::PIECE && (size_t)p.n_inputs * F::BPS % piece == 0 && reinterpret_cast<uintptr_t>(p.d_in) % piece == 0)
+            return piece;
+    return 0;
+}
+
+template <int KIND, int LGL, int ROW>
 cudaError_t launch_plain(const FWideArgs& p, cudaStream_t s) {
-    using F = FW<KIND, LGL, 0>;
-    auto kern = fengine_wide_kernel<KIND, LGL>;
+    using F = FW<KIND, LGL, 0, ROW>;
+    auto kern = fengine_wide_kernel<KIND, LGL, ROW>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F::SMEM);
     if (e != cudaSuccess) return e;
     const int groups = (p.n_inputs + F::G - 1) / F::G;
-    constexpr int kPerSm = 1024 / F::T < 227 * 1024 / (F::SMEM + 1024) ? 1024 / F::T : 227 * 1024 / (F::SMEM + 1024);
-    const int rows = fw_rows(groups, (p.n_frames + F::FB - 1) / F::FB, p.n_sm * kPerSm);
-    const int vec = F::PIECE >= 4 && (size_t)p.n_inputs * F::BPS % F::PIECE == 0 &&
-                    reinterpret_cast<uintptr_t>(p.d_in) % F::PIECE == 0;
+    const int rows = fw_rows(groups, (p.n_frames + F::FB - 1) / F::FB, p.n_sm * plain_per_sm<F>());
     return launch_kernel(kern, dim3(groups, rows), F::T, F::SMEM, s, 1, false, static_cast<const uint8_t*>(p.d_in),
-                          static_cast<float2*>(p.d_out), static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames, vec);
+                          static_cast<float2*>(p.d_out), static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames,
+                          plain_piece<F>(p));
+}
+
+// Inputs of a row of a plain transform's CTAs.  Rows of 16 leave columns empty where the inputs are few or no
+// multiple of 16 (one input of 2048 real points: 1/16 of the CTA) and give a call of few frames a few CTAs
+// of 1024 threads.  CTAs of 4096 points with rows of 4 (of one, for one or two inputs of long
+// transforms) cost 1.2 to 2.2 times as much for as many points where both are full, so the choice is by the
+// batches that a slot walks, weighted.  us, rows of 16 -> chosen: c8 512 points, 1 / 8 inputs x 4096 frames
+// 142 -> 50 / 126 -> 51; r8 2048 points, 2 inputs x 4096 frames 305 -> 61, 20 x 256 47 -> 23, 16 x 1 10.6 -> 6.4;
+// c8 1024 points, 100 x 64 31 -> 27.  128 inputs and more keep rows of 16.
+template <int KIND, int LGL>
+int plain_row(const FWideArgs& p) {
+    using W = FW<KIND, LGL, 0, 16>;
+    using N = FW<KIND, LGL, 0, 4>;
+    if (p.n_inputs <= 12 - W::LGH && W::LGH >= 10) return 1;   // up to 2 / 1 inputs of 1024 / 2048 points
+    const int gn = (p.n_inputs + N::G - 1) / N::G, bn = (p.n_frames + N::FB - 1) / N::FB;
+    if (W::LGH >= 9 && (long long)gn * bn <= p.n_sm) return 4;   // a CTA each at most
+    long long walk_w = 0, walk_n = 0;
+    fw_rows((p.n_inputs + W::G - 1) / W::G, (p.n_frames + W::FB - 1) / W::FB, p.n_sm * plain_per_sm<W>(), &walk_w);
+    fw_rows(gn, bn, p.n_sm * plain_per_sm<N>(), &walk_n);
+    // rows of one or two inputs (LGH 12, 11) write parts of sectors where there are more
+    const double cost = W::LGH <= 8 ? 1.45 : W::LGH <= 10 ? 1.2 : W::LGH == 11 ? (p.n_inputs <= 6 ? 1.0 : 1.5)
+                                                                               : (p.n_inputs <= 2 ? 0.9 : 2.2);
+    return walk_n * cost <= walk_w ? 4 : 16;
 }
 
 template <int KIND, int LGL, int MT>
@@ -622,7 +671,13 @@ cudaError_t launch_len(const FWideArgs& p, cudaStream_t s) {
         if (p.d_taps) return p.n_taps <= 4 ? launch_pfb<KIND, LGL, 4>(p, s) : launch_pfb<KIND, LGL, 8>(p, s);
     }
     if constexpr (KIND != CORR_F_REAL8 || LGL >= 8) {
-        if (!p.d_taps) return launch_plain<KIND, LGL>(p, s);
+        if (!p.d_taps) {
+            const int row = plain_row<KIND, LGL>(p);
+            constexpr int lgh = FW<KIND, LGL, 0>::LGH;
+            if constexpr (lgh == 10 || lgh == 11)
+                if (row == 1) return launch_plain<KIND, LGL, 1>(p, s);
+            return row == 4 ? launch_plain<KIND, LGL, 4>(p, s) : launch_plain<KIND, LGL, 16>(p, s);
+        }
     }
     return cudaErrorInvalidValue;
 }
@@ -658,11 +713,37 @@ cudaError_t launch_kind(const FWideArgs& p, cudaStream_t s) {
 // The few taps of a long complex transform stay with fengine.cu, which pays for each tap: c8 of 128
 // inputs, L = 512, 2 / 3 / 4 taps: 267 / 304 / 335 there, 313 here; c4, L = 256, 2 / 4 taps: 193 / 258
 // there, 205 / 200 here; L = 1024, 4 / 6 taps: 476 / 823 there, 544 / 577 here.
-bool fwide_takes(int kind, int log2L, int n_inputs, int n_taps) {
+// A CTA of the filterbank spends 3 or 7 frames of samples before its first batch of four, so calls that give
+// a slot one batch, and fengine.cu no more than one either, stay there (8 taps, 1 input x 64 frames, r8
+// L = 1024: 8.9 us there, 14.5 here; 256 inputs x 8 frames 41 there, 19 here), except the cheap ones (complex, up
+// to 128 points, up to 4 taps: 7.5 there, 6.3 here); and so do the few taps of short transforms where groups
+// are part empty or more than one (L = 32, 1 tap, 16 inputs, c8 / r8: 1.2 / 1.6 times faster there; 64 points, 1 / 2
+// taps, 40 to 256 inputs 1.2 / 1.05; r8 2048 points, 1 tap 1.1).
+bool fwide_takes(int kind, int log2L, int n_inputs, int n_taps, int n_frames, int n_sm) {
     const bool real = kind == CORR_F_REAL8;
     if (log2L < 5) return false;
-    if (n_taps > 0) return n_taps <= 8 && log2L <= (real ? 11 : 10) && (real || log2L < 8 || n_taps >= log2L - 5);
-    return real ? log2L >= 8 : log2L != 6 || n_inputs % 64 != 0;
+    if (n_taps == 0) {
+        // rows of no whole words, of 64 and 128 points: read sample by sample, better there (c4, 50 inputs, 31 / 60
+        // us there, 42 / 84 here)
+        if (!real && (log2L == 6 || log2L == 7) && n_inputs > 32 && n_inputs * (kind == CORR_F_COMPLEX8 ? 2 : 1) % 4) return false;
+        return real ? log2L >= 8 : log2L != 6 || n_inputs % 64 != 0;
+    }
+    if (n_taps > 8 || log2L > (real ? 11 : 10)) return false;
+    const int group = 2048 >> (log2L - (real ? 1 : 0));   // inputs of a CTA
+    if (real) {
+        if (log2L == 5 && n_inputs <= 64) return false;
+        if (n_taps == 1 && (log2L <= 8 || log2L == 11) && log2L != 5) return false;
+        if (n_taps == 2 && log2L <= 7 && n_inputs < 8) return false;
+    } else {
+        if (log2L >= 8 && n_taps < log2L - 5) return false;
+        if (log2L == 5 && (n_taps == 1 || (n_taps == 2 && n_inputs % 4))) return false;
+        if ((log2L == 6 || log2L == 7) && n_taps <= 2 && n_inputs > group) return false;
+        if (log2L < 8 && n_taps <= 4) return true;
+    }
+    long long walk = 0;
+    fw_rows((n_inputs + group - 1) / group, (n_frames + 3) / 4, n_sm, &walk);
+    const long long there = log2L >= 6 ? 4096 >> log2L : 64;   // fengine.cu's inputs per CTA, two CTAs per SM
+    return walk >= 2 || (n_inputs + there - 1) / there * n_frames > 2LL * n_sm;
 }
 
 std::vector<float2> fwide_tables(int kind, int log2L) {

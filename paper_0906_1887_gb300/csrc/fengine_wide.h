@@ -1,4 +1,5 @@
-// F-stage kernels for long transforms and short filterbanks (fengine_wide.cu), called by fengine.cu.
+// F-stage kernels of fengine_wide.cu, called by fengine.cu where fwide_takes says so: transforms of 32 points and
+// more, filterbanks of at most 8 taps.
 #pragma once
 
 #include <vector>
@@ -15,7 +16,7 @@ struct FWideArgs {
     const float* d_taps;   // filterbank prototype, n_taps x L values (null: plain transform)
 };
 
-bool fwide_takes(int kind, int log2L, int n_inputs, int n_taps);   // n_taps = 0: plain transform
+bool fwide_takes(int kind, int log2L, int n_inputs, int n_taps, int n_frames, int n_sm);   // n_taps = 0: plain transform
 std::vector<float2> fwide_tables(int kind, int log2L);
 cudaError_t launch_fwide(const FWideArgs& p, cudaStream_t s);
 
