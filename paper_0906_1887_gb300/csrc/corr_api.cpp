@@ -214,7 +214,7 @@ corr_status corr_xengine_run_batch(corr_plan plan, const void* d_packed, int n_d
     if (engine == CORR_ENGINE_TC) {
         if (p->sample_bits == 32)
             return set_error(CORR_EUNSUPPORTED, "float samples run on CORR_ENGINE_BF16X3 or CORR_ENGINE_FP32");
-        if (!d_workspace || !tc_use_planes(*p) || tc_raw_by_packing(*p)) {
+        if (!d_workspace || !tc_use_planes(*p) || tc_raw_by_packing(*p, n_dumps, accumulate)) {
             e = launch_xeng_tc_raw(*p, d_packed, n_dumps, d_vis, accumulate, s);
         } else {
             e = launch_tc_plane_path(*p, d_packed, n_dumps, d_workspace, d_vis, accumulate, s);
@@ -225,10 +225,10 @@ corr_status corr_xengine_run_batch(corr_plan plan, const void* d_packed, int n_d
         if (p->sample_bits != 32)
             return set_error(CORR_EUNSUPPORTED, "CORR_ENGINE_BF16X3 takes float samples (sample_bits=32)");
         // fused: TMA loads the floats, the converter warps split them
-        if (need == 0 || (tc_rawf32_pairs(*p) && aligned16(d_packed) &&
+        if (need == 0 || (tc_rawf32_pairs(*p, n_dumps, accumulate) && aligned16(d_packed) &&
                           (int64_t)n_dumps * p->n_chan < (int64_t{1} << 31))) {
             e = launch_xeng_tc_rawf32(*p, d_packed, n_dumps, d_vis, accumulate, s);
-        } else if (tc_rawf32_odd(*p, n_dumps)) {
+        } else if (tc_rawf32_odd(*p, n_dumps, accumulate)) {
             e = launch_xeng_tc_rawf32_odd(*p, d_packed, n_dumps, d_workspace, d_vis, accumulate, s);
         } else {
             char* hi = static_cast<char*>(d_workspace);

@@ -94,13 +94,16 @@ bool tc_use_planes(const Plan& p);
 bool tc_raw_supported(int n_inputs, int sample_bits);
 // Rows that TMA cannot address one channel at a time, of a small array whose channels it can address
 // packed side by side (tc_channel_pack): the packed feed takes them too, and needs no planes.
-bool tc_raw_by_packing(const Plan& p);
+bool tc_raw_by_packing(const Plan& p, int n_dumps, int accumulate);
 // The workspace's planes: e4m3 bytes for 4-bit samples of TMA-addressable rows (rows of
 // tc_kp_e4m3 = n_time rounded up to 128 bytes, read by kind::f8f6f4 MMAs), fp16 otherwise.  The
 // public planes calls (corr_unpack, corr_xengine_run_planes) keep fp16 planes.
 bool tc_planes_e4m3(const Plan& p);
 bool tc_use_pairs(const Plan& p, bool packed);   // CTA pairs (PAIR in xeng_tc.cu) rather than single CTAs
-// the packed feed although the plan has a plane workspace
+// the packed feed although the plan has a plane workspace, and the launches that read planes although it
+// could convert (few items of long dumps)
+bool int_planes_faster(const Plan& p, int n_dumps, int accumulate);
+bool float_planes_faster(const Plan& p, int n_dumps, int accumulate);
 bool tc_packed_pairs(const Plan& p, int accumulate);
 int tc_kp_e4m3(const Plan& p);
 size_t tc_workspace_planes_bytes(const Plan& p, int n_dumps);
@@ -143,10 +146,11 @@ int tc_default_cpi(int n_inputs, int64_t channels, int n_sm);   // channels = du
 // BF16x3 on float samples with the hi/lo split done in the tensor-core kernel: without a workspace
 // (single-block arrays of an even count), by pairs of CTAs, and for odd counts
 bool tc_rawf32_supported(const Plan& p);
-bool tc_rawf32_pairs(const Plan& p);   // float samples of several blocks that CTA pairs split in the kernel
+// float samples of several blocks that CTA pairs split in the kernel
+bool tc_rawf32_pairs(const Plan& p, int n_dumps, int accumulate);
 cudaError_t launch_xeng_tc_rawf32(const Plan& p, const void* d_samples, int n_dumps, void* d_vis, int accumulate,
                                   cudaStream_t s, int64_t pitch = 0);   // pitch: bytes of a padded row, 0: dense
-bool tc_rawf32_odd(const Plan& p, int n_dumps);
+bool tc_rawf32_odd(const Plan& p, int n_dumps, int accumulate);
 cudaError_t launch_xeng_tc_rawf32_odd(const Plan& p, const void* d_samples, int n_dumps, void* d_ws, void* d_vis,
                                       int accumulate, cudaStream_t s);
 // Fused dump mode: float32 [n_dumps][C][P][2] = V / n_accum * phasor_i conj(phasor_j) (phasor

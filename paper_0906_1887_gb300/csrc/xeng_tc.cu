@@ -1545,6 +1545,14 @@ cudaError_t launch_jobs(const TcJobSpec* specs, int n_jobs, const CUtensorMap* m
     return e;
 }
 
+// Pairs on planes, except for short accumulating dumps of few squares, whose read-modify-write single tiles spread
+// over more CTAs (256 inputs x 1 channel x 128 samples 16.5 -> 12.6 us, 512 x 16 x 64 24.5 -> 22.7).
+bool plane_pairs(const Plan& p, int n_dumps, int accumulate) {
+    const int ng = (p.nb + 1) / 2;
+    if (accumulate && p.kp <= 512 && (int64_t)ng * (ng + 1) / 2 * n_dumps * p.n_chan <= p.n_sm) return false;
+    return tc_use_pairs(p, false);
+}
+
 }  // namespace
 
 cudaError_t launch_xeng_tc(const Plan& p, const void* d_planes, const void* d_planes_lo, int n_dumps, void* d_vis,
@@ -1567,7 +1575,7 @@ cudaError_t launch_xeng_tc(const Plan& p, const void* d_planes, const void* d_pl
     // read-modify-write epilogue bounds them and which run faster on the deeper operand ring of
     // 32 KB stages (measured: 1024 inputs x 1228 channels x 472 samples, 4.05 against 4.41 ms)
     const bool wide = p.tc_items == 2 || (p.tc_items == 0 && !(accumulate && p.kp < 1024));
-    tune.pair = tc_use_pairs(p, false);
+    tune.pair = plane_pairs(p, n_dumps, accumulate);
     CUtensorMap mw;
     if (!tune.pair && p.nb >= 2 && wide && make_plane_map(&mw, d_planes, p.kp, rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
                                             2 * kBlockRows)) {
@@ -1598,15 +1606,45 @@ bool tc_use_pairs(const Plan& p, bool packed) {
 // Accumulating dumps gain more: the read-modify-write of the sums leaves the packed feed's port and
 // the memory system less to share than planes do.  8-bit, 400 inputs x 512 / 1024 samples 424 -> 358 /
 // 702 -> 642, 1024 x 512 / 768 / 1024 536 -> 446 / 579 -> 549 / 666 -> 695; 4-bit, 192 x 384 94 -> 77,
-// 400 x 512 320 -> 308, 1024 x 512 / 768 527 -> 488 / 505 -> 457, but 400 x 768 356 -> 417.
+// 400 x 512 320 -> 308, 1024 x 512 / 768 527 -> 488 / 505 -> 457, 256 / 384 inputs x 1024 channels x 1000
+// samples 450 -> 264 / 869 -> 572, but 400 x 768 356 -> 417.
+// Few items of long dumps go the other way (int_planes_faster).
 bool tc_packed_pairs(const Plan& p, int accumulate) {
     // one operand stage (set_tuning): the plane feed ignores it, the packed one could not run
     if (p.tc_operands != 0 || p.tc_items != 0 || p.nb < 2 || p.tc_op_stages == 1) return false;
     const bool even = p.nb % 2 == 0;
     if (accumulate)
-        return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= (p.nb <= 12 ? 1024 : 768) : p.kp <= (even ? 768 : 512);
+        return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= (p.nb <= 12 ? 1024 : 768) : p.kp <= (even ? 1024 : 512);
     if (!even || !tc_use_pairs(p, true)) return false;
     return p.sample_bits == 8 ? p.nb <= 8 || p.kp <= 256 : p.nb == 4 && p.kp <= 512;
+}
+
+// Planes are written by the whole chip and then read at the MMAs' own pace; the packed feeds convert in the few
+// CTAs that have an item, at 1.3 to 1.6 times the time per 64 samples.  Where the launch does not fill the
+// chip and the dump is long, that is what it takes, planes or no planes.  Both estimated in us, from the waves of
+// items, the time of an item's stage and the bytes that the extra kernel and the planes move; measured, packed ->
+// planes: 8-bit, 256 inputs x 1 channel x 20000 / 60000 samples 207 -> 140 / 600 -> 392, x 4 x 20000 209 -> 155; 129 x 1 x
+// 20000 201 -> 134; 9 inputs x 1 channel x 20000 143 -> 113; 320 x 16 x 20000, accumulating, 392 -> 274; but 256 x 16 x 20000
+// 300 there, 318 with planes.  Dumps of fewer than 1500 samples, and 4-bit ones, are no slower packed.
+bool int_planes_faster(const Plan& p, int n_dumps, int accumulate) {
+    const int stages = p.kp / kTimeBlock;
+    const int64_t cd = (int64_t)n_dumps * p.n_chan;
+    if (p.sample_bits != 8 || stages < 24 || cd * p.nb * kBlockRows >= (int64_t{1} << 31)) return false;
+    const int ng = (p.nb + 1) / 2;
+    const bool pairs = tc_use_pairs(p, true), ragged = !tc_raw_supported(p);
+    const int pack = tc_channel_pack(p.n_inputs, 2, p.n_chan, n_dumps, p.n_sm);
+    const int64_t tiles = p.nb * (p.nb + 1) / 2 * cd, squares = ng * (ng + 1) / 2 * cd;
+    auto waves = [](int64_t items, int64_t slots) { return (double)((items + slots - 1) / slots); };
+    const double w = pairs ? waves(squares, p.n_sm / 2) : waves(p.nb == 1 && pack > 1 ? tiles / pack : tiles, p.n_sm);
+    if (w > (p.nb == 1 ? 1 : 2)) return false;   // full chips hide the conversion
+    const double mb = 2e-6 * p.n_inputs * (double)p.n_time * cd;
+    double packed = w * stages * (!pairs ? 0.44 : p.nb == 2 ? 0.48 : 0.66);
+    if (ragged && pack < 2) packed += 5 + 0.31 * mb;   // the repacked copy
+    const double w_pl = tc_use_pairs(p, false)                                            ? waves(squares, p.n_sm / 2)
+                        : p.nb >= 2 && !(accumulate && p.kp < 1024) ? waves(wide_items(p.nb) * cd, p.n_sm)
+                                                                    : waves(tiles, p.n_sm);
+    const double planes = 5 + w_pl * stages * (p.nb == 1 ? 0.35 : 0.41) + 0.14 * (mb + 512e-6 * p.nb * (double)p.kp * cd);
+    return planes < packed;
 }
 
 bool tc_planes_e4m3(const Plan& p) { return p.sample_bits == 4 && tc_raw_supported(p); }
@@ -1625,7 +1663,7 @@ cudaError_t launch_xeng_tc_e4m3_planes(const Plan& p, const void* d_planes, int 
     if (!make_plane_map(&mh, d_planes, kp8, rows, CU_TENSOR_MAP_DATA_TYPE_UINT8)) return cudaErrorInvalidValue;
     // item shape as for fp16 planes
     const bool wide = p.tc_items == 2 || (p.tc_items == 0 && !(accumulate && kp8 < 1024));
-    tune.pair = tc_use_pairs(p, false);
+    tune.pair = plane_pairs(p, n_dumps, accumulate);
     if (!tune.pair && p.nb >= 2 && wide &&
         make_plane_map(&mw, d_planes, kp8, rows, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2 * kBlockRows)) {
         sp.tw = 2;
@@ -1650,10 +1688,11 @@ bool tc_raw_supported(int n_inputs, int sample_bits) {
 
 bool tc_raw_supported(const Plan& p) { return tc_raw_supported(p.n_inputs, p.sample_bits); }
 
-bool tc_raw_by_packing(const Plan& p) {
+bool tc_raw_by_packing(const Plan& p, int n_dumps, int accumulate) {
     return (p.sample_bits == 4 || p.sample_bits == 8) && !tc_raw_supported(p) && p.tc_operands == 0 &&
            p.tc_op_stages != 1 &&   // as in tc_packed_pairs
-           tc_channel_pack(p.n_inputs, p.sample_bits == 8 ? 2 : 1, p.n_chan, 1, p.n_sm) > 1;
+           tc_channel_pack(p.n_inputs, p.sample_bits == 8 ? 2 : 1, p.n_chan, 1, p.n_sm) > 1 &&
+           !int_planes_faster(p, n_dumps, accumulate);
 }
 
 // Channel pairs (256-byte TMA rows, one item's epilogue under the next item's MMAs) for
@@ -1811,6 +1850,38 @@ bool tc_rawf32_supported(const Plan& p) {
     return p.sample_bits == 32 && p.n_inputs <= kBlockInputs && (p.n_inputs % 2) == 0;
 }
 
+// As int_planes_faster, for float samples that the kernel could split itself.  Measured, in the kernel -> planes:
+// 128 inputs x 1 channel x 4000 / 20000 samples 57 -> 41 / 254 -> 171 us, 256 x 1 / 4 x 20000 347 -> 175 / 441 -> 232, 512 x 8 x
+// 4000 161 -> 130, 65 x 1 x 1000 23 -> 19, 33 x 2 x 20000 202 -> 169; but 128 x 16 x 20000 257 in the kernel, 297 with planes, and
+// from five waves on (nine of long dumps) always the kernel.  Accumulating dumps also pay for the tiles' read-modify-write,
+// in pairs by few CTAs: short ones of two blocks (65 inputs x 256 channels x 64 samples 62 -> 45) are better spread.
+bool float_planes_faster(const Plan& p, int n_dumps, int accumulate) {
+    const int stages = p.kp / kTimeBlock, ng = (p.nb + 1) / 2;
+    const int64_t cd = (int64_t)n_dumps * p.n_chan;
+    if (cd * p.nb * kBlockRows >= (int64_t{1} << 31)) return false;
+    const int pack = accumulate ? 1 : tc_channel_pack(p.n_inputs, 8, p.n_chan, n_dumps, p.n_sm);
+    const bool repack = p.n_inputs % 2 && pack < 2;
+    const int64_t tiles = p.nb * (p.nb + 1) / 2 * cd, squares = ng * (ng + 1) / 2 * cd;
+    auto waves = [](int64_t items, int64_t slots) { return (double)((items + slots - 1) / slots); };
+    const double mb = 8e-6 * p.n_inputs * (double)p.n_time * cd;
+    double split;
+    if (p.nb == 1) {
+        const double w = waves((cd + (pack > 1 ? pack : 1) - 1) / (pack > 1 ? pack : 1), p.n_sm);
+        if (w > 1) return false;
+        split = w * stages * 0.66;
+    } else {
+        const double w = waves(squares, p.n_sm / 2);
+        if (accumulate && p.nb == 2 && w > 1 && stages <= (repack ? 4 : 2)) return true;
+        if (w > (stages >= 32 ? 8 : 4)) return false;
+        const double item = accumulate ? (p.nb == 2 ? 13 : p.nb % 2 ? 6.5 : 9) : 1.5;
+        split = w * (stages * (p.nb == 2 ? 0.82 : w == 1 || p.nb > 4 ? 1.45 : 1.15) + item);
+    }
+    if (repack) split += 4.5 + 0.31 * mb;
+    const double planes = 5 + waves(tiles, p.n_sm) * (stages * 0.5 + (accumulate && p.nb > 1 ? 6.2 : 0.8)) +
+                          0.14 * (mb + 1024e-6 * p.nb * (double)p.kp * cd);
+    return split > 1.03 * planes;
+}
+
 // Arrays of several blocks: the CTAs of a pair split the blocks of a square themselves, where the plane
 // feed writes hi and lo planes (half of its time) and reads them back.  Measured, planes -> pairs: 128
 // inputs x 512 channels x 64 / 128 / 256 / 512 samples 50 -> 27 / 69 -> 31 / 99 -> 38 / 173 -> 63 us (45
@@ -1819,10 +1890,11 @@ bool tc_rawf32_supported(const Plan& p) {
 // 433 -> 238, 192 x 202 x 506 116 -> 78, 130 x 139 x 1222 180 -> 136, 512 x 128 x 512 283 -> 178, 1024 x 64
 // x 256 / 1024 281 -> 180 / 780 -> 602.  Odd block counts above one compute half-empty squares and gain
 // nothing on long dumps (320 x 200 x 500 220 -> 167, but 320 x 30 x 2000 126 -> 127).
-bool tc_rawf32_pairs(const Plan& p) {
+bool tc_rawf32_pairs(const Plan& p, int n_dumps, int accumulate) {
     return p.sample_bits == 32 && p.nb >= 2 && (p.nb % 2 == 0 || p.kp <= 1536) && (p.n_inputs % 2) == 0 &&
            !p.tc_float_planes &&
-           p.tc_op_stages != 1;   // one operand stage: the plane feed ignores it, this one could not run
+           p.tc_op_stages != 1 &&   // one operand stage: the plane feed ignores it, this one could not run
+           !float_planes_faster(p, n_dumps, accumulate);
 }
 
 // Odd counts of inputs, whose rows TMA cannot address: several channels of at most 32 inputs packed into
@@ -1832,9 +1904,9 @@ bool tc_rawf32_pairs(const Plan& p) {
 // 1222 113 -> 73, 127 x 512 x 512 181 -> 145, x 20 x 100 15 -> 13, 255 x 202 x 506 177 -> 149, 1023 x 64 x
 // 256 289 -> 227; odd block counts, whose squares are half empty, stay with the planes (141 x 179 x 833 172
 // there, 182 here).
-bool tc_rawf32_odd(const Plan& p, int n_dumps) {
+bool tc_rawf32_odd(const Plan& p, int n_dumps, int accumulate) {
     return p.sample_bits == 32 && p.n_inputs % 2 && (p.nb == 1 || p.nb % 2 == 0) && !p.tc_float_planes && p.tc_op_stages != 1 &&
-           (int64_t)n_dumps * p.n_time * p.n_chan < (int64_t{1} << 31);
+           (int64_t)n_dumps * p.n_time * p.n_chan < (int64_t{1} << 31) && !float_planes_faster(p, n_dumps, accumulate);
 }
 
 cudaError_t launch_xeng_tc_rawf32_odd(const Plan& p, const void* d_samples, int n_dumps, void* d_ws, void* d_vis,
@@ -1894,8 +1966,10 @@ cudaError_t launch_xeng_tc_raw(const Plan& p, const void* d_packed, int n_dumps,
 cudaError_t launch_tc_plane_path(const Plan& p, const void* d_packed, int n_dumps, void* d_ws, void* d_vis,
                                  int accumulate, cudaStream_t s) {
     const bool ragged = !tc_raw_supported(p), aligned = (reinterpret_cast<uintptr_t>(d_packed) & 15u) == 0;
-    const bool packed = tc_packed_pairs(p, accumulate) || (ragged && p.tc_operands == 0 && p.tc_op_stages != 1 &&
-                                               p.nb < (p.sample_bits == 4 ? kPlaneMinBlocksE4m3 : kPlaneMinBlocks));
+    const bool packed = (tc_packed_pairs(p, accumulate) ||
+                         (ragged && p.tc_operands == 0 && p.tc_op_stages != 1 &&
+                          p.nb < (p.sample_bits == 4 ? kPlaneMinBlocksE4m3 : kPlaneMinBlocks))) &&
+                        !int_planes_faster(p, n_dumps, accumulate);
     if (packed && aligned) {
         if (!ragged) return launch_xeng_tc_raw(p, d_packed, n_dumps, d_vis, accumulate, s);
         if ((int64_t)n_dumps * p.n_time * p.n_chan < (int64_t{1} << 31)) {
