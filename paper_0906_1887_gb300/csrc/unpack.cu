@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
     constexpr int kPieces = F::kRowBytes / 16;          // 16-byte pieces per packed row
     constexpr int kPer = kTimeBlock * kPieces / F::kThreads;   // pieces a thread moves per tile (2)
     static_assert(kPer * F::kThreads == kTimeBlock * kPieces, "whole pieces per thread");
+    const uint32_t tail = RAGGED ? tail_word(packed, n_bytes) : 0u;
     // conversion task of this thread
     const int q = tid & 7, pw = tid >> 3;             // sample group, word within the row
     const uint32_t* src = tile + (size_t)(8 * q) * F::kWords;
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(FastTile<BITS>::kThreads) unpack_fast_kernel(
                         ((d * n_time + tg) * n_chan + c) * row_bytes + (int64_t)nb * F::kRowBytes + piece * 16;
                     if constexpr (RAGGED) {
                         uint32_t x[4];
-                        load_piece(packed, off, n_bytes, (int)(valid - piece * 16 < 16 ? valid - piece * 16 : 16), x);
+                        load_piece(packed, off, n_bytes, (int)(valid - piece * 16 < 16 ? valid - piece * 16 : 16), tail, x);
                         v[gi][u] = make_uint4(x[0], x[1], x[2], x[3]);
                     } else {
                         v[gi][u] = *reinterpret_cast<const uint4*>(packed + off);
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __rest
                                                      unsigned char* __restrict__ out, uint32_t rows, int row_bytes,
                                                      int pieces, uint32_t rows_per_block, int64_t n_bytes) {
     grid_release();
+    const uint32_t tail = FLOAT ? 0u : tail_word(packed, n_bytes);
     for (uint32_t r0 = blockIdx.x * rows_per_block; r0 < rows; r0 += gridDim.x * rows_per_block) {
         const uint32_t n = min(rows_per_block, rows - r0) * (uint32_t)pieces;
         uint4* dst = reinterpret_cast<uint4*>(out) + (int64_t)r0 * pieces;
@@ -291,7 +293,7 @@ __global__ void __launch_bounds__(256) repack_kernel(const unsigned char* __rest
                 dst[e] = make_uint4(a.x, a.y, b.x, b.y);
             } else {
                 uint32_t x[4];
-                load_piece(packed, off, n_bytes, 16, x);
+                load_piece(packed, off, n_bytes, 16, tail, x);
                 dst[e] = make_uint4(x[0], x[1], x[2], x[3]);
             }
         }

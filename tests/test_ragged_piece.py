@@ -23,7 +23,7 @@ int main() {
                     for (int whole = 0; whole < 2; ++whole) {
                         const int off = r * row_bytes + 16 * c, left = row_bytes - 16 * c < 16 ? row_bytes - 16 * c : 16;
                         uint32_t v[4];
-                        corr::load_piece(p, off, n, whole ? 16 : left, v);   // as the repack / the unpack asks for it
+                        corr::load_piece(p, off, n, whole ? 16 : left, corr::tail_word(p, n), v);   // as the repack / the unpack asks for it
                         for (int b = 0; b < 16; ++b) {
                             const unsigned got = (v[b >> 2] >> (8 * (b & 3))) & 255u;
                             if (b < left ? got != p[off + b] : (!whole && got)) return 1;
