@@ -33,8 +33,10 @@
 //              64-input x 64-sample block (128 samples for 4-bit e4m3 operands) and eight
 //              converter warps turn them into the swizzled operand tiles in shared memory: the
 //              unpack/transpose step (Sec. 4) fused into the X kernel, so the samples cross
-//              HBM once.  Float samples of single-block arrays go the same way (8-byte
-//              complex floats in, bf16 hi and lo tiles out) instead of through planes.
+//              HBM once.  Float samples go the same way (8-byte complex floats in, bf16 hi and lo
+//              tiles out) where that is faster than planes (tc_rawf32_pairs, tc_rawf32_odd).
+//
+// Arrays of several blocks mostly run in pairs of CTAs on 2 x 2 squares of tiles (PAIR below).
 //
 // CTA roles (one CTA per SM, persistent over work items = (dump, channel, I, J)):
 //   warp 0       TMA producer
@@ -110,7 +112,8 @@ struct Cfg {
     static constexpr int kConvWarps = 8;
     // groups of converter warps, each taking every other stage: the e4m3 and float conversions gain (4-bit
     // 64 inputs 126 -> 116 us, 128 inputs x 2048 samples 106 -> 86; BF16x3 109 -> 105), the 8-bit one,
-    // whose loads and stores crowd the shared-memory port, does not (129 -> 136)
+    // whose loads and stores crowd the shared-memory port, does not on single blocks (129 -> 136; not
+    // measured in pairs)
     static constexpr int kConvGroups = kF8 || kFloat ? 2 : 1;
     static constexpr int kGroupWarps = kConvWarps / kConvGroups;
     static constexpr int kThreads = 64 + 32 * kEpiWarps + (kRaw ? 32 * kConvWarps : 0);
@@ -1174,6 +1177,12 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         }
         // every bulk copy of ours must have completed before the CTA exits
         if (lane < 16) bulk_wait_all();
+        // The issuing CTA's commits arrive in its peer as well, and the last must have before the peer exits.  The
+        // limit runs from here, where the last accumulator has been seen, not from the start of a launch that may take
+        // longer; it covers an issuer that gives up one wait later.  (Behind the closing barrier, outside
+        // the roles, the same wait cost every pass of them: 224 inputs x 1218 channels x 77 samples x 4 640 -> 652 us.)
+        if (PAIR && rank != 0 && warp == 2 && lane == 0)
+            ptx::mbar_wait_drain(bar_drain, 0, prm.wait_limit_ns + kDrainLimitNs);
     } else if constexpr (C::kRaw) {
         // ---------------- converters (the last kConvWarps warps) ----------------
         // With two groups, one converts a whole stage while the other converts the next one: waits,
@@ -1313,10 +1322,6 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel(const _
         ptx::cluster_sync();   // neither CTA's memory goes while the other may still arrive there or read it
         // The issuing CTA has seen its last commit; the same commits must have arrived here before
         // this CTA exits.  The limit runs from here, not from the start of a launch that may take longer.
-        if (rank != 0 && warp == 1) {
-            if (lane == 0) ptx::mbar_wait_drain(bar_drain, 0, kDrainLimitNs);
-            __syncwarp();
-        }
     } else {
         __syncthreads();
     }

@@ -9,16 +9,20 @@ import pytest
 SRC = pathlib.Path(__file__).resolve().parents[1] / "paper_0906_1887_gb300" / "csrc" / "xeng_tc.cu"
 
 
-def test_odd_cta_waits_for_the_last_commits_after_both_ctas_are_done():
+def test_odd_cta_waits_for_the_last_commits_at_the_end_of_its_work():
     src = SRC.read_text()
     kernel = src[src.index("__global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1) xeng_tc_kernel"):]
     kernel = kernel[:kernel.index("// ---- host side")]
-    roles, tail = kernel[:kernel.rindex("ptx::tc_fence_before();")], kernel[kernel.rindex("ptx::tc_fence_before();"):]
     wait = "ptx::mbar_wait_drain(bar_drain"
-    assert roles.count(wait) == 1 and roles.index("commit(bar_drain)") < roles.index(wait)   # the issuer's own
-    assert tail.count(wait) == 1
-    order = [tail.index("ptx::cluster_sync()"), tail.index(wait), tail.index("tmem_dealloc"), tail.rindex("ptx::cluster_sync()")]
-    assert order == sorted(order) and order[0] != order[-1]
+    mma, epilogue = kernel.index("// ---------------- MMA issuer"), kernel.index("// ---------------- epilogue")
+    conv, end = kernel.index("// ---------------- converters"), kernel.rindex("ptx::cluster_sync()")
+    at = [i for i in range(len(kernel)) if kernel.startswith(wait, i)]
+    assert len(at) == 2                                     # the issuer's own, and its peer's
+    assert mma < kernel.index("commit(bar_drain)") < at[0] < epilogue
+    assert epilogue < kernel.index("mbar_arrive_cluster(ptx::map_shared(bar_acc_empty") < at[1] < conv < end
+    assert "rank != 0" in kernel[at[1] - 100:at[1]] and "wait_limit_ns" in kernel[at[1]:at[1] + 80]
+    # an issuer with nothing to commit says so
+    assert mma < kernel.index("mbar_arrive_cluster(ptx::map_shared(bar_drain, 1))") < epilogue
 
 
 @pytest.mark.gpu
