@@ -342,7 +342,9 @@ __device__ __forceinline__ void cp_async(uint32_t dst, const void* src, int byte
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // packed samples of `rows` sample rows of the CTA's inputs -> shared memory [row][G], in pieces of P bytes
-// where rows and their first byte are multiples of that (plain_piece), else sample by sample
+// where rows and their first byte are multiples of that (plain_piece), else sample by sample.  ODD: shorter
+// pieces than F::PIECE, or none, in a kernel of their own: beside the whole ones they cost those 3% (c8 1024 points,
+// 176 inputs x 1087 frames 506 -> 520 us)
 template <class F, int P>
 __device__ __forceinline__ void fw_fetch_pieces(uint8_t* raw, const uint8_t* src, int rows, int N, int g_n) {
     constexpr int PP = F::ROWB / P;
@@ -353,11 +355,11 @@ __device__ __forceinline__ void fw_fetch_pieces(uint8_t* raw, const uint8_t* src
     }
 }
 
-template <class F>
+template <class F, bool ODD>
 __device__ __forceinline__ void fw_fetch(uint8_t* raw, const uint8_t* src, int rows, int N, int g_n, int piece) {
-    if (F::PIECE >= 16 && piece == 16) return fw_fetch_pieces<F, F::PIECE >= 16 ? 16 : F::ROWB>(raw, src, rows, N, g_n);
-    if (F::PIECE >= 8 && piece == 8) return fw_fetch_pieces<F, F::PIECE >= 8 ? 8 : F::ROWB>(raw, src, rows, N, g_n);
-    if (F::PIECE >= 4 && piece == 4) return fw_fetch_pieces<F, F::PIECE >= 4 ? 4 : F::ROWB>(raw, src, rows, N, g_n);
+    if constexpr (!ODD) return fw_fetch_pieces<F, F::PIECE>(raw, src, rows, N, g_n);
+    if (F::PIECE > 8 && piece == 8) return fw_fetch_pieces<F, F::PIECE >= 8 ? 8 : F::ROWB>(raw, src, rows, N, g_n);
+    if (F::PIECE > 4 && piece == 4) return fw_fetch_pieces<F, F::PIECE >= 4 ? 4 : F::ROWB>(raw, src, rows, N, g_n);
     // a thread's samples are rows apart: eight loads in flight
     using S = std::conditional_t<F::BPS == 2, unsigned short, uint8_t>;
     const int g = threadIdx.x % F::G;
@@ -383,7 +385,7 @@ __device__ __forceinline__ float2 fw_point(const uint8_t* raw, int i) {
     else return make_float2(unpack1<KIND>(raw[2 * i * F::ROWB]).x, unpack1<KIND>(raw[(2 * i + 1) * F::ROWB]).x);
 }
 
-template <int KIND, int LGL, int ROW>
+template <int KIND, int LGL, int ROW, bool ODD>
 __global__ void __launch_bounds__(FW<KIND, LGL, 0, ROW>::T, 1024 / FW<KIND, LGL, 0, ROW>::T)
     fengine_wide_kernel(const uint8_t* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tw, int N,
                         int n_frames, int piece) {
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, 0, ROW>::T, 1024 / FW<KIND, LGL,
     const uint8_t* const col = raw + cf * F::L * F::ROWB + cg * F::BPS;
     int b = blockIdx.y;
     if (b < n_batches)
-        fw_fetch<F>(raw, in0 + (size_t)b * F::FB * frame_bytes, min(F::FB, n_frames - b * F::FB) * F::L, N, g_n, piece);
+        fw_fetch<F, ODD>(raw, in0 + (size_t)b * F::FB * frame_bytes, min(F::FB, n_frames - b * F::FB) * F::L, N, g_n, piece);
     for (; b < n_batches; b += gridDim.y) {
         cp_async_wait();
         __syncthreads();   // this batch's samples are here, and the last one's columns are read
@@ -425,7 +427,7 @@ __global__ void __launch_bounds__(FW<KIND, LGL, 0, ROW>::T, 1024 / FW<KIND, LGL,
         // the samples are consumed: the next batch's arrive while the stages run
         const int bn = b + gridDim.y;
         if (bn < n_batches)
-            fw_fetch<F>(raw, in0 + (size_t)bn * F::FB * frame_bytes, min(F::FB, n_frames - bn * F::FB) * F::L, N, g_n,
+            fw_fetch<F, ODD>(raw, in0 + (size_t)bn * F::FB * frame_bytes, min(F::FB, n_frames - bn * F::FB) * F::L, N, g_n,
                         piece);
         const int f = b * F::FB + cf;
         float2* const o = (cg < g_n && f < n_frames) ? out + (size_t)f * F::NOUT * N + n0 + cg : nullptr;
@@ -615,14 +617,17 @@ int plain_piece(const FWideArgs& p) {
 template <int KIND, int LGL, int ROW>
 cudaError_t launch_plain(const FWideArgs& p, cudaStream_t s) {
     using F = FW<KIND, LGL, 0, ROW>;
-    auto kern = fengine_wide_kernel<KIND, LGL, ROW>;
+    const int piece = plain_piece<F>(p);
+    auto kern = fengine_wide_kernel<KIND, LGL, ROW, true>;
+    if constexpr (F::PIECE >= 4)
+        if (piece == F::PIECE) kern = fengine_wide_kernel<KIND, LGL, ROW, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F::SMEM);
     if (e != cudaSuccess) return e;
     const int groups = (p.n_inputs + F::G - 1) / F::G;
     const int rows = fw_rows(groups, (p.n_frames + F::FB - 1) / F::FB, p.n_sm * plain_per_sm<F>());
     return launch_kernel(kern, dim3(groups, rows), F::T, F::SMEM, s, 1, false, static_cast<const uint8_t*>(p.d_in),
                           static_cast<float2*>(p.d_out), static_cast<const float2*>(p.d_tw), p.n_inputs, p.n_frames,
-                          plain_piece<F>(p));
+                          piece);
 }
 
 // Inputs of a row of a plain transform's CTAs.  Rows of 16 leave columns empty where the inputs are few or no
