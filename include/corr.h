@@ -118,8 +118,8 @@ corr_status corr_plan_info(corr_plan plan, int64_t *n_baselines, size_t *packed_
  * sample ring is reduced to what fits; the plane feed uses the requested depth when it is
  * smaller than what fits (by default as deep as fits).  float_planes (CORR_ENGINE_BF16X3 on float samples): 0 = the
  * default, the tensor-core kernel loads the floats and splits them into bf16 hi + lo itself
- * where it can (an even count of inputs, at most 64, needs no workspace; larger arrays leave theirs
- * unused, odd counts copy their rows into it); 1 = always split into hi/lo planes in the workspace first.  Results are
+ * where it can and that is faster (an even count of inputs, at most 64, needs no workspace; larger arrays
+ * leave theirs unused, odd counts copy their rows into it; few items of long dumps use planes); 1 = always split into hi/lo planes in the workspace first.  Results are
  * identical for every setting.
  * CORR_EINVAL when op_stages is outside [0, 16] or float_planes outside [0, 1].
  */
@@ -136,7 +136,8 @@ corr_status corr_plan_set_tuning(corr_plan plan, int op_stages, int float_planes
  *   CORR_OPERANDS_AUTO    arrays of at least 256 inputs (4 blocks; 192 inputs, 3 blocks, for
  *                         4-bit samples) when a workspace is given, and rows that are not 16-byte
  *                         multiples: planes, or the fused conversion where pairs of CTAs convert
- *                         faster than planes are read (shorter and accumulating dumps) and, for
+ *                         faster than planes are read (shorter and accumulating dumps, unless few
+ *                         channels of a long dump would leave most of the chip idle) and, for
  *                         smaller arrays of unaligned rows, where the rows are copied to 16-byte
  *                         multiples in the workspace; otherwise the fused conversion, into e4m3
  *                         operands for 4-bit samples;
@@ -153,7 +154,7 @@ corr_status corr_plan_set_tuning(corr_plan plan, int op_stages, int float_planes
  * M = 128, N = 256 MMA (a quarter fewer operand loads per tile); CORR_ITEMS_TILES = one 64 x 64
  * input tile per item; CORR_ITEMS_AUTO = pairs of CTAs on 2 x 2 squares of tiles for most arrays
  * (both feeds), else wide items, except single tiles for accumulating dumps of fewer than 1024
- * samples (bound by their read-modify-write of the output).  CORR_EINVAL on unknown values.
+ * samples, and short accumulating ones of few squares (bound by their read-modify-write of the output).  CORR_EINVAL on unknown values.
  */
 enum { CORR_OPERANDS_AUTO = 0, CORR_OPERANDS_PACKED = 1, CORR_OPERANDS_PLANES = 2, CORR_OPERANDS_PACKED_F8 = 3 };
 enum { CORR_ITEMS_AUTO = 0, CORR_ITEMS_TILES = 1, CORR_ITEMS_WIDE = 2 };

@@ -519,17 +519,18 @@ cudaError_t launch_fengine_l(const FPlan& p, const void* d_in, int n_frames, voi
     return cudaGetLastError();
 }
 
-// fengine_wide.cu takes the longer plain transforms (fwide_takes)
+// fengine_wide.cu takes the other lengths of plain transforms, and most filterbanks (fwide_takes)
 template <int KIND, bool PFB>
 cudaError_t launch_fengine(const FPlan& p, const void* d_in, int n_frames, void* d_out, cudaStream_t s) {
     switch (p.log2L) {
         case 3: return launch_fengine_l<KIND, PFB, 3>(p, d_in, n_frames, d_out, s);
         case 4: return launch_fengine_l<KIND, PFB, 4>(p, d_in, n_frames, d_out, s);
-        case 5: return launch_fengine_l<KIND, PFB, 5>(p, d_in, n_frames, d_out, s);
         case 6: return launch_fengine_l<KIND, PFB, 6>(p, d_in, n_frames, d_out, s);
         case 7: return launch_fengine_l<KIND, PFB, 7>(p, d_in, n_frames, d_out, s);
         default: break;
     }
+    if constexpr (PFB || KIND == CORR_F_REAL8)
+        if (p.log2L == 5) return launch_fengine_l<KIND, PFB, 5>(p, d_in, n_frames, d_out, s);
     if constexpr (PFB) {
         switch (p.log2L) {
             case 8: return launch_fengine_l<KIND, PFB, 8>(p, d_in, n_frames, d_out, s);

@@ -128,10 +128,12 @@ __device__ __forceinline__ uint32_t map_shared(uint32_t addr, uint32_t rank) {
     return r;
 }
 
-// Arrive on a barrier of either CTA of the cluster (an address of map_shared).  The CTA scope is
-// enough: what the arrival announces is shared or tensor memory that this CTA's own warps have
-// finished with (and fenced towards the async proxy where the tensor core reads it), not memory the
-// waiting thread reads.  With .release.cluster every arrival took 1000 clocks more.
+// Arrive on a barrier of either CTA of the cluster (an address of map_shared), with the default release at
+// CTA scope.  What it announces is shared or tensor memory that this CTA's own warps have finished with (and
+// fenced towards the async proxy), which the waiting thread does not read itself, but the pair's tensor core
+// does; the PTX memory model orders that only at cluster scope.  This leans on what is observed, not on the
+// model: published kernels for CTA pairs arrive in the same form, and every integer result here is bit-exact.
+// With .release.cluster every arrival took 1000 clocks more.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
