@@ -23,7 +23,10 @@ CORR_HOST_DEVICE uint32_t tail_word(const unsigned char* base, int64_t n_bytes) 
 
 // Bytes off .. off + 15 of the n_bytes at `base` (4-byte aligned) as four little-endian words, from the
 // aligned words around them; bytes from off + n_valid on are zero.  Nothing past base + n_bytes is
-// read: the last word of a buffer that is no multiple of 4 bytes is `tail` (tail_word), those after it are zero.
+// read: the last word of a buffer that is no multiple of 4 bytes is `tail` (tail_word), and so is what stands for
+// the words after it, of which no byte is wanted: off + n_valid <= n_bytes, or the caller reads the bytes that
+// are there only (a zero for them is one more select per word: 57 inputs x 282 channels x 158 samples,
+// 4-bit, 12.4 -> 13.4 us).
 CORR_HOST_DEVICE void load_piece(const unsigned char* base, int64_t off, int64_t n_bytes, int n_valid, uint32_t tail,
                                  uint32_t (&v)[4]) {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(base);
@@ -31,7 +34,7 @@ CORR_HOST_DEVICE void load_piece(const unsigned char* base, int64_t off, int64_t
     const uint32_t sh = (uint32_t)(off & 3) * 8;
     const int avail = (int)(whole - i < 5 ? whole - i : 5);   // whole words from the first on
     uint32_t x[5];
-    for (int k = 0; k < 5; ++k) x[k] = k < avail ? w[i + k] : k == avail ? tail : 0u;
+    for (int k = 0; k < 5; ++k) x[k] = k < avail ? w[i + k] : tail;
     for (int k = 0; k < 4; ++k) {
         const int left = n_valid - 4 * k;   // bytes of this word that are wanted
         v[k] = (uint32_t)((((uint64_t)x[k + 1] << 32) | x[k]) >> sh);
